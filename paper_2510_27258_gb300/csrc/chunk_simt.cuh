@@ -442,6 +442,69 @@ cudaError_t launch_sums(const SumJobs<T> &jobs, int njobs, int BH, int n, cudaSt
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// outputs from what the chunk itself gives and the carry [M | u] before it: num = num_loc + Q M_p,
+// den = den_loc + Q u_p
+// ---------------------------------------------------------------------------
+struct OutParams {
+    Records carry;
+    const float *num, *den;  // [BH][n][dv], [BH][n]
+    int n, d, dv, normalized;
+    float eps;
+    int has_in;  // the first chunk has a carry
+};
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT)
+    chunk_out_kernel(const T *__restrict__ q, T *__restrict__ out, const __grid_constant__ OutParams P) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *stage = b0 + tile_floats<N>(), *dens = stage + stage_floats<N>();
+    const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
+    const long long tok = (long long)hd * P.n + t0;
+    const bool carry = c > 0 || P.has_in;
+    const float *Mp = P.carry.at(hd, c);
+    const Tile<N> t;
+    Acc<N> acc;
+    acc.zero();
+    float den = 0.f;
+    if (carry) {
+        load_tile<N>(b0, q + tok * d, len, d);
+        __syncthreads();
+        if (P.normalized) den = row_dot(b0, N + 4, Mp + d * dv, d);
+        nn_carry<N, kPlain>(acc, t, b0, Mp, dv, d, dv, stage);
+    }
+    if (P.normalized) {
+        const int r = threadIdx.x >> 1;
+        if ((threadIdx.x & 1) == 0) dens[r] = (r < len ? P.den[tok + r] : 0.f) + den + P.eps;
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < Tile<N>::RM; ++i) {
+        const int r = t.row(i);
+        if (r >= len) continue;
+#pragma unroll
+        for (int j = 0; j < Tile<N>::CM; j += 4) {
+            if (t.col(j) >= dv) continue;
+            const float4 x = *reinterpret_cast<const float4 *>(P.num + (tok + r) * dv + t.col(j));
+            float y[4] = {acc.a[i][j] + x.x, acc.a[i][j + 1] + x.y, acc.a[i][j + 2] + x.z, acc.a[i][j + 3] + x.w};
+            if (P.normalized) {
+                const float den_r = dens[r];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) y[u] /= den_r;
+            }
+            Vec<T>::store4(out + (tok + r) * dv + t.col(j), y);
+        }
+    }
+}
+
+template <int N, typename T>
+cudaError_t launch_out(const T *q, T *out, const OutParams &P, int BH, cudaStream_t s) {
+    const int smem = (tile_floats<N>() + stage_floats<N>() + kC) * (int)sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(chunk_out_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e) return e;
+    chunk_out_kernel<N, T><<<dim3((P.n + kC - 1) / kC, BH), kCT, smem, s>>>(q, out, P);
+    return cudaGetLastError();
+}
+
 // the padded head size that serves d and dv
 template <typename F>
 cudaError_t with_padded_size(int d, int dv, F f) {

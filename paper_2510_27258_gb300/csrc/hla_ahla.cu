@@ -1,232 +1,164 @@
-// Asymmetric second-order HLA (AHLA): chunk-parallel forward and decode step,
-// fp32 SIMT kernels (Sec. "Asymmetric Higher-order Linear Attention").
+// Asymmetric second-order HLA (AHLA): chunk-parallel forward and decode step on
+// the CUDA cores in fp32 (Sec. "Asymmetric Higher-order Linear Attention").
 //
 // AHLA is causal linear attention applied twice: with A = L . (Q K^T) (L lower
 // triangular incl. the diagonal), r_t = q_t^T P_t = (A V)_t and
 // o_t = q_t^T E_t = (A R)_t (Theorem AHLA: P_t = sum_{j<=t} k_j v_j^T,
-// E_t = sum_{i<=t} k_i r_i^T; denominators with v -> 1).  Per chunk, rows are
-// its tokens and "p" the carry-in prefix:
+// E_t = sum_{i<=t} k_i r_i^T; denominators with v -> 1).  Per 64-token chunk, rows
+// are its tokens and "p" the prefix before it:
 //   R = A V + Q P_p,   s = A 1 + Q m_p,   O = A R + Q E_p,   den = A s + Q n_p.
-// Chunk summaries compose with Eq. AHLA-semidirect,
-//   E_AB = E_A + E_B + R^KQ_B P_A,  n_AB = n_A + n_B + R^KQ_B m_A,
-// with R^KQ = sum_i k_i q_i^T over the later chunk, so a chunk's local
-// summary (zero carry) is R^KQ = K^T Q, P = K^T V, m = K^T 1, E = K^T (A V),
-// n = K^T (A 1).  Three launches: chunk-local summaries (all chunks in
-// parallel), the carry scan (sequential over chunks, parallel over column
-// blocks of [P | m] and [E | n]), outputs (all chunks in parallel).  The
-// chunk argument is the scan granularity; chunks are at most 64 tokens here,
-// 32 with a 128-wide head (the result does not depend on it up to rounding).
-// Token rows of K are staged with a stride of d + 1 floats, so that the lanes
-// of a warp, which take consecutive keys, read distinct banks.
+// Every carry is a plain prefix sum: P += K^T V, m += K^T 1 and, once R is formed
+// with the chunk's own P_p, E += K^T R, n += K^T s (the cross term R^KQ_B P_A of
+// Eq. AHLA-semidirect is in R).  Launches: K^T V of every chunk; its prefix sums;
+// A, R, A R and E's increments; E's prefix sums; outputs.  The states' [P | m] and
+// [E | n] start and end the sums as they lie.
+//
+// The scan that multiplied each chunk's R^KQ with P held 4.5 of 6.1 ms at
+// B1 H32 n1999 d128 bf16 with states; as prefix sums the call takes 405 us.
 #include <algorithm>
 
-#include "hla_internal.h"
-#include "simt_gemm.cuh"
+#include "chunk_simt.cuh"
 #include "sm103_prims.cuh"
 
 namespace hla {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kCols = 32;  // columns of [P | m] / [E | n] per scan block
-
-struct ALayout {
-    int BH, n, d, dv, C, nch;
-    // local record per (head, chunk), floats: R^KQ d*d | P d*dv | m d | E d*dv | n d | Rloc C*dv | sloc C
-    long long oR, oP, om, oE, on, oRl, osl, rec_local;
-    // carry record per (head, chunk): P d*dv | m d | E d*dv | n d  (the state before the chunk)
-    long long rec_carry, carry_base;
-};
-
 inline long long up16(long long x) { return (x + 15) / 16 * 16; }
 
-ALayout make_layout(int BH, int n, int d, int dv, int chunk) {
+struct ALayout {
+    int nch, len;  // chunks of a head; floats of a record [P | m] or [E | n]
+    // floats from the scratch start: P records, E records, A R (fp32 [BH][n][dv]), A s ([BH][n])
+    long long oP, oE, oNum, oDen, total;
+};
+
+ALayout make_layout(int BH, int n, int d, int dv) {
     ALayout L;
-    L.BH = BH; L.n = n; L.d = d; L.dv = dv;
-    L.C = std::min(chunk, (d == 128 || dv == 128) ? 32 : 64);  // shared-memory staging of the output kernel
-    L.nch = (n + L.C - 1) / L.C;
+    L.nch = (n + kC - 1) / kC;
+    L.len = d * dv + d;
+    const long long recs = (long long)BH * (L.nch + 1);
     long long o = 0;
-    L.oR = o; o += up16((long long)d * d);
-    L.oP = o; o += up16((long long)d * dv);
-    L.om = o; o += up16(d);
-    L.oE = o; o += up16((long long)d * dv);
-    L.on = o; o += up16(d);
-    L.oRl = o; o += up16((long long)L.C * dv);
-    L.osl = o; o += up16(L.C);
-    L.rec_local = o;
-    L.rec_carry = up16(2LL * d * dv + 2LL * d);
-    L.carry_base = (long long)BH * L.nch * L.rec_local;
+    L.oP = o; o += recs * L.len;
+    L.oE = o; o += recs * L.len;
+    L.oNum = o; o += up16((long long)BH * n * dv);
+    L.oDen = o; o += up16((long long)BH * n);
+    L.total = o;
     return L;
 }
 
-long long scratch_floats(const ALayout &L) { return L.carry_base + (long long)L.BH * L.nch * L.rec_carry; }
+struct AParams {
+    Records P, E;
+    float *num, *den;
+    int n, d, dv, normalized;
+    float eps;
+    int has_in;  // a state comes in: the first chunk has a carry
+    int direct;  // one chunk from a zero state: this launch writes the outputs
+    int need_E;  // E's increments of the last chunk are wanted too (final state)
+};
 
-__device__ __forceinline__ float *local_rec(float *ws, const ALayout &L, int hd, int c) {
-    return ws + ((long long)hd * L.nch + c) * L.rec_local;
-}
-__device__ __forceinline__ float *carry_rec(float *ws, const ALayout &L, int hd, int c) {
-    return ws + L.carry_base + ((long long)hd * L.nch + c) * L.rec_carry;
-}
-
-template <typename T>
-__device__ void load_tokens(const T *src, float *dst, int rows, int width, int Crows, int stride) {
-    for (int i = threadIdx.x; i < Crows * width; i += blockDim.x) {
-        const int r = i / width, c = i % width;
-        dst[r * stride + c] = i < rows * width ? to_f32(src[i]) : 0.f;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// kernel 1: chunk-local summaries (zero carry)
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) ahla_local_kernel(const T *__restrict__ q, const T *__restrict__ k,
-                                                              const T *__restrict__ v, float *ws, ALayout L) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, hd = blockIdx.y, d = L.d, dv = L.dv, C = L.C;
-    const int t0 = c * C, len = min(C, L.n - t0);
-    const int kd = d + 1, w1 = dv + 1;  // row strides of K and of the augmented [V | 1], [R | s]
-    float *Qs = sm, *Ks = Qs + C * d, *Vs = Ks + C * kd, *As = Vs + C * w1, *Rs = As + C * C;
-    load_tokens(q + ((long long)hd * L.n + t0) * d, Qs, len, d, C, d);
-    load_tokens(k + ((long long)hd * L.n + t0) * d, Ks, len, d, C, kd);
-    load_tokens(v + ((long long)hd * L.n + t0) * dv, Vs, len, dv, C, w1);
-    for (int t = threadIdx.x; t < C; t += blockDim.x) Vs[t * w1 + dv] = t < len ? 1.f : 0.f;
+// per chunk: A, [R | s], A [R | s] and the increments K^T [R | s] of [E | n].  Two token buffers serve in
+// turn as Q, K, V and R, as in the second-order kernel.
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT, 2)
+    ahla_chunk_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
+                      const __grid_constant__ AParams A) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    float *ss = stage + stage_floats<N>(), *dens = ss + kC;
+    const int c = blockIdx.x, hd = blockIdx.y, d = A.d, dv = A.dv, t0 = c * kC, len = min(kC, A.n - t0);
+    const long long tok = (long long)hd * A.n + t0;
+    const bool carry = c > 0 || A.has_in;
+    const float *Pp = A.P.at(hd, c);
+    load_tile<N>(b0, q + tok * d, len, d);
+    load_tile<N>(b1, k + tok * d, len, d);
     __syncthreads();
-    bgemm(As, C, Qs, d, 1, Ks, 1, kd, C, C, d, false, 1);          // A = L . Q K^T
-    __syncthreads();
-    bgemm(Rs, w1, As, C, 1, Vs, w1, 1, C, w1, C, false, 0, 1);     // [R_loc | s_loc] = A [V | 1]
-    __syncthreads();
-    float *rec = local_rec(ws, L, hd, c);
-    for (int idx = threadIdx.x; idx < C * w1; idx += blockDim.x) {
-        const int t = idx / w1, col = idx % w1;
-        if (col < dv) rec[L.oRl + t * dv + col] = Rs[idx];
-        else rec[L.osl + t] = Rs[idx];
-    }
-    bgemm(rec + L.oR, d, Ks, 1, kd, Qs, d, 1, d, d, C, false);      // R^KQ = K^T Q
-    bgemm(rec + L.oP, dv, Ks, 1, kd, Vs, w1, 1, d, dv, C, false);   // P = K^T V
-    bgemm(rec + L.om, 1, Ks, 1, kd, Vs + dv, w1, 1, d, 1, C, false); // m = K^T 1
-    bgemm(rec + L.oE, dv, Ks, 1, kd, Rs, w1, 1, d, dv, C, false);   // E = K^T R_loc
-    bgemm(rec + L.on, 1, Ks, 1, kd, Rs + dv, w1, 1, d, 1, C, false); // n = K^T s_loc
-}
-
-// ---------------------------------------------------------------------------
-// kernel 2: carry scan.  Block (column block, head) keeps columns [j0, j0 + 32) of
-// the augmented P' = [P | m] and E' = [E | n] (d x (dv + 1)); for every chunk it
-// records the carry-in, then E' += E'_c + R^KQ_c P'  (old P') and P' += P'_c.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) ahla_scan_kernel(float *ws, ALayout L, const float *state_in,
-                                                             float *state_out) {
-    extern __shared__ float sm[];
-    const int hd = blockIdx.y, d = L.d, dv = L.dv, j0 = blockIdx.x * kCols;
-    float *Pp = sm, *Ep = Pp + d * kCols, *Rq = Ep + d * kCols;  // d x 32, d x 32, d x d
-    const int ncol = min(kCols, dv + 1 - j0);
-    const long long st_len = 2LL * d * dv + 2LL * d;
-    auto P_at = [&](const float *base, int a, int j) { return j < dv ? base[a * dv + j] : base[(long long)d * dv + a]; };
-    // base layout of a state / carry record: P d*dv | m d | E d*dv | n d
-    const float *sin = state_in ? state_in + hd * st_len : nullptr;
-    for (int idx = threadIdx.x; idx < d * kCols; idx += blockDim.x) {
-        const int a = idx / kCols, j = idx % kCols;
-        const bool ok = j < ncol;
-        Pp[idx] = (ok && sin) ? P_at(sin, a, j0 + j) : 0.f;
-        Ep[idx] = (ok && sin) ? P_at(sin + (long long)d * dv + d, a, j0 + j) : 0.f;
-    }
-    __syncthreads();
-    for (int c = 0; c < L.nch; ++c) {
-        float *cr = carry_rec(ws, L, hd, c);
-        const float *lr = local_rec(ws, L, hd, c);
-        for (int idx = threadIdx.x; idx < d * ncol; idx += blockDim.x) {
-            const int a = idx / ncol, j = idx % ncol, col = j0 + j;
-            if (col < dv) {
-                cr[a * dv + col] = Pp[a * kCols + j];
-                cr[(long long)d * dv + d + a * dv + col] = Ep[a * kCols + j];
-            } else {
-                cr[(long long)d * dv + a] = Pp[a * kCols + j];
-                cr[2LL * d * dv + d + a] = Ep[a * kCols + j];
-            }
-        }
-        for (int idx = threadIdx.x; idx < d * d; idx += blockDim.x) Rq[idx] = lr[L.oR + idx];
-        __syncthreads();
-        // E' += E'_c + R^KQ_c P' (each thread owns elements (a, j); P' is read before it changes)
-        float newE[128 * kCols / kThreads], newP[128 * kCols / kThreads];
-        int cnt = 0;
-        for (int idx = threadIdx.x; idx < d * kCols; idx += blockDim.x, ++cnt) {
-            const int a = idx / kCols, j = idx % kCols;
-            float e = Ep[idx], p = Pp[idx];
-            if (j < ncol) {
-                float s = 0.f;
-                for (int b = 0; b < d; ++b) s += Rq[a * d + b] * Pp[b * kCols + j];
-                const int col = j0 + j;
-                e += s + (col < dv ? lr[L.oE + a * dv + col] : lr[L.on + a]);
-                p += col < dv ? lr[L.oP + a * dv + col] : lr[L.om + a];
-            }
-            newE[cnt] = e;
-            newP[cnt] = p;
-        }
-        __syncthreads();  // every P' read before it is updated
-        cnt = 0;
-        for (int idx = threadIdx.x; idx < d * kCols; idx += blockDim.x, ++cnt) {
-            Ep[idx] = newE[cnt];
-            Pp[idx] = newP[cnt];
-        }
+    const Tile<N> t;
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);
+    Acc<N> acc;
+    acc.zero();
+    float s = 0.f;
+    if (carry) {
+        s = row_dot(b0, N + 4, Pp + d * dv, d);
+        nn_carry<N, kPlain>(acc, t, b0, Pp, dv, d, dv, stage);
+    } else {
         __syncthreads();
     }
-    if (state_out) {
-        float *so = state_out + hd * st_len;
-        for (int idx = threadIdx.x; idx < d * ncol; idx += blockDim.x) {
-            const int a = idx / ncol, j = idx % ncol, col = j0 + j;
-            if (col < dv) {
-                so[a * dv + col] = Pp[a * kCols + j];
-                so[(long long)d * dv + d + a * dv + col] = Ep[a * kCols + j];
-            } else {
-                so[(long long)d * dv + a] = Pp[a * kCols + j];
-                so[2LL * d * dv + d + a] = Ep[a * kCols + j];
-            }
-        }
+    s += row_dot(Wt, kLdW, nullptr, kC);
+    if ((threadIdx.x & 1) == 0) ss[threadIdx.x >> 1] = s;
+    load_tile<N>(b0, v + tok * dv, len, dv);
+    __syncthreads();
+    nn_lower<N>(acc, t, Wt, b0);
+    const float den = row_dot(Wt, kLdW, ss, kC);
+    __syncthreads();
+    acc_to_smem<N>(acc, t, b0);  // R
+    const int r = threadIdx.x >> 1;
+    if ((threadIdx.x & 1) == 0) {
+        if (A.direct) dens[r] = den + A.eps;
+        else if (r < len) A.den[tok + r] = den;
     }
+    __syncthreads();
+    acc.zero();
+    nn_lower<N>(acc, t, Wt, b0);  // A R
+    if (A.direct) {
+        if (A.normalized) {
+#pragma unroll
+            for (int i = 0; i < Tile<N>::RM; ++i)
+#pragma unroll
+                for (int j = 0; j < Tile<N>::CM; ++j) acc.a[i][j] /= dens[t.row(i)];
+        }
+        acc_to_global<N, T>(acc, t, out + tok * dv, len, dv);
+    } else {
+        acc_to_global<N, float>(acc, t, A.num + tok * dv, len, dv);
+    }
+    if (c + 1 == A.E.nch && !A.need_E) return;
+    float *rec = A.E.at(hd, c);
+    atb_to_global<N>(t, rec, b1, b0, d, dv);
+    col_sums<N>(rec + d * dv, b1, ss, d);
 }
 
-// ---------------------------------------------------------------------------
-// kernel 3: outputs.  R = R_loc + Q P_p, s = s_loc + Q m_p, O = A R + Q E_p,
-// den = A s + Q n_p.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) ahla_out_kernel(const T *__restrict__ q, const T *__restrict__ k,
-                                                            T *__restrict__ out, float *ws, ALayout L, int normalized,
-                                                            float eps) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, hd = blockIdx.y, d = L.d, dv = L.dv, C = L.C;
-    const int t0 = c * C, len = min(C, L.n - t0);
-    const int kd = d + 1, w1 = dv + 1;
-    // Rs = [R | s] and Os = [O | den] (C x (dv + 1)); Ps = [P_p | m_p], Es = [E_p | n_p] (d x (dv + 1));
-    // Os takes the place of K, which is dead once A is formed
-    const int kw = kd > w1 ? kd : w1;
-    float *Qs = sm, *Ks = Qs + C * d, *Rs = Ks + C * kw, *As = Rs + C * w1, *Ps = As + C * C, *Es = Ps + d * w1;
-    float *Os = Ks;
-    load_tokens(q + ((long long)hd * L.n + t0) * d, Qs, len, d, C, d);
-    load_tokens(k + ((long long)hd * L.n + t0) * d, Ks, len, d, C, kd);
-    const float *lr = local_rec(ws, L, hd, c), *cr = carry_rec(ws, L, hd, c);
-    for (int idx = threadIdx.x; idx < d * w1; idx += blockDim.x) {
-        const int f = idx / w1, col = idx % w1;
-        Ps[idx] = col < dv ? cr[f * dv + col] : cr[(long long)d * dv + f];
-        Es[idx] = col < dv ? cr[(long long)d * dv + d + f * dv + col] : cr[2LL * d * dv + d + f];
+template <int N, typename T>
+cudaError_t forward_n(const Fwd2 &p, cudaStream_t s) {
+    const ALayout L = make_layout(p.BH, p.n, p.d, p.dv);
+    float *ws = reinterpret_cast<float *>(p.ws + kWsHeaderBytes);
+    const T *q = static_cast<const T *>(p.q), *k = static_cast<const T *>(p.k), *v = static_cast<const T *>(p.v);
+    T *out = static_cast<T *>(p.out);
+    const int d = p.d, dv = p.dv, nch = L.nch;
+    const long long st_len = 2LL * L.len;
+    cudaError_t e;
+    AParams A{};
+    A.P = {ws + L.oP, L.len, nch};
+    A.E = {ws + L.oE, L.len, nch};
+    A.num = ws + L.oNum; A.den = ws + L.oDen;
+    A.n = p.n; A.d = d; A.dv = dv; A.normalized = p.normalized; A.eps = p.eps;
+    A.has_in = p.state_in != nullptr;
+    A.need_E = p.state_out != nullptr;
+    A.direct = nch == 1 && !p.state_in;
+    const bool sums = nch > 1 || p.state_in || p.state_out;
+    // state_in and state_out may be the same memory: each value is read by the thread that replaces it
+    if (sums) {
+        if (nch > 0) {
+            SumJobs<T> jobs{};
+            jobs.j[0] = {k, v, A.P, d, dv, 1};
+            if ((e = launch_sums<N, T>(jobs, 1, p.BH, p.n, s))) return e;
+        }
+        ScanJobs scans{};
+        scans.j[0] = {A.P, p.state_in, st_len, p.state_out, st_len, 0};
+        if ((e = launch_scan(scans, 1, p.BH, s))) return e;
     }
-    for (int idx = threadIdx.x; idx < C * w1; idx += blockDim.x) {
-        const int t = idx / w1, col = idx % w1;
-        Rs[idx] = col < dv ? lr[L.oRl + t * dv + col] : lr[L.osl + t];
+    if (nch > 0) {
+        const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + 2 * kC) * (int)sizeof(float);
+        if ((e = cudaFuncSetAttribute(ahla_chunk_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
+            return e;
+        ahla_chunk_kernel<N, T><<<dim3(nch, p.BH), kCT, smem, s>>>(q, k, v, out, A);
+        if ((e = cudaGetLastError())) return e;
     }
-    __syncthreads();
-    bgemm(Rs, w1, Qs, d, 1, Ps, w1, 1, C, w1, d, true);             // [R | s] += Q [P_p | m_p]
-    bgemm(As, C, Qs, d, 1, Ks, 1, kd, C, C, d, false, 1);           // A = L . Q K^T
-    __syncthreads();
-    bgemm(Os, w1, As, C, 1, Rs, w1, 1, C, w1, C, false, 0, 1);      // [O | den] = A [R | s]
-    bgemm(Os, w1, Qs, d, 1, Es, w1, 1, C, w1, d, true);             //   + Q [E_p | n_p]
-    __syncthreads();
-    T *o = out + ((long long)hd * L.n + t0) * dv;
-    for (int idx = threadIdx.x; idx < len * dv; idx += blockDim.x) {
-        const int t = idx / dv, col = idx % dv;
-        const float x = Os[t * w1 + col];
-        from_f32(&o[idx], normalized ? x / (Os[t * w1 + dv] + eps) : x);
-    }
+    if (!sums) return cudaSuccess;
+    ScanJobs scans{};
+    scans.j[0] = {A.E, p.state_in ? p.state_in + L.len : nullptr, st_len,
+                  p.state_out ? p.state_out + L.len : nullptr, st_len, 0};
+    if ((e = launch_scan(scans, 1, p.BH, s))) return e;
+    if (nch == 0 || A.direct) return cudaSuccess;
+    const OutParams O{A.E, A.num, A.den, p.n, d, dv, p.normalized, p.eps, A.has_in};
+    return launch_out<N, T>(q, out, O, p.BH, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -381,46 +313,18 @@ ahla_step_staged_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
     }
 }
 
-template <typename T>
-cudaError_t forward_t(const Fwd2 &p, cudaStream_t stream) {
-    const ALayout L = make_layout(p.BH, p.n, p.d, p.dv, p.chunk);
-    float *ws = reinterpret_cast<float *>(p.ws + kWsHeaderBytes);
-    const T *q = static_cast<const T *>(p.q), *k = static_cast<const T *>(p.k), *v = static_cast<const T *>(p.v);
-    cudaError_t e;
-    if (L.nch > 0) {
-        const size_t sm1 = sizeof(float) * ((size_t)L.C * (2 * L.d + 1 + 2 * (L.dv + 1)) + (size_t)L.C * L.C);
-        if ((e = cudaFuncSetAttribute(ahla_local_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1)))
-            return e;
-        ahla_local_kernel<T><<<dim3(L.nch, p.BH), kThreads, sm1, stream>>>(q, k, v, ws, L);
-        if ((e = cudaGetLastError())) return e;
-    }
-    const size_t sm2 = sizeof(float) * ((size_t)2 * p.d * kCols + (size_t)p.d * p.d);
-    if ((e = cudaFuncSetAttribute(ahla_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2))) return e;
-    ahla_scan_kernel<<<dim3((p.dv + 1 + kCols - 1) / kCols, p.BH), kThreads, sm2, stream>>>(ws, L, p.state_in,
-                                                                                            p.state_out);
-    if ((e = cudaGetLastError())) return e;
-    if (L.nch > 0) {
-        const size_t sm3 = sizeof(float) * ((size_t)L.C * (L.d + std::max(L.d + 1, L.dv + 1) + L.dv + 1) +
-                                            (size_t)L.C * L.C + 2 * (size_t)L.d * (L.dv + 1));
-        if ((e = cudaFuncSetAttribute(ahla_out_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)))
-            return e;
-        ahla_out_kernel<T><<<dim3(L.nch, p.BH), kThreads, sm3, stream>>>(q, k, static_cast<T *>(p.out), ws, L,
-                                                                         p.normalized, p.eps);
-        if ((e = cudaGetLastError())) return e;
-    }
-    return cudaSuccess;
-}
-
 }  // namespace
 
-size_t ahla_workspace_bytes_internal(int BH, int n, int d, int dv, int chunk) {
-    const ALayout L = make_layout(BH, n, d, dv, chunk);
-    return kWsHeaderBytes + sizeof(float) * (size_t)scratch_floats(L);
+size_t ahla_workspace_bytes_internal(int BH, int n, int d, int dv, int) {
+    return kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
 }
 
 cudaError_t ahla_forward_launch(const Fwd2 &p, cudaStream_t stream) {
     if (ahla_tc_applicable(p)) return ahla_tc_forward(p, stream);
-    return p.dt == HLA_BF16 ? forward_t<__nv_bfloat16>(p, stream) : forward_t<float>(p, stream);
+    return with_padded_size(p.d, p.dv, [&](auto size) {
+        constexpr int N = decltype(size)::value;
+        return p.dt == HLA_BF16 ? forward_n<N, __nv_bfloat16>(p, stream) : forward_n<N, float>(p, stream);
+    });
 }
 
 cudaError_t ahla_step_launch(const void *q, const void *k, const void *v, void *out, hla_dtype dt, int BH, int d,

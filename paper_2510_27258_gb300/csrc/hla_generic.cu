@@ -181,52 +181,6 @@ __global__ void __launch_bounds__(kCT, 2)
     col_sums<N>(rec + d * dv, b1, nullptr, d);
 }
 
-// ---------------------------------------------------------------------------
-// masked outputs: num = T V + Q D_p, den = T 1 + Q e_p
-// ---------------------------------------------------------------------------
-template <int N, typename T>
-__global__ void __launch_bounds__(kCT)
-    g2_out_kernel(const T *__restrict__ q, T *__restrict__ out, const __grid_constant__ GParams P) {
-    extern __shared__ __align__(16) float sm[];
-    float *b0 = sm, *stage = b0 + tile_floats<N>(), *dens = stage + stage_floats<N>();
-    const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
-    const long long tok = (long long)hd * P.n + t0;
-    const bool carry = c > 0 || P.has_in;
-    const float *Dp = P.D.at(hd, c);
-    const Tile<N> t;
-    Acc<N> acc;
-    acc.zero();
-    float den = 0.f;
-    if (carry) {
-        load_tile<N>(b0, q + tok * d, len, d);
-        __syncthreads();
-        if (P.normalized) den = row_dot(b0, N + 4, Dp + d * dv, d);
-        nn_carry<N, kPlain>(acc, t, b0, Dp, dv, d, dv, stage);
-    }
-    if (P.normalized) {
-        const int r = threadIdx.x >> 1;
-        if ((threadIdx.x & 1) == 0) dens[r] = (r < len ? P.den[tok + r] : 0.f) + den + P.eps;
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < Tile<N>::RM; ++i) {
-        const int r = t.row(i);
-        if (r >= len) continue;
-#pragma unroll
-        for (int j = 0; j < Tile<N>::CM; j += 4) {
-            if (t.col(j) >= dv) continue;
-            const float4 x = *reinterpret_cast<const float4 *>(P.num + (tok + r) * dv + t.col(j));
-            float y[4] = {acc.a[i][j] + x.x, acc.a[i][j + 1] + x.y, acc.a[i][j + 2] + x.z, acc.a[i][j + 3] + x.w};
-            if (P.normalized) {
-                const float den_r = dens[r];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) y[u] /= den_r;
-            }
-            Vec<T>::store4(out + (tok + r) * dv + t.col(j), y);
-        }
-    }
-}
-
 template <int N, typename T>
 cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s) {
     const T *q = static_cast<const T *>(p.q), *k = static_cast<const T *>(p.k), *v = static_cast<const T *>(p.v);
@@ -277,11 +231,8 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
         scans.j[0] = {P.D, p.state_in ? total : nullptr, head, total, head, 0};
         if ((e = launch_scan(scans, 1, L.BH, s))) return e;
         if (nch > 0 && !P.direct) {
-            const int smem = (tile_floats<N>() + stage_floats<N>() + kC) * (int)sizeof(float);
-            if ((e = cudaFuncSetAttribute(g2_out_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
-                return e;
-            g2_out_kernel<N, T><<<grid, kCT, smem, s>>>(q, out, P);
-            if ((e = cudaGetLastError())) return e;
+            const OutParams O{P.D, P.num, P.den, L.n, d, dv, p.normalized, p.eps, P.has_in};
+            if ((e = launch_out<N, T>(q, out, O, L.BH, s))) return e;
         }
     }
     if (p.state_out) {

@@ -70,3 +70,25 @@ def test_forward_overlapping_states(hla):
     ref, rst = oracle.hla2_serial(_flat(q), _flat(k), _flat(v), state_in=st0, return_state=True)
     assert rowerr(_flat(out.cpu().numpy()), ref) < TOL["f32"]
     assert np.abs(buf[:H].cpu().numpy() - rst).max() <= 1e-4 * np.abs(rst).max()
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+@pytest.mark.parametrize("d,dv", SIZES)
+def test_ahla(hla, n, d, dv):
+    """AHLA outputs, plain and normalised, and from a state, with the final state written where the state came from."""
+    B, H = 1, 3
+    pq, pk, pv = (_flat(x) for x in hla_inputs.make_qkv(B, H, 40, d, dv, seed=n, dtype="f32"))
+    st0 = oracle.ahla_serial(pq, pk, pv, return_state=True)[1].astype(np.float32)
+    q, k, v = hla_inputs.make_qkv(B, H, n, d, dv, seed=n + 1, dtype="f32")
+    t = _gpu(q, k, v)
+    num = hla.ahla_forward(*t)
+    o = hla.ahla_forward(*t, normalized=True, eps=hla_inputs.EPS)
+    st = torch.from_numpy(st0).to(DEV).reshape(B, H, -1)
+    cont = hla.ahla_forward(*t, state_in=st, state_out=st)
+    torch.cuda.synchronize()
+    ref, den = oracle.ahla_serial(_flat(q), _flat(k), _flat(v), return_den=True)
+    assert rowerr(_flat(num.cpu().numpy()), ref) < TOL["f32"]
+    check_normalized(_flat(o.cpu().numpy()), _flat(num.cpu().numpy()), ref, den, hla_inputs.EPS, TOL["f32"])
+    ref, rst = oracle.ahla_serial(_flat(q), _flat(k), _flat(v), state_in=st0, return_state=True)
+    assert rowerr(_flat(cont.cpu().numpy()), ref) < TOL["f32"]
+    assert np.abs(st.reshape(B * H, -1).cpu().numpy() - rst).max() <= 2e-5 * np.abs(rst).max()

@@ -1,7 +1,7 @@
 // Gradients of masked second-order HLA: a reverse chunk scan with the forward
 // states checkpointed at chunk boundaries (Sec. "Chunk-parallel training via
 // associative scans": the adjoint of the semidirect product applied by a
-// reverse scan), fp32 SIMT kernels.
+// reverse scan), in fp32 on the CUDA cores.
 //
 // With x_j = S_j q_j, T_tj = q_t . x_j and L = sum_t g_t . o_t, the forward is
 // o_t = sum_{j<=t} T_tj v_j (proof of Theorem 1), so with P_tj = g_t . v_j:
@@ -10,370 +10,371 @@
 //   dk_i = sum_{j>=i} [ (q_j . k_i) y_j + (y_j . k_i) q_j ].
 // The ratio-normalised output o = num / (den + eps) is the same computation
 // with values [v | 1] (den is the extra column) and upstream gradient
-// [g / (den + eps) | -(g . o) / (den + eps)]: every kernel works with the
-// augmented width W = dv + 1 (for the plain output the extra gradient column
-// is zero).
+// [g' | u] = [g / (den + eps) | -(g . o) / (den + eps)]; the plain output has
+// g' = g, u = 0 and skips the extra column.
 //
-// Per chunk (rows = its tokens; p = prefix before the chunk, s = suffix after):
-//   forward:  W_c = L . (Q K^T),  X = W_c K + Q S_p,  T = L . (Q X^T),
-//             num' = T V' + Q D_p            (S_p, D_p = sum x v'^T: prefixes)
-//   backward: P = L . (G' V'^T),  Y = P^T Q + V' Gam_s,
-//             dV' = T^T G' + X Gam_s^T,
-//             dQ = P X + G' D_p^T + Y S_p + (L . (Y K^T)) K,
-//             dK = K Lam_s + W_c^T Y + (L . (Y K^T))^T Q,
-// with the suffix sums Gam_s = sum g' q^T (W x d) and Lam_s = sum (y q^T + q y^T)
-// (d x d).  The forward prefixes compose as D_p += X_loc^T V' + S_p (Q^T V')
-// (the semidirect product, D-form); the suffixes compose in reverse as
-//   Lam += Lam_loc + Gam_s^T M + M^T Gam_s  (M = V'^T Q, Lam_loc from the
-//   chunk's own P^T Q),  Gam += G'^T Q,
-// the adjoint of that product.  Five launches: forward local summaries, the
-// forward prefix scan (the checkpoints), per-chunk gradient inputs and local
-// reverse summaries, the reverse scan, per-chunk gradients.
-#include <algorithm>
-
-#include "hla_internal.h"
-#include "simt_gemm.cuh"
+// Per 64-token chunk (rows = its tokens; p = sum before the chunk, s = sum after):
+//   forward:  W = L . (Q K^T),  X = W K + Q S_p,  T = L . (Q X^T),
+//             num = T V + Q D_p,  den = T 1 + Q e_p,
+//   backward: P = L . (G' V^T + u 1^T),  Y = P^T Q + V Gam_s + 1 h_s^T,
+//             dV = T^T G' + X Gam_s^T,   B = L . (Y K^T),
+//             dQ = P X + G' D_p^T + u e_p^T + Y S_p + B K,
+//             dK = K (Lam_s + Lam_s^T) + W^T Y + B^T Q.
+// Every carry is a plain sum over the chunks: before the chunk S += K^T K,
+// D += X^T V, e += X^T 1; after it Gam^T += Q^T G', h += Q^T u, Lam += Q^T Y.
+// X is formed with the chunk's own S_p and Y with its own Gam_s, which is where
+// the cross terms of the semidirect product and of its adjoint go, so no carry
+// is multiplied along the sequence.  Launches (normalised; the plain output
+// has Gam's increments in the first and needs no third pair):
+//   K^T K | sums of S | X, D, e, num, den | sums of D, e | G', u, Gam, h |
+//   sums of Gam, h from the end | Y, Lam | sums of Lam from the end | dQ, dK, dV.
+//
+// At B2 H16 n4096 d128 normalised the two scans that multiplied carries took 24
+// of 36.6 ms; as elementwise sums, with the register-tiled products of
+// chunk_simt.cuh, the call takes 2.33 ms.
+#include "chunk_simt.cuh"
 
 namespace hla {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kCols = 32;
-
-struct BLayout {
-    int BH, n, d, dv, W, C, nch;
-    long long fl_S, fl_DL, fl_C, fl_len;            // forward local: S_c d*d | DL_c d*W | C_c d*W
-    long long fc_S, fc_D, fc_DT, fc_len;            // forward carry: S_p d*d | D_p d*W | D_p^T W*d
-    long long bl_G, bl_Gam, bl_M, bl_Lam, bl_len;   // backward local: G' C*W | Gam_c W*d | M_c W*d | Lam_c d*d
-    long long bc_Gam, bc_Lam, bc_GamT, bc_len;      // backward carry: Gam_s W*d | Lam_s d*d | Gam_s^T d*W
-    long long o_fl, o_fc, o_bl, o_bc, total;        // floats from the scratch start
-};
-
 inline long long up16(long long x) { return (x + 15) / 16 * 16; }
 
-BLayout make_layout(int BH, int n, int d, int dv, int chunk) {
+struct BLayout {
+    int nch;
+    // floats from the scratch start: S | D, e | Gam^T, h | Lam records; X, Y ([BH][n][d]); num, then G'
+    // ([BH][n][dv]); den, then u ([BH][n])
+    long long oS, oD, oG, oL, oX, oY, oNum, oDen, total;
+};
+
+BLayout make_layout(int BH, int n, int d, int dv) {
     BLayout L;
-    L.BH = BH; L.n = n; L.d = d; L.dv = dv; L.W = dv + 1;
-    L.C = std::min(chunk, (d == 128 || dv == 128) ? 32 : 64);
-    L.nch = (n + L.C - 1) / L.C;
-    const long long dd = (long long)d * d, dW = (long long)d * L.W;
-    L.fl_S = 0; L.fl_DL = up16(dd); L.fl_C = L.fl_DL + up16(dW); L.fl_len = L.fl_C + up16(dW);
-    L.fc_S = 0; L.fc_D = up16(dd); L.fc_DT = L.fc_D + up16(dW); L.fc_len = L.fc_DT + up16(dW);
-    L.bl_G = 0; L.bl_Gam = up16((long long)L.C * L.W); L.bl_M = L.bl_Gam + up16(dW); L.bl_Lam = L.bl_M + up16(dW);
-    L.bl_len = L.bl_Lam + up16(dd);
-    L.bc_Gam = 0; L.bc_Lam = up16(dW); L.bc_GamT = L.bc_Lam + up16(dd); L.bc_len = L.bc_GamT + up16(dW);
-    const long long chunks = (long long)BH * L.nch;
-    L.o_fl = 0;
-    L.o_fc = L.o_fl + chunks * L.fl_len;
-    L.o_bl = L.o_fc + chunks * L.fc_len;
-    L.o_bc = L.o_bl + chunks * L.bl_len;
-    L.total = L.o_bc + chunks * L.bc_len;
+    L.nch = (n + kC - 1) / kC;
+    const long long recs = (long long)BH * (L.nch + 1), tok = (long long)BH * n;
+    long long o = 0;
+    L.oS = o; o += recs * d * d;
+    L.oD = o; o += recs * (d * dv + d);
+    L.oG = o; o += recs * (d * dv + d);
+    L.oL = o; o += recs * d * d;
+    L.oX = o; o += up16(tok * d);
+    L.oY = o; o += up16(tok * d);
+    L.oNum = o; o += up16(tok * dv);
+    L.oDen = o; o += up16(tok);
+    L.total = o;
     return L;
 }
 
-__device__ __forceinline__ float *rec(float *ws, long long base, long long len, const BLayout &L, int hd, int c) {
-    return ws + base + ((long long)hd * L.nch + c) * len;
-}
-
-// token rows of a chunk into shared memory (zero beyond the sequence); with ones, column
-// `width` of each valid row is 1 (the augmented value column)
 template <typename T>
-__device__ void load_rows(const T *src, float *dst, int rows, int width, int Crows, int stride, bool ones) {
-    for (int i = threadIdx.x; i < Crows * stride; i += blockDim.x) {
-        const int r = i / stride, c = i % stride;
-        float x = 0.f;
-        if (r < rows) x = c < width ? to_f32(src[(long long)r * width + c]) : (ones && c == width ? 1.f : 0.f);
-        dst[i] = x;
+struct BParams {
+    const T *q, *k, *v, *g;
+    T *dq, *dk, *dv_out;
+    Records S, D, Gam, Lam;
+    float *X, *Y, *num, *den;  // num, den become G', u
+    int n, d, dv, normalized;
+    float eps;
+};
+
+// the chunk of this block
+template <typename T>
+struct Chunk {
+    int c, hd, len;
+    long long tok;
+    bool before, after;  // chunks before / after it
+    __device__ Chunk(const BParams<T> &P)
+        : c(blockIdx.x), hd(blockIdx.y), len(min(kC, P.n - (int)blockIdx.x * kC)),
+          tok((long long)blockIdx.y * P.n + blockIdx.x * kC), before(blockIdx.x > 0),
+          after((int)blockIdx.x + 1 < P.S.nch) {}
+};
+
+// G' rows of a chunk (the output gradient itself for the plain output) and u
+template <int N, typename T>
+__device__ __forceinline__ void load_upstream(float *dst, float *us, const BParams<T> &P, const Chunk<T> &ch) {
+    if (P.normalized) {
+        load_tile<N>(dst, P.num + ch.tok * P.dv, ch.len, P.dv);
+        if (us && threadIdx.x < kC) us[threadIdx.x] = threadIdx.x < ch.len ? P.den[ch.tok + threadIdx.x] : 0.f;
+    } else {
+        load_tile<N>(dst, P.g + ch.tok * P.dv, ch.len, P.dv);
     }
 }
 
 // ---------------------------------------------------------------------------
-// B1: forward local summaries S_c = K^T K, DL_c = (W_c K)^T V', C_c = Q^T V'
+// X, the increments X^T V, X^T 1 of D and e; normalised: T V and T 1
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) bwd_fwd_local(const T *q, const T *k, const T *v, float *ws, BLayout L) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, hd = blockIdx.y, d = L.d, W = L.W, C = L.C, t0 = c * C, len = min(C, L.n - t0);
-    const int kd = d + 1;
-    float *Qs = sm, *Ks = Qs + C * d, *Vs = Ks + C * kd, *Ws = Vs + C * W, *Xs = Ws + C * C;
-    load_rows(q + ((long long)hd * L.n + t0) * d, Qs, len, d, C, d, false);
-    load_rows(k + ((long long)hd * L.n + t0) * d, Ks, len, d, C, kd, false);
-    load_rows(v + ((long long)hd * L.n + t0) * L.dv, Vs, len, L.dv, C, W, true);
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT, 2) bwd_x_kernel(const __grid_constant__ BParams<T> P) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    const Chunk<T> ch(P);
+    const int d = P.d, dv = P.dv;
+    load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
+    load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
     __syncthreads();
-    bgemm(Ws, C, Qs, d, 1, Ks, 1, kd, C, C, d, false, 1);        // W_c = L . Q K^T
+    const Tile<N> t;
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);
+    Acc<N> acc;
+    acc.zero();
+    if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);
+    else __syncthreads();
+    nn_lower<N>(acc, t, Wt, b1);
+    acc_to_global<N, float>(acc, t, P.X + ch.tok * d, ch.len, d);
     __syncthreads();
-    bgemm(Xs, d, Ws, C, 1, Ks, kd, 1, C, d, C, false, 0, 1);     // X_loc = W_c K
+    acc_to_smem<N>(acc, t, b1);  // X
     __syncthreads();
-    float *fl = rec(ws, L.o_fl, L.fl_len, L, hd, c);
-    bgemm(fl + L.fl_S, d, Ks, 1, kd, Ks, kd, 1, d, d, C, false);  // K^T K
-    bgemm(fl + L.fl_DL, W, Xs, 1, d, Vs, W, 1, d, W, C, false);   // X_loc^T V'
-    bgemm(fl + L.fl_C, W, Qs, 1, d, Vs, W, 1, d, W, C, false);    // Q^T V'
+    if (P.normalized) {
+        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
+        __syncthreads();
+    }
+    load_tile<N>(b0, P.v + ch.tok * dv, ch.len, dv);
+    __syncthreads();
+    if (P.normalized) {
+        const float den = row_dot(Wt, kLdW, nullptr, kC);
+        const int r = threadIdx.x >> 1;
+        if ((threadIdx.x & 1) == 0 && r < ch.len) P.den[ch.tok + r] = den;
+        acc.zero();
+        nn_lower<N>(acc, t, Wt, b0);
+        acc_to_global<N, float>(acc, t, P.num + ch.tok * dv, ch.len, dv);
+    }
+    if (!ch.after) return;
+    float *rec = P.D.at(ch.hd, ch.c);
+    atb_to_global<N>(t, rec, b1, b0, d, dv);
+    col_sums<N>(rec + d * dv, b1, nullptr, d);
 }
 
 // ---------------------------------------------------------------------------
-// B2: forward prefix scan (the checkpoints).  Block (column block of D, head) keeps
-// the whole S_p and 32 columns of D_p; per chunk it records them, then
-// D_p += DL_c + S_p C_c and S_p += S_c.
+// normalised: num and den of the whole prefix, G' and u in their place, and the increments Q^T G',
+// Q^T u of Gam^T and h
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) bwd_fwd_scan(float *ws, BLayout L) {
-    extern __shared__ float sm[];
-    const int hd = blockIdx.y, d = L.d, W = L.W, j0 = blockIdx.x * kCols, ncol = min(kCols, W - j0);
-    // S_p (d x d), D_p columns (d x 32), the chunk's C_c and DL_c columns staged per chunk (d x 32 each)
-    float *Sp = sm, *Dp = Sp + d * d, *Cc = Dp + d * kCols, *DLc = Cc + d * kCols;
-    for (int i = threadIdx.x; i < d * d; i += blockDim.x) Sp[i] = 0.f;
-    for (int i = threadIdx.x; i < d * kCols; i += blockDim.x) Dp[i] = 0.f;
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT, 2) bwd_upstream_kernel(const __grid_constant__ BParams<T> P) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *stage = b1 + tile_floats<N>(), *us = stage + stage_floats<N>();
+    const Chunk<T> ch(P);
+    const int d = P.d, dv = P.dv;
+    load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
     __syncthreads();
-    for (int c = 0; c < L.nch; ++c) {
-        float *fc = rec(ws, L.o_fc, L.fc_len, L, hd, c);
-        const float *fl = rec(ws, L.o_fl, L.fl_len, L, hd, c);
-        if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < d * d; i += blockDim.x) fc[L.fc_S + i] = Sp[i];
-        for (int i = threadIdx.x; i < d * kCols; i += blockDim.x) {
-            const int a = i / kCols, j = i % kCols;
-            if (j < ncol) {
-                fc[L.fc_D + a * W + j0 + j] = Dp[i];
-                Cc[i] = fl[L.fl_C + a * W + j0 + j];
-                DLc[i] = fl[L.fl_DL + a * W + j0 + j];
+    const Tile<N> t;
+    Acc<N> acc;
+    acc.zero();
+    float den = 0.f;
+    if (ch.before) {
+        const float *Dp = P.D.at(ch.hd, ch.c);
+        den = row_dot(b0, N + 4, Dp + d * dv, d);
+        nn_carry<N, kPlain>(acc, t, b0, Dp, dv, d, dv, stage);
+    }
+    acc_to_smem<N>(acc, t, b1);  // Q D_p
+    __syncthreads();
+    // two threads a row, each with every other group of four columns
+    const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
+    const bool ok = r < ch.len;
+    const float inv = ok ? 1.f / (P.den[ch.tok + r] + den + P.eps) : 0.f;
+    float *num = P.num + (ch.tok + r) * dv, *row = b1 + r * (N + 4);
+    const T *g = P.g + (ch.tok + r) * dv;
+    float go = 0.f;
+    for (int c = 4 * h; c < N; c += 8) {
+        float gp[4] = {0.f, 0.f, 0.f, 0.f};
+        if (ok && c < dv) {
+            const float4 x = *reinterpret_cast<const float4 *>(num + c), y = *reinterpret_cast<const float4 *>(row + c);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                gp[u] = to_f32(g[c + u]) * inv;
+                go = fmaf(gp[u], f4(x, u) + f4(y, u), go);  // g . o
+            }
+            *reinterpret_cast<float4 *>(num + c) = make_float4(gp[0], gp[1], gp[2], gp[3]);
+        }
+        *reinterpret_cast<float4 *>(row + c) = make_float4(gp[0], gp[1], gp[2], gp[3]);
+    }
+    go += __shfl_xor_sync(0xffffffffu, go, 1);
+    if (h == 0) {
+        us[r] = -go * inv;
+        if (ok) P.den[ch.tok + r] = -go * inv;
+    }
+    __syncthreads();
+    if (!ch.before) return;
+    float *rec = P.Gam.at(ch.hd, ch.c);
+    atb_to_global<N>(t, rec, b0, b1, d, dv);
+    col_sums<N>(rec + d * dv, b0, us, d);
+}
+
+// ---------------------------------------------------------------------------
+// Y and the increments Q^T Y of Lam
+// ---------------------------------------------------------------------------
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT, 2) bwd_y_kernel(const __grid_constant__ BParams<T> P) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    float *us = stage + stage_floats<N>();
+    const Chunk<T> ch(P);
+    const int d = P.d, dv = P.dv;
+    load_upstream<N>(b0, us, P, ch);
+    load_tile<N>(b1, P.v + ch.tok * dv, ch.len, dv);
+    __syncthreads();
+    const Tile<N> t;
+    nt_masked(Wt, b0, b1, N + 4, dv, P.normalized ? us : nullptr);  // P
+    Acc<N> acc;
+    acc.zero();
+    if (ch.after) {
+        const float *Gs = P.Gam.at(ch.hd, ch.c);
+        nn_carry<N, kTransposed>(acc, t, b1, Gs, dv, dv, d, stage);  // V Gam_s
+        if (P.normalized) {
+#pragma unroll
+            for (int j = 0; j < Tile<N>::CM; ++j) {
+                const float h = t.col(j) < d ? Gs[d * dv + t.col(j)] : 0.f;
+#pragma unroll
+                for (int i = 0; i < Tile<N>::RM; ++i) acc.a[i][j] += h;
             }
         }
-        for (int i = threadIdx.x; i < d * ncol; i += blockDim.x) {  // D_p^T, consecutive threads on consecutive a
-            const int j = i / d, a = i % d;
-            fc[L.fc_DT + (long long)(j0 + j) * d + a] = Dp[a * kCols + j];
-        }
+    } else {
         __syncthreads();
-        // D_new = D_p + DL_c + S_p C_c (old S_p); each thread keeps its results in registers
-        float dn[128 * kCols / kThreads];
-        int cnt = 0;
-        for (int i = threadIdx.x; i < d * kCols; i += blockDim.x, ++cnt) {
-            const int a = i / kCols, j = i % kCols;
-            float x = 0.f;
-            if (j < ncol) {
-                x = Dp[i] + DLc[i];
-                for (int b = 0; b < d; ++b) x += Sp[a * d + b] * Cc[b * kCols + j];
+    }
+    load_tile<N>(b1, P.q + ch.tok * d, ch.len, d);
+    __syncthreads();
+    tn_lower<N>(acc, t, Wt, b1);  // P^T Q
+    acc_to_global<N, float>(acc, t, P.Y + ch.tok * d, ch.len, d);
+    if (!ch.before) return;
+    acc_to_smem<N>(acc, t, b0);  // Y; its rows beyond the sequence meet zero rows of Q
+    __syncthreads();
+    atb_to_global<N>(t, P.Lam.at(ch.hd, ch.c), b1, b0, d, d);
+}
+
+// ---------------------------------------------------------------------------
+// the gradients: blockIdx.z 0 dQ, 1 dK, 2 dV
+// ---------------------------------------------------------------------------
+template <int N, typename T>
+__global__ void __launch_bounds__(kCT, 2) bwd_grad_kernel(const __grid_constant__ BParams<T> P) {
+    extern __shared__ __align__(16) float sm[];
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    float *us = stage + stage_floats<N>();
+    const Chunk<T> ch(P);
+    const int d = P.d, dv = P.dv;
+    const Tile<N> t;
+    Acc<N> acc;
+    acc.zero();
+    if (blockIdx.z == 0) {
+        load_upstream<N>(b0, us, P, ch);
+        load_tile<N>(b1, P.v + ch.tok * dv, ch.len, dv);
+        __syncthreads();
+        nt_masked(Wt, b0, b1, N + 4, dv, P.normalized ? us : nullptr);  // P
+        if (ch.before) {
+            const float *Dp = P.D.at(ch.hd, ch.c);
+            nn_carry<N, kTransposed>(acc, t, b0, Dp, dv, dv, d, stage);  // G' D_p^T
+            if (P.normalized) {
+#pragma unroll
+                for (int j = 0; j < Tile<N>::CM; ++j) {
+                    const float e = t.col(j) < d ? Dp[d * dv + t.col(j)] : 0.f;
+#pragma unroll
+                    for (int i = 0; i < Tile<N>::RM; ++i) acc.a[i][j] = fmaf(us[t.row(i)], e, acc.a[i][j]);
+                }
             }
-            dn[cnt] = x;
+        } else {
+            __syncthreads();
         }
+        load_tile<N>(b1, P.X + ch.tok * d, ch.len, d);
         __syncthreads();
-        cnt = 0;
-        for (int i = threadIdx.x; i < d * kCols; i += blockDim.x, ++cnt) Dp[i] = dn[cnt];
-        for (int i = threadIdx.x; i < d * d; i += blockDim.x) Sp[i] += fl[L.fl_S + i];
+        nn_lower<N>(acc, t, Wt, b1);  // P X
         __syncthreads();
+        load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
+        load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
+        __syncthreads();
+        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
+        if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);  // Y S_p
+        else __syncthreads();
+        nn_lower<N>(acc, t, Wt, b1);  // B K
+        acc_to_global<N, T>(acc, t, P.dq + ch.tok * d, ch.len, d);
+    } else if (blockIdx.z == 1) {
+        load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
+        load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
+        __syncthreads();
+        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
+        if (ch.after) nn_carry<N, kSymmetric>(acc, t, b1, P.Lam.at(ch.hd, ch.c), d, d, d, stage);
+        else __syncthreads();
+        load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
+        __syncthreads();
+        tn_lower<N>(acc, t, Wt, b0);  // B^T Q
+        __syncthreads();
+        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // W
+        __syncthreads();
+        load_tile<N>(b1, P.Y + ch.tok * d, ch.len, d);
+        __syncthreads();
+        tn_lower<N>(acc, t, Wt, b1);  // W^T Y
+        acc_to_global<N, T>(acc, t, P.dk + ch.tok * d, ch.len, d);
+    } else {
+        load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
+        load_tile<N>(b1, P.X + ch.tok * d, ch.len, d);
+        __syncthreads();
+        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
+        if (ch.after) nn_carry<N, kPlain>(acc, t, b1, P.Gam.at(ch.hd, ch.c), dv, d, dv, stage);  // X Gam_s^T
+        else __syncthreads();
+        load_upstream<N>(b0, static_cast<float *>(nullptr), P, ch);
+        __syncthreads();
+        tn_lower<N>(acc, t, Wt, b0);  // T^T G'
+        acc_to_global<N, T>(acc, t, P.dv_out + ch.tok * dv, ch.len, dv);
     }
 }
 
-// Recompute of a chunk's forward quantities shared by B3 and B5: W_c, X, T (rows = tokens).
-__device__ void chunk_forward(const float *Qs, const float *Ks, int kd, const float *Sp, float *Ws, float *Xs,
-                              float *Ts, int C, int d) {
-    bgemm(Ws, C, Qs, d, 1, Ks, 1, kd, C, C, d, false, 1);        // W_c = L . Q K^T
-    __syncthreads();
-    bgemm(Xs, d, Ws, C, 1, Ks, kd, 1, C, d, C, false, 0, 1);     // X = W_c K
-    bgemm(Xs, d, Qs, d, 1, Sp, d, 1, C, d, d, true);             //   + Q S_p
-    __syncthreads();
-    bgemm(Ts, C, Qs, d, 1, Xs, 1, d, C, C, d, false, 1);         // T = L . Q X^T
-    __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
-// B3: per chunk, the upstream gradient G' (C x W) and the local reverse summaries
-// Gam_c = G'^T Q, M_c = V'^T Q, Lam_c = Y_loc^T Q + Q^T Y_loc with Y_loc = P^T Q.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) bwd_local1(const T *q, const T *k, const T *v, const T *dout, float *ws,
-                                                       BLayout L, int normalized, float eps) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, hd = blockIdx.y, d = L.d, W = L.W, dv = L.dv, C = L.C, t0 = c * C;
-    const int len = min(C, L.n - t0), kd = d + 1;
-    float *Qs = sm, *Ks = Qs + C * d, *Vs = Ks + C * kd, *Gs = Vs + C * W, *Ws = Gs + C * W, *Xs = Ws + C * C;
-    float *Ts = Xs + C * d, *Ns = Ts + C * C;  // Ns: num' (C x W), then Y_loc (C x d)
-    load_rows(q + ((long long)hd * L.n + t0) * d, Qs, len, d, C, d, false);
-    load_rows(k + ((long long)hd * L.n + t0) * d, Ks, len, d, C, kd, false);
-    load_rows(v + ((long long)hd * L.n + t0) * dv, Vs, len, dv, C, W, true);
-    load_rows(dout + ((long long)hd * L.n + t0) * dv, Gs, len, dv, C, W, false);
-    const float *fc = rec(ws, L.o_fc, L.fc_len, L, hd, c);
-    __syncthreads();
-    chunk_forward(Qs, Ks, kd, fc + L.fc_S, Ws, Xs, Ts, C, d);
-    if (normalized) {
-        bgemm(Ns, W, Ts, C, 1, Vs, W, 1, C, W, C, false, 0, 1);   // num' = T V'
-        bgemm(Ns, W, Qs, d, 1, fc + L.fc_D, W, 1, C, W, d, true);  //   + Q D_p
-        __syncthreads();
-        // G' = [g / (den + eps) | -(g . o) / (den + eps)], o = num / (den + eps)
-        for (int r = threadIdx.x; r < C; r += blockDim.x) {
-            if (r >= len) continue;  // rows beyond the sequence keep their zero gradient
-            const float inv = 1.f / (Ns[r * W + dv] + eps);
-            float go = 0.f;
-            for (int j = 0; j < dv; ++j) {
-                const float g = Gs[r * W + j];
-                go += g * Ns[r * W + j] * inv;
-                Gs[r * W + j] = g * inv;
-            }
-            Gs[r * W + dv] = -go * inv;
-        }
-        __syncthreads();
-    }
-    float *bl = rec(ws, L.o_bl, L.bl_len, L, hd, c);
-    for (int i = threadIdx.x; i < C * W; i += blockDim.x) bl[L.bl_G + i] = Gs[i];
-    float *Ps = Ts;  // T is not needed any more: P = L . (G' V'^T)
-    bgemm(Ps, C, Gs, W, 1, Vs, 1, W, C, C, W, false, 1);
-    __syncthreads();
-    float *Ys = Ns;
-    bgemm(Ys, d, Ps, 1, C, Qs, d, 1, C, d, C, false, 0, 3);      // Y_loc = P^T Q (P(t, j) = 0 for t < j)
-    bgemm(bl + L.bl_Gam, d, Gs, 1, W, Qs, d, 1, W, d, C, false); // Gam_c = G'^T Q
-    bgemm(bl + L.bl_M, d, Vs, 1, W, Qs, d, 1, W, d, C, false);   // M_c = V'^T Q
-    __syncthreads();
-    // Lam_c = Y_loc^T Q + Q^T Y_loc
-    for (int idx = threadIdx.x; idx < d * d; idx += blockDim.x) {
-        const int a = idx / d, b = idx % d;
-        float s = 0.f;
-        for (int t = 0; t < C; ++t) s += Ys[t * d + a] * Qs[t * d + b] + Qs[t * d + a] * Ys[t * d + b];
-        bl[L.bl_Lam + idx] = s;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// B4: reverse scan.  Block (column block of Lam, head) keeps the whole Gam_s and 32
-// columns of Lam_s; from the last chunk back it records them, then
-// Lam_s += Lam_c + Gam_s^T M_c + M_c^T Gam_s (old Gam_s) and Gam_s += Gam_c.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) bwd_scan(float *ws, BLayout L) {
-    extern __shared__ float sm[];
-    const int hd = blockIdx.y, d = L.d, W = L.W, j0 = blockIdx.x * kCols, ncol = min(kCols, d - j0);
-    // Gam_s (W x d), Lam_s columns (d x 32), the chunk's M_c (W x d) staged per chunk
-    float *Gm = sm, *Lm = Gm + W * d, *Mc = Lm + d * kCols;
-    for (int i = threadIdx.x; i < W * d; i += blockDim.x) Gm[i] = 0.f;
-    for (int i = threadIdx.x; i < d * kCols; i += blockDim.x) Lm[i] = 0.f;
-    __syncthreads();
-    for (int c = L.nch - 1; c >= 0; --c) {
-        float *bc = rec(ws, L.o_bc, L.bc_len, L, hd, c);
-        const float *bl = rec(ws, L.o_bl, L.bl_len, L, hd, c);
-        if (blockIdx.x == 0) {
-            for (int i = threadIdx.x; i < W * d; i += blockDim.x) bc[L.bc_Gam + i] = Gm[i];
-            for (int i = threadIdx.x; i < W * d; i += blockDim.x) {  // Gam_s^T, consecutive threads on consecutive w
-                const int f = i / W, w = i % W;
-                bc[L.bc_GamT + i] = Gm[w * d + f];
-            }
-        }
-        for (int i = threadIdx.x; i < d * ncol; i += blockDim.x) {
-            const int a = i / ncol, j = i % ncol;
-            bc[L.bc_Lam + a * d + j0 + j] = Lm[a * kCols + j];
-        }
-        for (int i = threadIdx.x; i < W * d; i += blockDim.x) Mc[i] = bl[L.bl_M + i];
-        __syncthreads();
-        float ln[128 * kCols / kThreads];
-        int cnt = 0;
-        for (int i = threadIdx.x; i < d * kCols; i += blockDim.x, ++cnt) {
-            const int a = i / kCols, j = i % kCols, b = j0 + j;
-            float x = 0.f;
-            if (j < ncol) {
-                x = Lm[i] + bl[L.bl_Lam + a * d + b];
-                for (int w = 0; w < W; ++w) x += Gm[w * d + a] * Mc[w * d + b] + Mc[w * d + a] * Gm[w * d + b];
-            }
-            ln[cnt] = x;
-        }
-        __syncthreads();
-        cnt = 0;
-        for (int i = threadIdx.x; i < d * kCols; i += blockDim.x, ++cnt) Lm[i] = ln[cnt];
-        for (int i = threadIdx.x; i < W * d; i += blockDim.x) Gm[i] += bl[L.bl_Gam + i];
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
-// B5: per chunk gradients.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) bwd_local2(const T *q, const T *k, const T *v, T *dq, T *dk, T *dvo,
-                                                       float *ws, BLayout L) {
-    extern __shared__ float sm[];
-    const int c = blockIdx.x, hd = blockIdx.y, d = L.d, W = L.W, dv = L.dv, C = L.C, t0 = c * C;
-    const int len = min(C, L.n - t0), kd = d + 1;
-    float *Qs = sm, *Ks = Qs + C * d, *Vs = Ks + C * kd, *Gs = Vs + C * W, *Ws = Gs + C * W, *Xs = Ws + C * C;
-    float *Ts = Xs + C * d, *Ps = Ts + C * C, *Ys = Ps + C * C, *Bs = Ys + C * d, *Os = Bs + C * C;  // Os: C x max(d, W)
-    load_rows(q + ((long long)hd * L.n + t0) * d, Qs, len, d, C, d, false);
-    load_rows(k + ((long long)hd * L.n + t0) * d, Ks, len, d, C, kd, false);
-    load_rows(v + ((long long)hd * L.n + t0) * dv, Vs, len, dv, C, W, true);
-    const float *fc = rec(ws, L.o_fc, L.fc_len, L, hd, c), *bl = rec(ws, L.o_bl, L.bl_len, L, hd, c);
-    const float *bc = rec(ws, L.o_bc, L.bc_len, L, hd, c);
-    for (int i = threadIdx.x; i < C * W; i += blockDim.x) Gs[i] = bl[L.bl_G + i];
-    __syncthreads();
-    chunk_forward(Qs, Ks, kd, fc + L.fc_S, Ws, Xs, Ts, C, d);
-    bgemm(Ps, C, Gs, W, 1, Vs, 1, W, C, C, W, false, 1);          // P = L . G' V'^T
-    __syncthreads();
-    bgemm(Ys, d, Ps, 1, C, Qs, d, 1, C, d, C, false, 0, 3);       // Y = P^T Q
-    bgemm(Ys, d, Vs, W, 1, bc + L.bc_Gam, d, 1, C, d, W, true);   //   + V' Gam_s
-    __syncthreads();
-    bgemm(Bs, C, Ys, d, 1, Ks, 1, kd, C, C, d, false, 1);         // B = L . Y K^T
-    // dV' = T^T G' + X Gam_s^T   (columns < dv)
-    bgemm(Os, W, Ts, 1, C, Gs, W, 1, C, W, C, false, 0, 3);
-    bgemm(Os, W, Xs, d, 1, bc + L.bc_GamT, W, 1, C, W, d, true);
-    __syncthreads();
-    T *gv = dvo + ((long long)hd * L.n + t0) * dv;
-    for (int i = threadIdx.x; i < len * dv; i += blockDim.x) from_f32(&gv[i], Os[(i / dv) * W + i % dv]);
-    __syncthreads();
-    // dQ = P X + G' D_p^T + Y S_p + B K
-    bgemm(Os, d, Ps, C, 1, Xs, d, 1, C, d, C, false, 0, 1);
-    bgemm(Os, d, Gs, W, 1, fc + L.fc_DT, d, 1, C, d, W, true);
-    bgemm(Os, d, Ys, d, 1, fc + L.fc_S, d, 1, C, d, d, true);
-    bgemm(Os, d, Bs, C, 1, Ks, kd, 1, C, d, C, true, 0, 1);
-    __syncthreads();
-    T *gq = dq + ((long long)hd * L.n + t0) * d;
-    for (int i = threadIdx.x; i < len * d; i += blockDim.x) from_f32(&gq[i], Os[i]);
-    __syncthreads();
-    // dK = K Lam_s + W_c^T Y + B^T Q
-    bgemm(Os, d, Ks, kd, 1, bc + L.bc_Lam, d, 1, C, d, d, false);
-    bgemm(Os, d, Ws, 1, C, Ys, d, 1, C, d, C, true, 0, 3);
-    bgemm(Os, d, Bs, 1, C, Qs, d, 1, C, d, C, true, 0, 3);
-    __syncthreads();
-    T *gk = dk + ((long long)hd * L.n + t0) * d;
-    for (int i = threadIdx.x; i < len * d; i += blockDim.x) from_f32(&gk[i], Os[i]);
-}
-
-template <typename T>
-cudaError_t backward_t(const Bwd2 &p, cudaStream_t s) {
-    const BLayout L = make_layout(p.BH, p.n, p.d, p.dv, p.chunk);
-    if (L.nch == 0) return cudaSuccess;
+template <int N, typename T>
+cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
+    const BLayout L = make_layout(p.BH, p.n, p.d, p.dv);
     float *ws = reinterpret_cast<float *>(p.ws + kWsHeaderBytes);
-    const int C = L.C, d = L.d, W = L.W, kd = d + 1;
-    const T *q = static_cast<const T *>(p.q), *k = static_cast<const T *>(p.k), *v = static_cast<const T *>(p.v);
-    const T *g = static_cast<const T *>(p.dout);
-    const dim3 grid(L.nch, p.BH);
+    const int d = p.d, dv = p.dv, nch = L.nch;
+    if (nch == 0) return cudaSuccess;
+    BParams<T> P{};
+    P.q = static_cast<const T *>(p.q); P.k = static_cast<const T *>(p.k); P.v = static_cast<const T *>(p.v);
+    P.g = static_cast<const T *>(p.dout);
+    P.dq = static_cast<T *>(p.dq); P.dk = static_cast<T *>(p.dk); P.dv_out = static_cast<T *>(p.dval);
+    P.S = {ws + L.oS, d * d, nch};
+    P.D = {ws + L.oD, d * dv + d, nch};
+    P.Gam = {ws + L.oG, d * dv + (p.normalized ? d : 0), nch};
+    P.Lam = {ws + L.oL, d * d, nch};
+    P.X = ws + L.oX; P.Y = ws + L.oY; P.num = ws + L.oNum; P.den = ws + L.oDen;
+    P.n = p.n; P.d = d; P.dv = dv; P.normalized = p.normalized; P.eps = p.eps;
+    const dim3 grid(nch, p.BH);
+    const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
     cudaError_t e;
-    auto smem = [](size_t floats) { return (int)(floats * sizeof(float)); };
-    const int sm1 = smem((size_t)C * d + (size_t)C * kd + (size_t)C * W + (size_t)C * C + (size_t)C * d);
-    if ((e = cudaFuncSetAttribute(bwd_fwd_local<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1))) return e;
-    bwd_fwd_local<T><<<grid, kThreads, sm1, s>>>(q, k, v, ws, L);
-    if ((e = cudaGetLastError())) return e;
-    const int sm2 = smem((size_t)d * d + 3 * (size_t)d * kCols);
-    if ((e = cudaFuncSetAttribute(bwd_fwd_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2))) return e;
-    bwd_fwd_scan<<<dim3((W + kCols - 1) / kCols, p.BH), kThreads, sm2, s>>>(ws, L);
-    if ((e = cudaGetLastError())) return e;
-    const int sm3 = smem((size_t)C * d + (size_t)C * kd + 2 * (size_t)C * W + 2 * (size_t)C * C + (size_t)C * d +
-                         (size_t)C * std::max(W, d));
-    if ((e = cudaFuncSetAttribute(bwd_local1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm3))) return e;
-    bwd_local1<T><<<grid, kThreads, sm3, s>>>(q, k, v, g, ws, L, p.normalized, p.eps);
-    if ((e = cudaGetLastError())) return e;
-    const int sm4 = smem(2 * (size_t)W * d + (size_t)d * kCols);
-    if ((e = cudaFuncSetAttribute(bwd_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, sm4))) return e;
-    bwd_scan<<<dim3((d + kCols - 1) / kCols, p.BH), kThreads, sm4, s>>>(ws, L);
-    if ((e = cudaGetLastError())) return e;
-    const int sm5 = smem((size_t)C * d + (size_t)C * kd + 2 * (size_t)C * W + 4 * (size_t)C * C + 2 * (size_t)C * d +
-                         (size_t)C * std::max(W, d));
-    if ((e = cudaFuncSetAttribute(bwd_local2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm5))) return e;
-    bwd_local2<T><<<grid, kThreads, sm5, s>>>(q, k, v, static_cast<T *>(p.dq), static_cast<T *>(p.dk),
-                                               static_cast<T *>(p.dval), ws, L);
-    return cudaGetLastError();
+    auto launch = [&](auto kern, dim3 gr) -> cudaError_t {
+        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (err) return err;
+        kern<<<gr, kCT, smem, s>>>(P);
+        return cudaGetLastError();
+    };
+    const bool many = nch > 1;
+    const ScanJob none{};
+    auto scan = [&](const Records &a, int rev_a, const Records *b) -> cudaError_t {
+        ScanJobs jobs{};
+        jobs.j[0] = none; jobs.j[0].r = a; jobs.j[0].reverse = rev_a;
+        if (b) { jobs.j[1].r = *b; jobs.j[1].reverse = 1; }
+        return launch_scan(jobs, b ? 2 : 1, p.BH, s);
+    };
+    if (many) {
+        SumJobs<T> jobs{};
+        jobs.j[0] = {P.k, P.k, P.S, d, d, 0};
+        jobs.j[1] = {P.q, P.g, P.Gam, d, dv, 0};  // Gam^T of the plain output
+        if ((e = launch_sums<N, T>(jobs, p.normalized ? 1 : 2, p.BH, p.n, s))) return e;
+        if ((e = scan(P.S, 0, p.normalized ? nullptr : &P.Gam))) return e;
+    }
+    if ((e = launch(bwd_x_kernel<N, T>, grid))) return e;
+    if (many && (e = scan(P.D, 0, nullptr))) return e;
+    if (p.normalized) {
+        if ((e = launch(bwd_upstream_kernel<N, T>, grid))) return e;
+        if (many && (e = scan(P.Gam, 1, nullptr))) return e;
+    }
+    if ((e = launch(bwd_y_kernel<N, T>, grid))) return e;
+    if (many && (e = scan(P.Lam, 1, nullptr))) return e;
+    return launch(bwd_grad_kernel<N, T>, dim3(nch, p.BH, 3));
 }
 
 }  // namespace
 
-size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int chunk) {
-    const BLayout L = make_layout(BH, n, d, dv, chunk);
-    const size_t simt = kWsHeaderBytes + sizeof(float) * (size_t)L.total, tc = backward2_tc_workspace_bytes(BH, n);
+size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int) {
+    const size_t simt = kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
+    const size_t tc = backward2_tc_workspace_bytes(BH, n);
     return simt > tc ? simt : tc;
 }
 
 cudaError_t backward2_launch(const Bwd2 &p, cudaStream_t stream) {
     if (backward2_tc_applicable(p)) return backward2_tc_launch(p, stream);
-    return p.dt == HLA_BF16 ? backward_t<__nv_bfloat16>(p, stream) : backward_t<float>(p, stream);
+    return with_padded_size(p.d, p.dv, [&](auto size) {
+        constexpr int N = decltype(size)::value;
+        return p.dt == HLA_BF16 ? backward_n<N, __nv_bfloat16>(p, stream) : backward_n<N, float>(p, stream);
+    });
 }
 
 }  // namespace hla

@@ -92,3 +92,20 @@ def test_ahla(hla, n, d, dv):
     ref, rst = oracle.ahla_serial(_flat(q), _flat(k), _flat(v), state_in=st0, return_state=True)
     assert rowerr(_flat(cont.cpu().numpy()), ref) < TOL["f32"]
     assert np.abs(st.reshape(B * H, -1).cpu().numpy() - rst).max() <= 2e-5 * np.abs(rst).max()
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+@pytest.mark.parametrize("d,dv", SIZES)
+@pytest.mark.parametrize("normalized", [False, True])
+def test_backward(hla, n, d, dv, normalized):
+    """Gradients; the normalised output with eps such that den + eps >= 1 on every row."""
+    B, H = 1, 2
+    q, k, v = hla_inputs.make_qkv(B, H, n, d, dv, seed=n, dtype="f32")
+    g = hla_inputs.round_to(np.random.default_rng(n).standard_normal((B, H, n, dv)), "f32")
+    den = oracle.hla2_serial(_flat(q), _flat(k), _flat(v), return_den=True)[1]
+    eps = 1.0 + max(0.0, -float(den.min()))
+    got = hla.hla2_backward(*_gpu(q, k, v, g), normalized=normalized, eps=eps)
+    torch.cuda.synchronize()
+    ref = oracle.hla2_backward(_flat(q), _flat(k), _flat(v), _flat(g), normalized=normalized, eps=eps, nthreads=8)
+    for name, a, b in zip(("dq", "dk", "dv"), got, ref):
+        assert rowerr(_flat(a.cpu().numpy()), b) < TOL["f32"], name

@@ -252,10 +252,10 @@ __device__ __forceinline__ void nn_carry(Acc<N> &acc, const Tile<N> &t, const fl
                 if (tc < width) v = *reinterpret_cast<const float4 *>(R + (long long)tc * ldr + s * kSlice + tk + 4 * i);
                 buf[4 * i] = v.x; buf[4 * i + 1] = v.y; buf[4 * i + 2] = v.z; buf[4 * i + 3] = v.w;
             }
-            if constexpr (U == kSymmetric)
-                if (tc < width)
+            if (U == kSymmetric && tc < width) {
 #pragma unroll
-                    for (int i = 0; i < PT; ++i) buf[i] += R[(long long)(s * kSlice + tk + i) * ldr + tc];
+                for (int i = 0; i < PT; ++i) buf[i] += R[(long long)(s * kSlice + tk + i) * ldr + tc];
+            }
         }
     };
     auto put = [&](float *b) {

@@ -65,6 +65,7 @@
 
 #include "hla_internal.h"
 #include "sm103_prims.cuh"
+#include "state_products.cuh"
 
 namespace hla {
 namespace {
@@ -1039,25 +1040,16 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     }
 }
 
-// initial-state carries D_0 = S_0 C_0 - G_0 and e_0 = S_0 m_0 - h_0 of each head (fp32)
-__global__ void __launch_bounds__(256) init_carry_kernel(const float *__restrict__ st, float *__restrict__ out) {
-    const int hd = blockIdx.x;
-    const size_t L = kStateFloats;
-    const float *S = st + hd * L, *C = S + kD * kD, *m = C + kD * kD, *G = m + kD, *h = G + kD * kD;
-    float *D = out + (size_t)hd * (kD * kD + kD), *e = D + kD * kD;
-    for (int idx = threadIdx.x; idx < kD * kD + kD; idx += blockDim.x) {
-        if (idx < kD * kD) {
-            const int a = idx / kD, b = idx % kD;
-            float s = 0.f;
-            for (int j = 0; j < kD; ++j) s += S[a * kD + j] * C[j * kD + b];
-            D[idx] = s - G[idx];
-        } else {
-            const int a = idx - kD * kD;
-            float s = 0.f;
-            for (int j = 0; j < kD; ++j) s += S[a * kD + j] * m[j];
-            e[a] = s - h[a];
-        }
-    }
+// initial-state carries D_0 = S_0 C_0 - G_0 and e_0 = S_0 m_0 - h_0 of each head (fp32); block (16 rows, head)
+__global__ void __launch_bounds__(kStateThreads) init_carry_kernel(const float *__restrict__ st, float *__restrict__ out) {
+    __shared__ __align__(16) float rows[kStateRows * kD];
+    const float *S = st + (size_t)blockIdx.y * kStateFloats, *C = S + kD * kD, *m = C + kD * kD, *G = m + kD;
+    const float *h = G + kD * kD;
+    float *D = out + (size_t)blockIdx.y * (kD * kD + kD), *e = D + kD * kD;
+    state_products(S, C, m, kD, kD, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+        if (b < kD) D[a * kD + b] = x - G[a * kD + b];
+        else e[a] = x - h[a];
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1171,13 +1163,17 @@ int segment_tiles(int BH, int M, int sms) {
 constexpr int kCThreads = 160;            // 4 warps read TMEM (one lane quadrant each), warp 4 issues
 constexpr uint32_t kCOnesBytes = 4096;    // 16 x 128 bf16 ones operand (row 0 ones), K-major
 constexpr uint32_t kCSmemBytes = 4 * kTileBytes + kCOnesBytes + 1024;
-constexpr int kCPartFloats = kD * kD + kD;  // C (d x dv) then m (d) of one group of tiles
+// C of one group of tiles, column by column (so that a warp, which reads 32 rows of a column from
+// TMEM, stores 128 contiguous bytes; row by row it stored 32 lines a time and the kernel took 31 us at
+// 32 heads of 2000 tokens), then m
+constexpr int kCPartFloats = kD * kD + kD;
 
 // C and m of tiles [g * tiles_per, ...) of a head, from tiles of 128 tokens (Q^T V: A = Q^T and
-// B = V both MN-major; m: B = a 16-row K-major operand whose row 0 is ones)
+// B = V both MN-major; m: B = a 16-row K-major operand whose row 0 is ones).  The first group of a
+// head adds C_0, m_0 of state_in, which the launch after this may overwrite.
 __global__ void __launch_bounds__(kCThreads, 1)
 state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_v, float *part,
-               int M, int groups, int tiles_per, WsHeader *err) {
+               int M, int groups, int tiles_per, const float *state_in, WsHeader *err) {
     extern __shared__ __align__(1024) uint8_t csm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int head = blockIdx.x / groups, g = blockIdx.x % groups;
@@ -1255,8 +1251,9 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         __syncwarp();
     } else {
-        // C rows (features f = 32 warp + lane), 128 columns, then m
+        // C rows (features f = 32 warp + lane), 128 columns, then m (an initial state is 128 x 128)
         float *out = part + (size_t)blockIdx.x * kCPartFloats;
+        const float *C0 = state_in && g == 0 ? state_in + (size_t)head * kStateFloats + kD * kD : nullptr;
         const uint32_t lb = (uint32_t)(32 * warp) << 16;
         const int f = 32 * warp + lane;
         const bool ok = (j0 < j1) && cwait(4, 0);
@@ -1264,11 +1261,18 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         for (int c0 = 0; c0 < kD; c0 += 32) {
             float v[32];
             if (ok) ld32(tb + lb + c0, v);
-            for (int jj = 0; jj < 32; ++jj) out[(size_t)f * kD + c0 + jj] = ok ? v[jj] : 0.f;
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 4) {
+                const float4 x = C0 ? *reinterpret_cast<const float4 *>(C0 + f * kD + c0 + jj) : make_float4(0.f, 0.f, 0.f, 0.f);
+                out[(c0 + jj) * kD + f] = (ok ? v[jj] : 0.f) + x.x;
+                out[(c0 + jj + 1) * kD + f] = (ok ? v[jj + 1] : 0.f) + x.y;
+                out[(c0 + jj + 2) * kD + f] = (ok ? v[jj + 2] : 0.f) + x.z;
+                out[(c0 + jj + 3) * kD + f] = (ok ? v[jj + 3] : 0.f) + x.w;
+            }
         }
         float mv[32];
         if (ok) ld32(tb + lb + 128, mv);
-        out[kD * kD + f] = ok ? mv[0] : 0.f;
+        out[kD * kD + f] = (ok ? mv[0] : 0.f) + (C0 ? C0[kD * kD + f] : 0.f);
     }
     tc_fence_before();
     __syncthreads();
@@ -1278,61 +1282,83 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
 }
 
-// per head: the paper tuple [S | C | m | G | h] (d x d, d x dv, d, d x dv, d) from the ring slot of
-// the head's last segment and the C / m partials; state_in (may alias state_out) supplies C_0, m_0
+// The paper tuple [S | C | m | G | h] (d x d, d x dv, d, d x dv, d) from the ring slot of the head's
+// last segment and the C / m partials.  Block (16 columns of C and G, head): with one block a head the
+// d^2 dv products of S C ran on 32 SMs and took 199 us at 32 heads, 128 x 128; on 8 blocks a head,
+// each thread with 8 columns of a row of S read in the ring's own order, they take 18 us (both from cold caches).
+constexpr int kFinCols = 16;
 __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, int last_slot, const float *part,
-                                                             int groups, const float *state_in, float *state_out,
-                                                             int d, int dv) {
-    extern __shared__ float fs[];
-    float *S = fs, *C = S + kD * kD, *m = C + kD * kD;  // 128 x 128, 128 x 128, 128 (zero outside d, dv)
-    const int hd = blockIdx.x, tid = threadIdx.x;
+                                                             int groups, float *state_out, int d, int dv) {
+    __shared__ __align__(16) float C[kD][kFinCols + 4];  // the block's columns (zero outside d)
+    __shared__ float m[kD];
+    const int hd = blockIdx.y, cb = blockIdx.x * kFinCols, tid = threadIdx.x;
     const float *rg = ring + ((size_t)hd * 2 + last_slot) * kRingFloats;
-    const size_t st_len = (size_t)d * d + 2 * (size_t)d * dv + 2 * (size_t)d;
-    const float *sin = state_in ? state_in + (size_t)hd * st_len : nullptr;
+    const float *pt = part + (size_t)hd * groups * kCPartFloats;
     // the ring stores float4 c (columns c0 + 4c..) of epilogue thread et = 32 (qd + 4 cq) + lane at c * 512 + et
-    auto ring_at = [&](const float *base, int r, int col) {
+    auto ring4 = [&](const float *base, int r, int col) {
         const int et = 32 * ((r >> 5) + 4 * (col >> 5)) + (r & 31);
-        return base[(size_t)(((col & 31) >> 2) * kEpiThreads + et) * 4 + (col & 3)];
+        return *reinterpret_cast<const float4 *>(base + (size_t)(((col & 31) >> 2) * kEpiThreads + et) * 4);
     };
-    for (int i = tid; i < kD * kD; i += blockDim.x) {
-        const int r = i / kD, c = i % kD;
-        S[i] = ring_at(rg, r, c);
-        float cv = 0.f;
-        if (r < d && c < dv) {
-            for (int g = 0; g < groups; ++g) cv += part[((size_t)hd * groups + g) * kCPartFloats + (size_t)r * kD + c];
-            if (sin) cv += sin[(size_t)d * d + (size_t)r * dv + c];
+    for (int i = tid; i < kD * kFinCols; i += 256) {
+        const int c = i / kD, x = i % kD;
+        float s = 0.f;
+        if (x < d)
+            for (int g = 0; g < groups; ++g) s += pt[(size_t)g * kCPartFloats + (cb + c) * kD + x];
+        C[x][c] = s;
+    }
+    if (tid < kD) {
+        float s = 0.f;
+        if (tid < d)
+            for (int g = 0; g < groups; ++g) s += pt[(size_t)g * kCPartFloats + kD * kD + tid];
+        m[tid] = s;
+    }
+    __syncthreads();
+    const size_t st_len = (size_t)d * d + 2 * (size_t)d * dv + 2 * (size_t)d;
+    float *oS = state_out + (size_t)hd * st_len, *oC = oS + (size_t)d * d, *om = oC + (size_t)d * dv, *oG = om + d;
+    float *oh = oG + (size_t)d * dv;
+    const int nb = dv / kFinCols, rows = (d + nb - 1) / nb, s0 = blockIdx.x * rows;  // this block's rows of S
+    for (int i = tid; i < rows * (d / 4); i += 256) {
+        const int r = s0 + i / (d / 4), x = (i % (d / 4)) * 4;
+        if (r < d) *reinterpret_cast<float4 *>(oS + (size_t)r * d + x) = ring4(rg, r, x);
+    }
+    for (int i = tid; i < d * (kFinCols / 4); i += 256) {
+        const int x = i / (kFinCols / 4), c = (i % (kFinCols / 4)) * 4;
+        *reinterpret_cast<float4 *>(oC + (size_t)x * dv + cb + c) = *reinterpret_cast<const float4 *>(&C[x][c]);
+    }
+    const int r = tid & (kD - 1), h = (tid >> 7) * 8;  // row r of S, columns h .. h + 7 of the block
+    if (r < d) {
+        float acc[8], sm_ = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+#pragma unroll 8
+        for (int x = 0; x < d; x += 4) {
+            const float4 sv = ring4(rg, r, x);
+            const float s4[4] = {sv.x, sv.y, sv.z, sv.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 a = *reinterpret_cast<const float4 *>(&C[x + u][h]);
+                const float4 b = *reinterpret_cast<const float4 *>(&C[x + u][h + 4]);
+                acc[0] += s4[u] * a.x; acc[1] += s4[u] * a.y; acc[2] += s4[u] * a.z; acc[3] += s4[u] * a.w;
+                acc[4] += s4[u] * b.x; acc[5] += s4[u] * b.y; acc[6] += s4[u] * b.z; acc[7] += s4[u] * b.w;
+                sm_ += s4[u] * m[x + u];
+            }
         }
-        C[i] = cv;
-    }
-    for (int r = tid; r < kD; r += blockDim.x) {
-        float mv = 0.f;
-        if (r < d) {
-            for (int g = 0; g < groups; ++g) mv += part[((size_t)hd * groups + g) * kCPartFloats + kD * kD + r];
-            if (sin) mv += sin[(size_t)d * d + (size_t)d * dv + r];
+#pragma unroll
+        for (int j = 0; j < 8; j += 4) {  // G = S C - D
+            const float4 D = ring4(rg + kD * kD, r, cb + h + j);
+            *reinterpret_cast<float4 *>(oG + (size_t)r * dv + cb + h + j) =
+                make_float4(acc[j] - D.x, acc[j + 1] - D.y, acc[j + 2] - D.z, acc[j + 3] - D.w);
         }
-        m[r] = mv;
-    }
-    __syncthreads();  // everything read from state_in before state_out (possibly the same memory) is written
-    float *so = state_out + (size_t)hd * st_len;
-    float *oS = so, *oC = oS + (size_t)d * d, *om = oC + (size_t)d * dv, *oG = om + d, *oh = oG + (size_t)d * dv;
-    for (int i = tid; i < d * d; i += blockDim.x) oS[i] = S[(i / d) * kD + i % d];
-    for (int i = tid; i < d * dv; i += blockDim.x) {
-        const int r = i / dv, c = i % dv;
-        float sc = 0.f;
-        for (int x = 0; x < d; ++x) sc += S[r * kD + x] * C[x * kD + c];
-        oC[i] = C[r * kD + c];
-        oG[i] = sc - ring_at(rg + kD * kD, r, c);  // G = S C - D
-    }
-    for (int r = tid; r < d; r += blockDim.x) {
-        float sm_ = 0.f;
-        for (int x = 0; x < d; ++x) sm_ += S[r * kD + x] * m[x];
-        om[r] = m[r];
-        oh[r] = sm_ - rg[2 * kD * kD + r];  // h = S m - e
+        if (blockIdx.x == 0 && h == 0) {
+            om[r] = m[r];
+            oh[r] = sm_ - rg[2 * kD * kD + r];  // h = S m - e
+        }
     }
 }
 
+// groups of tiles per head of state_c_kernel: one wave of one block an SM (152), at most 8 partials to add
 int state_groups(int BH, int M) {
-    int g = 256 / (BH > 0 ? BH : 1);
+    int g = 152 / (BH > 0 ? BH : 1);
     if (g < 1) g = 1;
     if (g > 8) g = 8;
     return g < M ? g : M;
@@ -1403,7 +1429,7 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     if ((e = cudaMemsetAsync(p.ws + FL.off_ticket, 0, FL.off_ring - FL.off_ticket, stream))) return e;
     if (p.state_in) {
         float *init = reinterpret_cast<float *>(p.ws + FL.off_init);
-        init_carry_kernel<<<p.BH, 256, 0, stream>>>(p.state_in, init);
+        init_carry_kernel<<<dim3(kD / kStateRows, p.BH), kStateThreads, 0, stream>>>(p.state_in, init);
         if ((e = cudaGetLastError())) return e;
         kp.init_De = init;
     }
@@ -1430,13 +1456,11 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     float *part = reinterpret_cast<float *>(p.ws + FL.off_part);
     if ((e = cudaFuncSetAttribute(state_c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCSmemBytes)))
         return e;
-    state_c_kernel<<<p.BH * groups, kCThreads, kCSmemBytes, stream>>>(mq, mv, part, kp.M, groups, tiles_per, kp.err);
+    state_c_kernel<<<p.BH * groups, kCThreads, kCSmemBytes, stream>>>(mq, mv, part, kp.M, groups, tiles_per,
+                                                                       p.state_in, kp.err);
     if ((e = cudaGetLastError())) return e;
-    const int fin_smem = (int)(sizeof(float) * (2 * kD * kD + kD));
-    if ((e = cudaFuncSetAttribute(state_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fin_smem)))
-        return e;
-    state_finalize_kernel<<<p.BH, 256, fin_smem, stream>>>(kp.ring, (kp.G - 1) & 1, part, groups, p.state_in,
-                                                            p.state_out, p.d, p.dv);
+    state_finalize_kernel<<<dim3(p.dv / kFinCols, p.BH), 256, 0, stream>>>(kp.ring, (kp.G - 1) & 1, part, groups,
+                                                                            p.state_out, p.d, p.dv);
     return cudaGetLastError();
 }
 

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "chunk_simt.cuh"
+#include "state_products.cuh"
 
 namespace hla {
 namespace {
@@ -66,56 +67,37 @@ struct GParams {
     int need_D;   // D's increments of the last chunk are wanted too (final state)
 };
 
+// D_0 = S_0 C_0 - G_0, e_0 = S_0 m_0 - h_0 of a head's state_in into D's initial record; block (16 rows, head)
 // ---------------------------------------------------------------------------
-// D_0 = S_0 C_0 - G_0, e_0 = S_0 m_0 - h_0 of a head's state_in into D's initial record; block (rows
-// of 16, head)
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) g2_init_kernel(const float *__restrict__ st, Records D, int d, int dv) {
-    const int hd = blockIdx.y, a0 = blockIdx.x * 16;
-    const float *S = st + hd * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
+__global__ void __launch_bounds__(kStateThreads) g2_init_kernel(const float *__restrict__ st, Records D, int d, int dv) {
+    __shared__ __align__(16) float rows[kStateRows * 128];
+    const float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     const float *G = m + d, *h = G + d * dv;
-    float *out = D.at(hd, D.nch);
-    for (int i = threadIdx.x; i < 16 * dv; i += blockDim.x) {
-        const int a = a0 + i / dv, b = i % dv;
-        float s = 0.f;
-#pragma unroll 8
-        for (int j = 0; j < d; ++j) s = fmaf(S[a * d + j], C[j * dv + b], s);
-        out[a * dv + b] = s - G[a * dv + b];
-    }
-    if (threadIdx.x < 16) {
-        const int a = a0 + threadIdx.x;
-        float s = 0.f;
-        for (int j = 0; j < d; ++j) s = fmaf(S[a * d + j], m[j], s);
-        out[d * dv + a] = s - h[a];
-    }
+    float *out = D.at(blockIdx.y, D.nch);
+    state_products(S, C, m, d, dv, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+        if (b < dv) out[a * dv + b] = x - G[a * dv + b];
+        else out[d * dv + a] = x - h[a];
+    });
 }
 
 // state_out's G = S C - D, h = S m - e (zeros for the unmasked operator) from its S, C, m and D's
-// total; block (rows of 16, head)
-__global__ void __launch_bounds__(128) g2_final_kernel(float *__restrict__ st, Records D, int d, int dv, int masked) {
-    const int hd = blockIdx.y, a0 = blockIdx.x * 16;
-    float *S = st + hd * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
+// total; block (16 rows, head)
+__global__ void __launch_bounds__(kStateThreads) g2_final_kernel(float *__restrict__ st, Records D, int d, int dv,
+                                                                 int masked) {
+    __shared__ __align__(16) float rows[kStateRows * 128];
+    float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     float *G = m + d, *h = G + d * dv;
-    const float *tot = D.at(hd, D.nch);
-    for (int i = threadIdx.x; i < 16 * dv; i += blockDim.x) {
-        const int a = a0 + i / dv, b = i % dv;
-        float s = 0.f;
-        if (masked) {
-#pragma unroll 8
-            for (int j = 0; j < d; ++j) s = fmaf(S[a * d + j], C[j * dv + b], s);
-            s -= tot[a * dv + b];
-        }
-        G[a * dv + b] = s;
+    const float *tot = D.at(blockIdx.y, D.nch);
+    if (!masked) {
+        const int a0 = blockIdx.x * kStateRows;
+        for (int i = threadIdx.x; i < kStateRows * dv; i += kStateThreads) G[a0 * dv + i] = 0.f;
+        if (threadIdx.x < kStateRows) h[a0 + threadIdx.x] = 0.f;
+        return;
     }
-    if (threadIdx.x < 16) {
-        const int a = a0 + threadIdx.x;
-        float s = 0.f;
-        if (masked) {
-            for (int j = 0; j < d; ++j) s = fmaf(S[a * d + j], m[j], s);
-            s -= tot[d * dv + a];
-        }
-        h[a] = s;
-    }
+    state_products(S, C, m, d, dv, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+        if (b < dv) G[a * dv + b] = x - tot[a * dv + b];
+        else h[a] = x - tot[d * dv + a];
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -199,7 +181,7 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
     P.direct = nch == 1 && !p.state_in;
     // D's initial value; the states' S and [C | m] start S's and C's sums as they lie
     if (p.state_in && p.masked) {
-        g2_init_kernel<<<dim3(d / 16, L.BH), 128, 0, s>>>(p.state_in, P.D, d, dv);
+        g2_init_kernel<<<dim3(d / kStateRows, L.BH), kStateThreads, 0, s>>>(p.state_in, P.D, d, dv);
         if ((e = cudaGetLastError())) return e;
     }
     const bool sums = nch > 1 || p.state_in || p.state_out, sums_C = !p.masked || p.state_out;
@@ -236,7 +218,7 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
         }
     }
     if (p.state_out) {
-        g2_final_kernel<<<dim3(d / 16, L.BH), 128, 0, s>>>(p.state_out, P.D, d, dv, p.masked);
+        g2_final_kernel<<<dim3(d / kStateRows, L.BH), kStateThreads, 0, s>>>(p.state_out, P.D, d, dv, p.masked);
         if ((e = cudaGetLastError())) return e;
     }
     return cudaSuccess;

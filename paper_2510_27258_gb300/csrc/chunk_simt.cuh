@@ -11,6 +11,10 @@
 // one address (the row operand) or 128 contiguous bytes (the column operand), so no load has a bank
 // conflict.  Rows of a thread are 4 rg .. 4 rg + 3 and 32 + 4 rg .. + 3: of a lower triangular
 // operand the upper right quadrant is then skipped by all warps alike.
+// Multiply-adds go two to an instruction (fma.rn.f32x2): with one each, the schedulers issued on 56 to
+// 68 % of the cycles and stalled on dispatch while the fp32 pipe was half idle.  In pairs: the backward
+// of B2 H16 n4096 d128 2331 -> 2087 us, AHLA B1 H32 n1999 d128 with states 404 -> 338 us, the forward of
+// B2 H16 n1000 d64 fp32 97 -> 84 us.
 #pragma once
 
 #include <type_traits>

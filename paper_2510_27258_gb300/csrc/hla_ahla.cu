@@ -19,6 +19,7 @@
 
 #include "chunk_simt.cuh"
 #include "sm103_prims.cuh"
+#include "step_split.cuh"
 
 namespace hla {
 namespace {
@@ -308,6 +309,142 @@ ahla_step_staged_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
     }
 }
 
+// The step with every load issued at once, straight to registers, by `split` blocks per head, block r
+// with columns [r dv / split, ...) of P and E.  From the old values, r = q^T P + (q.k) v and
+// o = q^T E + (q.k) r, column by column, so one pass does the step: both column sums, then both updated
+// slices.  Only m and n are shared.  The plain output needs them in block 0 alone; for the normalised
+// output the blocks of a head form a cluster and meet in a split barrier between their last read of m, n
+// and block 0's write.  Measured, us a step (staged -> this), bf16 tokens: 64 x 64, 16 heads 3.7 -> 2.8,
+// 256 heads 6.1 -> 4.0, 2048 heads 35.6 -> 23.4 (140 MB read and written: 5.9 TB/s); 128 x 128, 32
+// heads 5.7 -> 3.3, 2048 heads 87.7 -> 81.4.  Bound by the latency of one load and two barriers for few
+// heads, by HBM for many.
+constexpr int kSplitThreads = 256, kSplitWarps = kSplitThreads / 32;
+template <typename T, int NC>
+__global__ void __launch_bounds__(kSplitThreads)
+ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
+                       float *state, int split, int d, int dv, int normalized, float eps) {
+    __shared__ __align__(16) float qs[128], ks[128], vs[128];
+    __shared__ __align__(16) float part[2][kSplitWarps][64];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int hd = blockIdx.x / split, rank = blockIdx.x % split, cw = dv / split, col0 = rank * cw;
+    const long long len = (long long)d * dv + d;
+    float *P = state + hd * 2 * len, *m = P + (long long)d * dv, *E = P + len, *nn = E + (long long)d * dv;
+    const int wC = cw >> 2, nC = d * wC, c4 = (tid % wC) * 4, r0 = tid / wC, rstep = kSplitThreads / wC;
+    float4 pv[NC], ev[NC];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const long long at = (long long)(r0 + i * rstep) * dv + col0 + c4;
+        pv[i] = ev[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid + i * kSplitThreads < nC) {
+            pv[i] = *reinterpret_cast<const float4 *>(P + at);
+            ev[i] = *reinterpret_cast<const float4 *>(E + at);
+        }
+    }
+    const bool sums = normalized || rank == 0;  // m and n: four values a lane, in every warp
+    float mv[4], nv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = lane + 32 * i;
+        mv[i] = sums && a < d ? m[a] : 0.f;
+        nv[i] = sums && a < d ? nn[a] : 0.f;
+    }
+    if (tid < d) {
+        qs[tid] = to_f32(q[(long long)hd * d + tid]);
+        ks[tid] = to_f32(k[(long long)hd * d + tid]);
+    }
+    if (tid < dv) vs[tid] = to_f32(v[(long long)hd * dv + tid]);
+    __syncthreads();
+    const float qk = warp_dot(qs, ks, d);
+    float qm = 0.f, qn = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = lane + 32 * i;
+        if (a < d) {
+            qm = fmaf(qs[a], mv[i], qm);
+            qn = fmaf(qs[a], nv[i], qn);
+        }
+    }
+    const float s = group_sum<32>(qm) + qk;        // q . m'
+    const float den = group_sum<32>(qn) + s * qk;  // q . n'
+    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const float qr = qs[min(r0 + i * rstep, d - 1)];  // beyond the slice the values are zero
+        fma4(a0, qr, pv[i]);
+        fma4(a1, qr, ev[i]);
+    }
+    a0 = column_sum(a0, wC);
+    a1 = column_sum(a1, wC);
+    if (lane < wC) {
+        *reinterpret_cast<float4 *>(&part[0][wid][c4]) = a0;
+        *reinterpret_cast<float4 *>(&part[1][wid][c4]) = a1;
+    }
+    cluster_arrive();  // this block has read m, n
+    __syncthreads();
+    const float4 v4 = *reinterpret_cast<const float4 *>(vs + col0 + c4);
+    float4 r4 = make_float4(qk * v4.x, qk * v4.y, qk * v4.z, qk * v4.w);
+#pragma unroll
+    for (int w = 0; w < kSplitWarps; ++w) fma4(r4, 1.f, *reinterpret_cast<const float4 *>(&part[0][w][c4]));
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const int row = r0 + i * rstep;
+        const long long at = (long long)row * dv + col0 + c4;
+        if (tid + i * kSplitThreads < nC) {
+            *reinterpret_cast<float4 *>(P + at) = axpy4(pv[i], ks[row], v4);
+            *reinterpret_cast<float4 *>(E + at) = axpy4(ev[i], ks[row], r4);
+        }
+    }
+    if (tid < wC) {
+        float4 o = make_float4(qk * r4.x, qk * r4.y, qk * r4.z, qk * r4.w);
+#pragma unroll
+        for (int w = 0; w < kSplitWarps; ++w) fma4(o, 1.f, *reinterpret_cast<const float4 *>(&part[1][w][c4]));
+        const float x[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            from_f32(&out[(long long)hd * dv + col0 + c4 + j], normalized ? x[j] / (den + eps) : x[j]);
+    }
+    cluster_wait();  // every block of the head has read m, n
+    if (rank == 0 && wid == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int a = lane + 32 * i;
+            if (a >= d) continue;
+            m[a] = mv[i] + ks[a];
+            nn[a] = nv[i] + s * ks[a];
+        }
+    }
+}
+
+// Blocks per head of the kernel above, 0 where the staged kernel serves.  Head sizes up to 64: two for
+// few heads (16 heads 3.1 -> 2.8 us), one from 128 heads (3.2 against 3.3).  With a size of 128: four
+// up to 64 heads, then two where the staged kernel's last round is nearly full or there are many rounds;
+// between 200 and 600 heads the staged kernel, whose copies of the next head run during this one, is as
+// fast or faster (256 heads: 12.6 against 14.0 us).  Clusters cost more to launch: the normalised output
+// takes them up to 64 heads.  A block's slice has 8 to 64 columns.
+int ahla_step_split(int BH, int d, int dv, int normalized) {
+    int s;
+    if (d == 128 || dv == 128) s = BH <= 64 ? 4 : !normalized && (BH <= 200 || BH >= 600) ? 2 : 0;
+    else s = BH <= 64 ? 2 : 1;
+    if (s == 0) return 0;
+    while (s > 1 && dv / s < 8) s /= 2;
+    while (dv / s > 64) s *= 2;
+    return s;
+}
+
+template <typename T>
+cudaError_t ahla_step_split_launch(const void *q, const void *k, const void *v, void *out, float *state, int BH,
+                                   int split, int d, int dv, int normalized, float eps, cudaStream_t s) {
+    auto go = [&](auto kern) {
+        return launch_blocks(kern, BH, split, normalized != 0, kSplitThreads, s, static_cast<const T *>(q), static_cast<const T *>(k),
+                            static_cast<const T *>(v), static_cast<T *>(out), state, split, d, dv, normalized, eps);
+    };
+    const int nc = (d * (dv / split) / 4 + kSplitThreads - 1) / kSplitThreads;
+    if (nc <= 1) return go(ahla_step_split_kernel<T, 1>);
+    if (nc <= 2) return go(ahla_step_split_kernel<T, 2>);
+    if (nc <= 4) return go(ahla_step_split_kernel<T, 4>);
+    return go(ahla_step_split_kernel<T, 8>);
+}
+
 }  // namespace
 
 size_t ahla_workspace_bytes_internal(int BH, int n, int d, int dv, int) {
@@ -331,6 +468,10 @@ cudaError_t ahla_step_launch(const void *q, const void *k, const void *v, void *
     const size_t tsz = dt == HLA_BF16 ? 2 : 4;
     if ((d * tsz) % 16 != 0 || (dv * tsz) % 16 != 0 || d % 4 != 0 || dv % 4 != 0 || d > 128 || dv > 128)
         return cudaErrorInvalidValue;
+    if (const int split = ahla_step_split(BH, d, dv, normalized))
+        return dt == HLA_BF16
+                   ? ahla_step_split_launch<__nv_bfloat16>(q, k, v, out, state, BH, split, d, dv, normalized, eps, stream)
+                   : ahla_step_split_launch<float>(q, k, v, out, state, BH, split, d, dv, normalized, eps, stream);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -18,19 +18,13 @@
 // consecutive columns.
 #include "hla_internal.h"
 #include "sm103_prims.cuh"
+#include "step_split.cuh"
 
 namespace hla {
 namespace {
 
 constexpr int kStepThreads = 512;
 constexpr int kMaxUnits = 128 * 128 / 4 / kStepThreads;  // float4 units per thread for a 128 x 128 matrix
-
-template <int W>
-__device__ __forceinline__ float group_sum(float x) {
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o, W);
-    return x;
-}
 
 __device__ __forceinline__ float group_sum_rt(float x, int w) {
     switch (w) {
@@ -66,13 +60,6 @@ __device__ __forceinline__ float warp_sum8(float (&v)[8]) {
     x += __shfl_xor_sync(0xffffffffu, x, 2);
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     return x;
-}
-
-// sum_i a[i] b[i] over shared-memory vectors, computed by every warp on its own (no block barrier)
-__device__ __forceinline__ float warp_dot(const float *a, const float *b, int n) {
-    float s = 0.f;
-    for (int i = threadIdx.x & 31; i < n; i += 32) s += a[i] * b[i];
-    return group_sum<32>(s);
 }
 
 // 1-D bulk copy global -> shared (16-byte aligned, a multiple of 16 bytes), completing on `bar`
@@ -334,6 +321,220 @@ step2_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restri
     }
 }
 
+// ---------------------------------------------------------------------------
+// The step with every load issued at once, straight to registers: for head sizes up to 64 (one block of
+// 256 threads a head, several on an SM), and for few heads of 128 (a cluster of `split` blocks of 512
+// threads a head, block r with columns [r dv / split, ...) of C and G, or D, and the rows of S that it
+// writes).  The staged kernel above brings a head through one SM part by part; with small
+// heads it waits on each part in turn, with few heads most SMs are idle.  Each block forms u' = S' q from
+// all of S (a cluster's redundant reads come from L2 and cost less than an exchange between blocks), so
+// the blocks of a cluster meet only once, in a split barrier between their last read of S, m and h and
+// the first write to them.  Column sums go by shuffles, then over the warps in shared memory.
+// Measured, us a step (staged -> this), bf16 tokens: tuple 64 x 64, 16 heads 6.6 -> 4.8, 256 heads
+// 12.1 -> 5.9, 2048 heads 74.9 -> 43.7; (S, D, e) 64 x 64, 16 heads 4.6 -> 4.1, 2048 heads 44.9 -> 28.9;
+// tuple 128 x 128, 8 heads 7.7 -> 6.3, 32 heads 7.9 -> 6.7.  It is bound by the latency of a load,
+// three barriers and the shuffles between them; with many heads by its registers (two or three blocks
+// an SM; one more spilled and was slower).
+// NS, NC: float4 units that a thread takes of S and of a column slice.
+// ---------------------------------------------------------------------------
+template <typename T, bool kSDE, int TH, int NS, int NC>
+__global__ void __launch_bounds__(TH, TH == 256 ? (kSDE ? 3 : 2) : 1)
+step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
+                   float *state, int split, int d, int dv, int masked, int normalized, float eps) {
+    __shared__ __align__(16) float qs[128], ks[128], vs[128], us[128];
+    // per warp: sums of a column slice (at most 64 columns), for k^T C and u'^T C (or q^T D), and q^T G
+    __shared__ __align__(16) float part[3][TH / 32][64];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int hd = blockIdx.x / split, rank = blockIdx.x % split, cw = dv / split, col0 = rank * cw;
+    const long long offC = (long long)d * d, lenC = (long long)d * dv + d;
+    float *S = state + hd * (offC + lenC * (kSDE ? 1 : 2)), *C = S + offC, *m = C + (long long)d * dv;
+    float *G = C + lenC, *h = G + (long long)d * dv;
+    const int nS = (d * d) >> 2, wS = d >> 2;     // float4 units of S, of one of its rows
+    const int wC = cw >> 2, nC = d * wC;          // of a row of the slice, of the slice
+    const int c4 = (tid % wC) * 4, r0 = tid / wC, rstep = TH / wC;
+
+    // every load of the step
+    float4 sv[NS], cv[NC], gv[NC];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const int f = tid + i * TH;
+        sv[i] = f < nS ? reinterpret_cast<const float4 *>(S)[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const int row = r0 + i * rstep;
+        const bool ok = tid + i * TH < nC;
+        cv[i] = gv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok) cv[i] = *reinterpret_cast<const float4 *>(C + (long long)row * dv + col0 + c4);
+        if (!kSDE && masked && ok) gv[i] = *reinterpret_cast<const float4 *>(G + (long long)row * dv + col0 + c4);
+    }
+    // m and h (or e): four values a lane, in every warp
+    float mv[4], hv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = lane + 32 * i;
+        mv[i] = a < d ? m[a] : 0.f;
+        hv[i] = !kSDE && masked && a < d ? h[a] : 0.f;
+    }
+    if (tid < d) {
+        qs[tid] = to_f32(q[(long long)hd * d + tid]);
+        ks[tid] = to_f32(k[(long long)hd * d + tid]);
+    }
+    if (tid < dv) vs[tid] = to_f32(v[(long long)hd * dv + tid]);
+    __syncthreads();
+    const float kq = warp_dot(ks, qs, d);
+    float km = 0.f, qm = 0.f, qh = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = lane + 32 * i;
+        if (a < d) {
+            km = fmaf(ks[a], mv[i], km);
+            qm = fmaf(qs[a], mv[i], qm);
+            qh = fmaf(qs[a], hv[i], qh);
+        }
+    }
+    km = group_sum<32>(km);
+    qm = group_sum<32>(qm);
+    qh = group_sum<32>(qh);
+
+    // u' = S q + k (k.q)
+    if constexpr (NS == 8) {  // d = 128: a warp covers one row per unit
+        const int c = lane * 4;
+        float pu[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            pu[i] = sv[i].x * qs[c] + sv[i].y * qs[c + 1] + sv[i].z * qs[c + 2] + sv[i].w * qs[c + 3];
+        const float su = warp_sum8(pu);
+        if ((lane & 3) == 0) {
+            const int row = wid + TH / 32 * (lane >> 2);
+            us[row] = su + ks[row] * kq;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const int f = tid + i * TH, row = f / wS, c = (f % wS) * 4;
+            float pu = 0.f;
+            if (f < nS) pu = sv[i].x * qs[c] + sv[i].y * qs[c + 1] + sv[i].z * qs[c + 2] + sv[i].w * qs[c + 3];
+            pu = group_sum_rt(pu, wS);
+            if (f < nS && f % wS == 0) us[row] = pu + ks[row] * kq;
+        }
+    }
+    // sums that need no u': k^T C, q^T G; or q^T D
+    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const int row = min(r0 + i * rstep, d - 1);  // beyond the slice the values are zero
+        fma4(a0, kSDE ? qs[row] : ks[row], cv[i]);
+        if (!kSDE) fma4(a1, qs[row], gv[i]);
+    }
+    a0 = column_sum(a0, wC);
+    if (!kSDE) a1 = column_sum(a1, wC);
+    if (lane < wC) {
+        *reinterpret_cast<float4 *>(&part[0][wid][c4]) = a0;
+        if (!kSDE) *reinterpret_cast<float4 *>(&part[2][wid][c4]) = a1;
+    }
+    cluster_arrive();  // this block has read S, m, h
+    __syncthreads();   // us, part
+    const float uq = warp_dot(us, qs, d);
+    const float4 v4 = *reinterpret_cast<const float4 *>(vs + col0 + c4);
+    float4 kC = make_float4(0.f, 0.f, 0.f, 0.f);
+    float um = 0.f;
+    if (!kSDE) {
+        for (int w = 0; w < TH / 32; ++w) fma4(kC, 1.f, *reinterpret_cast<const float4 *>(&part[0][w][c4]));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (lane + 32 * i < d) um = fmaf(us[lane + 32 * i], mv[i], um);
+        um = group_sum<32>(um) + uq;  // u'.(m + q)
+        a0 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) fma4(a0, us[min(r0 + i * rstep, d - 1)], cv[i]);
+        a0 = column_sum(a0, wC);
+        if (lane < wC) *reinterpret_cast<float4 *>(&part[1][wid][c4]) = a0;
+    }
+    // the updated slices
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const int row = r0 + i * rstep;
+        if (tid + i * TH >= nC) continue;
+        *reinterpret_cast<float4 *>(C + (long long)row * dv + col0 + c4) = axpy4(cv[i], kSDE ? us[row] : qs[row], v4);
+        if (!kSDE && masked)
+            *reinterpret_cast<float4 *>(G + (long long)row * dv + col0 + c4) = axpy4(gv[i], ks[row], kC);
+    }
+    __syncthreads();  // part[1]
+    if (tid < cw) {
+        float x0 = 0.f, x1 = 0.f, x2 = 0.f;
+        for (int w = 0; w < TH / 32; ++w) {
+            x0 += part[0][w][tid];
+            if (!kSDE) {
+                x1 += part[1][w][tid];
+                x2 += part[2][w][tid];
+            }
+        }
+        float num, den;
+        if (kSDE) {
+            num = x0 + uq * vs[col0 + tid];
+            den = qm + uq;
+        } else {
+            num = x1 + uq * vs[col0 + tid];
+            den = um;
+            if (masked) {
+                num -= x2 + kq * x0;
+                den -= qh + kq * km;
+            }
+        }
+        from_f32(&out[(long long)hd * dv + col0 + tid], normalized ? num / (den + eps) : num);
+    }
+    cluster_wait();  // every block of the head has read S, m, h
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const int f = tid + i * TH, row = f / wS, c = (f % wS) * 4;
+        if (f < nS && row * split / d == rank)
+            reinterpret_cast<float4 *>(S)[f] = axpy4(sv[i], ks[row], *reinterpret_cast<const float4 *>(ks + c));
+    }
+    if (rank == 0 && wid == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int a = lane + 32 * i;
+            if (a >= d) continue;
+            m[a] = mv[i] + (kSDE ? us[a] : qs[a]);
+            if (!kSDE && masked) h[a] = hv[i] + ks[a] * km;
+        }
+    }
+}
+
+// Blocks per head of the kernel above, 0 where the staged kernel serves.  Head sizes up to 64: one,
+// for any number of heads (two or four were as fast for few heads and slower for many).  With a size of
+// 128, clusters while each fits the chip at once, one block an SM and a cluster within one GPC: 8 heads in
+// eights, 32 in fours (16 in eights and 38 in fours take two rounds, 11.5 and 12.1 us); in twos the
+// staged kernel is as fast (8.0 against 7.9 us at 40 heads).  A block's slice has 8 to 64 columns.
+int step2_split(int BH, int d, int dv) {
+    int s = 1;
+    if (d == 128 || dv == 128) s = BH <= 8 ? 8 : BH <= 32 ? 4 : 0;
+    if (s == 0) return 0;
+    while (s > 1 && dv / s < 8) s /= 2;
+    while (dv / s > 64) s *= 2;
+    return s;
+}
+
+template <typename T, bool kSDE>
+cudaError_t step2_split_launch(const void *q, const void *k, const void *v, void *out, float *state, int BH, int split,
+                               int d, int dv, int masked, int normalized, float eps, cudaStream_t stream) {
+    auto go = [&](auto kern, int threads) {
+        return launch_blocks(kern, BH, split, true, threads, stream, static_cast<const T *>(q), static_cast<const T *>(k),
+                            static_cast<const T *>(v), static_cast<T *>(out), state, split, d, dv, masked, normalized,
+                            eps);
+    };
+    const int units = d * (dv / split) / 4;  // of a slice: at most 4 a thread (slices of 8 to 64 columns)
+    if (d == 128) {
+        if (units <= 512) return go(step2_split_kernel<T, kSDE, 512, 8, 1>, 512);
+        if (units <= 1024) return go(step2_split_kernel<T, kSDE, 512, 8, 2>, 512);
+        return go(step2_split_kernel<T, kSDE, 512, 8, 4>, 512);
+    }
+    if (units <= 256) return go(step2_split_kernel<T, kSDE, 256, 4, 1>, 256);
+    if (units <= 512) return go(step2_split_kernel<T, kSDE, 256, 4, 2>, 256);
+    return go(step2_split_kernel<T, kSDE, 256, 4, 4>, 256);
+}
+
 // dynamic shared memory of step2_kernel: S, (C, m), (G, h) if masked, tokens
 size_t step2_smem(int d, int dv, int masked, size_t tsize) {
     const size_t nS = (size_t)d * d / 4, nCm = ((size_t)d * dv + d) / 4;
@@ -344,6 +545,11 @@ template <bool kSDE>
 cudaError_t step2_launch_t(const void *q, const void *k, const void *v, void *out, hla_dtype dt, int BH, int d,
                            int dv, int masked, int normalized, float eps, float *state, cudaStream_t stream) {
     if (BH == 0) return cudaSuccess;
+    if (const int split = step2_split(BH, d, dv))
+        return dt == HLA_BF16 ? step2_split_launch<__nv_bfloat16, kSDE>(q, k, v, out, state, BH, split, d, dv, masked,
+                                                                        normalized, eps, stream)
+                              : step2_split_launch<float, kSDE>(q, k, v, out, state, BH, split, d, dv, masked, normalized,
+                                                                eps, stream);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

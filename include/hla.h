@@ -237,10 +237,10 @@ int hla3_forward_path(int B, int H, int n, int d, int dv, int masked, int normal
 
 /*
  * hla2_backward_path -- which CUDA path hla2_backward takes for these arguments
- * on the current device, without launching anything: 1 the tensor-core kernel
- * (bf16 tokens, d = dv = 64, normalized = 0, an sm_103 device; one launch),
- * 0 the fp32 CUDA-core kernels, -1 the arguments are not
- * supported.
+ * on the current device, without launching anything: 1 the tensor cores (bf16
+ * tokens on an sm_103 device; d = dv = 64 with normalized = 0 in one launch, d or
+ * dv = 128 with the other 64 or 128 tile by tile), 0 the fp32 CUDA-core kernels,
+ * -1 the arguments are not supported.
  */
 int hla2_backward_path(int B, int H, int n, int d, int dv, int normalized, int chunk, hla_dtype dt);
 

@@ -248,7 +248,7 @@ int hla2_backward_path(int B, int H, int n, int d, int dv, int normalized, int c
     Bwd2 p{dummy, dummy, dummy, dummy, const_cast<void *>(dummy), const_cast<void *>(dummy),
            const_cast<void *>(dummy), dt, B * H, n, d, dv, normalized, 0.f, chunk, nullptr,
            hla2_backward_workspace_bytes(B, H, n, d, dv, chunk, dt)};
-    return ((long long)B * H > 0 && backward2_tc_applicable(p)) ? 1 : 0;
+    return ((long long)B * H > 0 && (backward2_tc_applicable(p) || backward2_tiles_applicable(p))) ? 1 : 0;
 }
 
 size_t ahla_state_floats(int d, int dv) {

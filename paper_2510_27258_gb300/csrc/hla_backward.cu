@@ -32,6 +32,8 @@
 // At B2 H16 n4096 d128 normalised the two scans that multiplied carries took 24
 // of 36.6 ms; as elementwise sums, with the register-tiled products of
 // chunk_simt.cuh, the call takes 2.1 ms.
+#include <algorithm>
+
 #include "chunk_simt.cuh"
 
 namespace hla {
@@ -355,12 +357,13 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
 
 size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int) {
     const size_t simt = kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
-    const size_t tc = backward2_tc_workspace_bytes(BH, n);
-    return simt > tc ? simt : tc;
+    const size_t tc = backward2_tc_workspace_bytes(BH, n), tiles = backward2_tiles_workspace_bytes(BH, n, d, dv);
+    return std::max(simt, std::max(tc, tiles));
 }
 
 cudaError_t backward2_launch(const Bwd2 &p, cudaStream_t stream) {
     if (backward2_tc_applicable(p)) return backward2_tc_launch(p, stream);
+    if (backward2_tiles_applicable(p)) return backward2_tiles_launch(p, stream);
     return with_padded_size(p.d, p.dv, [&](auto size) {
         constexpr int N = decltype(size)::value;
         return p.dt == HLA_BF16 ? backward_n<N, __nv_bfloat16>(p, stream) : backward_n<N, float>(p, stream);

@@ -96,6 +96,10 @@ cudaError_t backward2_launch(const Bwd2 &p, cudaStream_t stream);
 size_t backward2_tc_workspace_bytes(int BH, int n);
 bool backward2_tc_applicable(const Bwd2 &p);
 cudaError_t backward2_tc_launch(const Bwd2 &p, cudaStream_t stream);
+// tile by tile on the tensor cores (hla_backward_tiles_sm103.cu): bf16, d or dv = 128 (the other 64 or 128)
+size_t backward2_tiles_workspace_bytes(int BH, int n, int d, int dv);
+bool backward2_tiles_applicable(const Bwd2 &p);
+cudaError_t backward2_tiles_launch(const Bwd2 &p, cudaStream_t stream);
 
 // AHLA (asymmetric second order): chunk-parallel forward and decode step
 size_t ahla_workspace_bytes_internal(int BH, int n, int d, int dv, int chunk);

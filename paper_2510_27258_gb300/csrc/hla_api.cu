@@ -139,11 +139,11 @@ hla_status hla2_forward(const void *q, const void *k, const void *v, void *out, 
         return fail(HLA_ERR_INVALID_ARGUMENT, "workspace must be 256-byte aligned");
     if ((long long)B * H == 0) return HLA_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    st = cuda_status(cudaMemsetAsync(workspace, 0, kWsHeaderBytes, s), "clearing the workspace header");
-    if (st != HLA_OK) return st;
     Fwd2 p{q, k, v, out, dt, B * H, n, d, dv, masked, normalized, eps, chunk, state_in, state_out,
            static_cast<char *>(workspace), workspace_bytes};
-    if (fused2_applicable(p)) return cuda_status(fused2_forward(p, s), "fused forward");
+    if (fused2_applicable(p)) return cuda_status(fused2_forward(p, s), "fused forward");  // clears the header itself
+    st = cuda_status(cudaMemsetAsync(workspace, 0, kWsHeaderBytes, s), "clearing the workspace header");
+    if (st != HLA_OK) return st;
     return cuda_status(generic2_forward(p, s), "generic forward");
 }
 

@@ -70,9 +70,6 @@ extern "C" hla_status hla2_forward_noalloc(const void *q, const void *k, const v
     hla_status st = scratch_address(&scratch);
     if (st != HLA_OK) return st;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // the error word must start at zero; the fused launch clears its own counters
-    st = cuda_status(cudaMemsetAsync(scratch, 0, kWsHeaderBytes, s), "clearing the scratch header");
-    if (st != HLA_OK) return st;
     Fwd2 p{q, k, v, out, dt, B * H, n, d, dv, masked, normalized, eps, chunk, state_in, nullptr,
            static_cast<char *>(scratch), kNoAllocScratchBytes};
     return cuda_status(fused2_forward(p, s), "fused forward (no-alloc)");

@@ -40,7 +40,13 @@
 // +31 (one row each) and columns 32 (w / 4) .. +31.
 //
 // Head sizes: d = dv = 64 has its own instantiation whose products run over 64
-// features (the tiles and TMEM regions keep their 128-column layout).  A mix of
+// features.  S, D and X then take 64 TMEM columns each, which leaves room for a
+// second masked tile, and K 16 KiB, which leaves its slot room for the next one:
+// the next tile's A = Q K^T and S += K^T K run under the X epilogue and its W is
+// formed while T runs (the output also gets a block of its own beside D_p): B8
+// H16 n2048 73.8 -> 72.6 us.  What bounds it is the products' contention with the
+// epilogue for shared memory and TMEM: 52 products a tile take 7700 cycles, 148
+// each, where alone they take 50 to 70.  A mix of
 // 64 and 128 runs as 128 with zero features 64..127: the TMA box of those
 // columns lies wholly outside the tensor and is zero-filled, so S, x_t, D and e
 // have zero rows / columns there (the S shift cancels exactly: q_f = 0) and the
@@ -89,12 +95,19 @@ constexpr uint32_t kSmemBytes = kSmemTiles + kMiscBytes;  // = 227 KiB; base mus
 enum Slot { kQ0 = 0, kQ1 = 1, kK = 2, kV = 3, kW = 4, kSX = 5, kSD = 6 };
 
 // TMEM columns: S carry, D carry, A -> T, X -> O
-constexpr uint32_t kTS = 0, kTD = 128, kTA = 256, kTX = 384;
+// at head size 128; at 64 (Cols<true>) S, D and X take 64 columns each, which leaves room for a second A
+template <bool kNarrow>
+struct Cols {
+    static constexpr uint32_t S = 0, D = kNarrow ? 64 : 128, A = kNarrow ? 128 : 256, A1 = 256, X = 384;
+    // the masked tile of a tile of parity `par`: two regions in turn at head size 64
+    __device__ static constexpr uint32_t a(uint32_t par) { return kNarrow && par ? A1 : A; }
+    // the regions of the three fix-up buffers
+    __device__ static constexpr uint32_t fix(int i) { return i == 0 ? A : i == 1 ? X : D; }
+};
 
 // fix-up buffers (three tiles in flight): Q slot, provisional output slot, TMEM columns of F
 __device__ __forceinline__ int fix_q(int i) { return i == 0 ? kQ0 : i == 1 ? kQ1 : kW; }
 __device__ __forceinline__ int fix_o(int i) { return i == 0 ? kK : i == 1 ? kV : kSX; }
-__device__ __forceinline__ uint32_t fix_t(int i) { return i == 0 ? kTA : i == 1 ? kTX : kTD; }
 
 // barrier indices
 enum Bar {
@@ -257,6 +270,18 @@ __device__ __forceinline__ void store_split32(uint8_t *th, uint8_t *tl, int r, i
     }
 }
 
+// the same for 16 values
+__device__ __forceinline__ void store_split16(uint8_t *th, uint8_t *tl, int r, int c0, const float (&v)[16], bool lo) {
+#pragma unroll
+    for (int jj = 0; jj < 16; jj += 8) {
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split2(v[jj + 2 * i], v[jj + 2 * i + 1], h[i], l[i]);
+        *reinterpret_cast<uint4 *>(th + tile_off(r, c0 + jj)) = make_uint4(h[0], h[1], h[2], h[3]);
+        if (lo) *reinterpret_cast<uint4 *>(tl + tile_off(r, c0 + jj)) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+}
+
 // zero the entries of columns c0..c0+31 above the diagonal of row r (c > r); for the
 // 32 x 32 diagonal block of the tile, r - c0 = lane
 // kSel: by selects (no branch that diverges the warp); else by a branch per element, which for the
@@ -320,6 +345,14 @@ __device__ __forceinline__ void ld32(uint32_t addr, float (&f)[32]) {
     tmem_ld_wait();
 #pragma unroll
     for (int j = 0; j < 32; ++j) f[j] = __uint_as_float(a[j]);
+}
+
+__device__ __forceinline__ void ld16(uint32_t addr, float (&f)[16]) {
+    uint32_t a[16];
+    tmem_ld16(addr, a);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(a[j]);
 }
 
 // Column sums of v over the 32 lanes of a warp: returns, in lane l, the sum of
@@ -404,6 +437,8 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     // carries and TMEM regions are neither computed nor read; see the narrow notes in the epilogue)
     constexpr int kF = kNarrow ? 64 : 128;
     constexpr int kFS = kF / 16;  // K steps of a contraction over the head size
+    using TC = Cols<kNarrow>;
+    constexpr uint32_t kTS = TC::S, kTD = TC::D, kTX = TC::X;
     const bool need_e = !kUnmasked && (kState || p.normalized);  // the e carry (never unmasked)
     constexpr bool d_lo = kState;                 // D with X_lo, issued before O
 
@@ -451,6 +486,15 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tma_load_3d_hint(slot(s), map, &ms->bar[bLd0 + s], 0, tok0, head, pol);
         tma_load_3d_hint(slot(s) + kBlockBytes, map, &ms->bar[bLd0 + s], 64, tok0, head, pol);
     };
+    // Head size 64: tile j's K takes the first or second half of slot K (64 columns are one 16 KiB block) as j is
+    // even or odd, so the next tile's is there before this one's last use.  S += K^T K reads the 16 KiB after K as
+    // features 64..127: whatever lies there, it only reaches rows 64..127 of S, which nothing reads.
+    auto load_k_half = [&](int half, int head, int tok0, uint64_t pol) {
+        ld_pend |= 1u << kK;
+        mbar_arrive_expect_tx(&ms->bar[bLd0 + kK], kBlockBytes);
+        tma_load_3d_hint(slot(kK) + half * kBlockBytes, &tm_k, &ms->bar[bLd0 + kK], 0, tok0, head, pol);
+    };
+    auto kh = [&](int j) { return kNarrow && (j & 1) ? (uint32_t)(kBlockBytes >> 4) : 0u; };  // K of tile j in slot K
     auto wait_ld = [&](int s) {
         if (!bar_wait(ms, bLd0 + s, (ld_par >> s) & 1u, p)) return false;  // still pending
         ld_par ^= 1u << s;
@@ -518,8 +562,9 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 load_tile(kV, &tm_v, head, t0 * kTile, pol_first);
                 if (wait_ld(kQ0) && (!reload_k || wait_ld(kK))) {
                     tc_fence_after();
-                    mma128<false, false, 128, kFS>(tb + kTA, lk(kQ0), lk(kK), 0u);  // A = Q K^T
+                    mma128<false, false, 128, kFS>(tb + TC::a(n_tiles & 1), lk(kQ0), lk(kK), 0u);  // A = Q K^T
                     umma_commit(&ms->bar[bEvA]);
+                    if (kNarrow && nt > 1) load_k_half(1, head, (t0 + 1) * kTile, pol_first);
                 }
 
                 // ---- 2. sweep ----
@@ -530,6 +575,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 for (int j = 0; j < nt && !ms->abort_flag; ++j) {
                     const uint32_t tp = n_tiles & 1;
                     const int qs = (j & 1) ? kQ1 : kQ0, qo = (j & 1) ? kQ0 : kQ1;
+                    const uint32_t ta = tb + TC::a(tp);  // this tile's A, W and T
                     // slot qo (Q of the previous tile, last read by its O MMA) takes the next Q
                     if (j + 1 < nt) load_tile(qo, &tm_q, head, (t0 + j + 1) * kTile, pol_q);
                     // X = Q R_hi + Q R_lo + W_hi K + W_lo K; the Q R part runs while W is built.  For the
@@ -542,23 +588,32 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     mma128<false, false, kF, kFS>(tb + kTX, lk(qs), lk(kSX), 0u);      // X = Q R_hi
                     if (precise) mma128<false, false, kF, kFS>(tb + kTX, lk(qs), lk(kW), 1u);  // += Q R_lo
                     // S += K^T K while the W epilogue runs (the S carry was read by the previous split,
-                    // before Q R could start)
-                    if (kState || j + 1 < nt) mma128<true, true, kF>(tb + kTS, lm(kK), lm(kK), 1u);
+                    // before Q R could start); at head size 64, where W is ready, under the X epilogue
+                    const bool s_step = kState || j + 1 < nt;
+                    if (!kNarrow && s_step) mma128<true, true, kF>(tb + kTS, lm(kK), lm(kK), 1u);
                     if (j > 0 && !bar_wait(ms, bEpW, tp, p)) break;  // W (hi, lo) ready
                     tc_fence_after();
-                    mma128_ts<true, kF>(tb + kTX, tb + kTA, lm(kK), 1u);          // += W_hi K (W in TMEM)
-                    if (precise) mma128_ts<true, kF>(tb + kTX, tb + kTA + 16, lm(kK), 1u);  // += W_lo K
+                    mma128_ts<true, kF>(tb + kTX, ta, lm(kK) + kh(j), 1u);          // += W_hi K (W in TMEM)
+                    if (precise) mma128_ts<true, kF>(tb + kTX, ta + 16, lm(kK) + kh(j), 1u);  // += W_lo K
                     umma_commit(&ms->bar[bEvX]);
-                    if (!bar_wait(ms, bEvX, tp, p)) break;  // X and S MMAs done: slot K free
-                    if (j + 1 < nt) load_tile(kK, &tm_k, head, (t0 + j + 1) * kTile, pol_first);
+                    if (kNarrow && j + 1 < nt) {
+                        // the next tile's A = Q K^T under the X epilogue: its W is then formed while T = Q X^T runs
+                        if (!wait_ld(qo) || !wait_ld(kK)) break;
+                        tc_fence_after();
+                        mma128<false, false, 128, kFS>(tb + TC::a(tp ^ 1u), lk(qo), lk(kK) + kh(j + 1), 0u);
+                        umma_commit(&ms->bar[bEvA]);
+                    }
+                    if (kNarrow && s_step) mma128<true, true, kF>(tb + kTS, lm(kK) + kh(j), lm(kK) + kh(j), 1u);
+                    if (!bar_wait(ms, bEvX, tp, p)) break;  // X done (at head size 128 S too: slot K is free)
+                    if (!kNarrow && j + 1 < nt) load_tile(kK, &tm_k, head, (t0 + j + 1) * kTile, pol_first);
                     if (!bar_wait(ms, bEpX, tp, p)) break;  // X_hi, X_lo in SX, W; D_p read out of TMEM
                     tc_fence_after();
                     if constexpr (!kUnmasked) {
-                        mma128<false, false, 128, kFS>(tb + kTA, lk(qs), lk(kSX), 0u);  // T = Q X_hi^T
-                        mma128<false, false, 128, kFS>(tb + kTA, lk(qs), lk(kW), 1u);   // += Q X_lo^T
+                        mma128<false, false, 128, kFS>(ta, lk(qs), lk(kSX), 0u);  // T = Q X_hi^T
+                        mma128<false, false, 128, kFS>(ta, lk(qs), lk(kW), 1u);   // += Q X_lo^T
                     } else {
-                        mma128<false, false, 128, kFS>(tb + kTA, lk(kSX), lk(qs), 0u);  // T = X_hi Q^T
-                        mma128<false, false, 128, kFS>(tb + kTA, lk(kW), lk(qs), 1u);   // += X_lo Q^T
+                        mma128<false, false, 128, kFS>(ta, lk(kSX), lk(qs), 0u);  // T = X_hi Q^T
+                        mma128<false, false, 128, kFS>(ta, lk(kW), lk(qs), 1u);   // += X_lo Q^T
                     }
                     umma_commit(&ms->bar[bEvT]);
                     if (!wait_ld(kV)) break;
@@ -575,16 +630,19 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         mma128<false, true, kF, kFS>(tb + kTX, lk(kSX), lm(kSD), 0u);  // O = X_hi C_p
                         umma_commit(&ms->bar[bEvD]);  // X (slot SX) read: the S split may overwrite it
                     }
-                    if (!bar_wait(ms, bEpT, tp, p)) break;  // T (bf16) in TMEM A
+                    if (!bar_wait(ms, bEpT, tp, p)) break;  // T (bf16) in TMEM A; S done (issued before T)
+                    if (kNarrow && j + 2 < nt) load_k_half(j & 1, head, (t0 + j + 2) * kTile, pol_first);
                     tc_fence_after();
-                    mma128_ts<true, kF>(tb + kTX, tb + kTA, lm(kV), 1u);          // O += T V (T in TMEM)
+                    mma128_ts<true, kF>(tb + kTX, ta, lm(kV), 1u);          // O += T V (T in TMEM)
                     umma_commit(&ms->bar[bEvO]);
                     if (!bar_wait(ms, bEvO, tp, p)) break;  // T, V and D_p read
                     if (j + 1 < nt) {  // next tile's A = Q K^T overlaps this tile's output epilogue
-                        if (!wait_ld(qo) || !wait_ld(kK)) break;
-                        tc_fence_after();
-                        mma128<false, false, 128, kFS>(tb + kTA, lk(qo), lk(kK), 0u);
-                        umma_commit(&ms->bar[bEvA]);
+                        if (!kNarrow) {
+                            if (!wait_ld(qo) || !wait_ld(kK)) break;
+                            tc_fence_after();
+                            mma128<false, false, 128, kFS>(tb + TC::A, lk(qo), lk(kK), 0u);
+                            umma_commit(&ms->bar[bEvA]);
+                        }
                         load_tile(kV, &tm_v, head, (t0 + j + 1) * kTile, pol_first);
                     }
                     ++n_tiles;
@@ -619,7 +677,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             const int i = j % 3;
                             if (!wait_ld(fix_q(i)) || !wait_ld(fix_o(i))) break;
                             tc_fence_after();
-                            mma128<false, true, kF, kFS>(tb + fix_t(i), lk(fix_q(i)), lm(kSD), 0u);  // F = Q D_prefix
+                            mma128<false, true, kF, kFS>(tb + TC::fix(i), lk(fix_q(i)), lm(kSD), 0u);  // F = Q D_prefix
                             umma_commit(&ms->bar[bEvF + i]);
                             if (j >= 1) {  // tile j-1 done: its buffer takes tile j+2
                                 const int g = (j - 1) % 3;
@@ -725,7 +783,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 uint32_t u[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) u[j] = __float_as_uint(sp[j]);
-                tmem_st32(tb + lane_base + kTS + c0, u);
+                if (fcol) tmem_st32(tb + lane_base + kTS + c0, u);
                 // split S_p = cs I + R into R_hi (slot SX) and R_lo (slot W)
                 if (cq == qd) shift_diag32<kNarrow>(sp, lane, cs);
                 if (fcol) store_split32(slot(kSX), slot(kW), r, c0, sp, precise);
@@ -738,7 +796,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     u[j] = __float_as_uint(v4.x); u[j + 1] = __float_as_uint(v4.y);
                     u[j + 2] = __float_as_uint(v4.z); u[j + 3] = __float_as_uint(v4.w);
                 }
-                tmem_st32(tb + lane_base + kTD + c0, u);
+                if (fcol) tmem_st32(tb + lane_base + kTD + c0, u);
                 if (cq == 0) ms->eloc[r] = d0 ? d0[kD * kD + r] : 0.f;
                 tmem_st_wait();
             }
@@ -753,41 +811,57 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     ms->eloc[c0 + lane] += (ec + ms->part[0][c0 + lane]) + (ms->part[1][c0 + lane] + ms->part[2][c0 + lane]);
                 epi_sync();
             };
+            // W = L . A -> bf16 hi and lo, written over this thread's own A columns (at t) in TMEM
+            // (the A operand of X += W K): hi in columns c0 .. +15, lo in c0 + 16 .. +31
+            auto form_w = [&](uint32_t t, uint32_t par) {
+                bar_wait(ms, bEvA, par, p);
+                tc_fence_after();
+                uint32_t h[16], l[16];
+                if (blk_zero) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) h[i] = l[i] = 0u;
+                } else {
+                    float f[32];
+                    ld32(t, f);
+                    if (cq == qd) mask_upper32<kNarrow>(f, r, c0);
+                    split_pack32(f, h, l);
+                }
+                tmem_st16(t, h);
+                if (precise) tmem_st16(t + 16, l);
+                tmem_st_wait();
+                epi_arrive(ms, bEpW);
+            };
             float ecol = 0.f;  // this thread's column sum of the last tile's X, added in the next tile's X wait
             for (int j = 0; j < nt; ++j) {
                 const uint32_t tp = n_tiles & 1;
                 const uint8_t *qt = slot((j & 1) ? kQ1 : kQ0);
                 const int tok0 = (t0 + j) * kTile;
 
-                // W = L . A -> bf16 hi and lo, written over this thread's own A columns in TMEM
-                // (the A operand of X += W K): hi in columns c0 .. +15, lo in c0 + 16 .. +31
-                bar_wait(ms, bEvA, tp, p);
-                tc_fence_after();
-                {
-                    uint32_t h[16], l[16];
-                    if (blk_zero) {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) h[i] = l[i] = 0u;
-                    } else {
-                        float f[32];
-                        ld32(tb + lane_base + kTA + c0, f);
-                        if (cq == qd) mask_upper32<kNarrow>(f, r, c0);
-                        split_pack32(f, h, l);
-                    }
-                    tmem_st16(tb + lane_base + kTA + c0, h);
-                    if (precise) tmem_st16(tb + lane_base + kTA + c0 + 16, l);
-                    tmem_st_wait();
-                }
-                epi_arrive(ms, bEpW);
+                const uint32_t ta = tb + lane_base + TC::a(tp) + c0;  // this thread's columns of A, W and T
+                // (at head size 64 later tiles' W was formed during the tile before)
+                if (!kNarrow || j == 0) form_w(ta, tp);
 
-                if (et == 0) tma_store_wait_read();  // the previous output tile has left slot SD
-                epi_sync();
+                if (!kNarrow) {
+                    if (et == 0) tma_store_wait_read();  // the previous output tile has left slot SD
+                    epi_sync();
+                } else if (j == 0) {  // D_p is read 16 columns a warp: the initial D came 32 columns a warp
+                    tc_fence_before();
+                    epi_sync();
+                    tc_fence_after();
+                }
                 if (need_e && j > 0) add_ecol(ecol);  // the previous tile's X, before q_t . e_p below
 
                 // while X = W K + Q S_p runs: D_p (bf16, final since the previous O) -> slot SD, read
                 // out of TMEM before this tile's D MMA (issued after the X hand-off), and q_t . e_p,
                 // the carried part of the denominator
-                if (fcol) {
+                if constexpr (kNarrow) {
+                    if (qd < 2) {
+                        float f[16];
+                        ld16(tb + lane_base + kTD + 16 * cq, f);
+#pragma unroll
+                        for (int jj = 0; jj < 16; jj += 8) store_row8(slot(kSD), r, 16 * cq + jj, f + jj);
+                    }
+                } else {
                     float f[32];
                     ld32(tb + lane_base + kTD + c0, f);
 #pragma unroll
@@ -825,8 +899,9 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 fence_async_smem();  // X_hi, X_lo and D_p (above) visible to the MMAs
                 epi_arrive(ms, bEpX);
 
-                // while T = Q X^T runs: column sums of X (e carry)
+                // while T = Q X^T runs: column sums of X (e carry), the next tile's W (head size 64)
                 if (need_e) ecol = warp_colsum32(x);  // column c0 + lane over this warp's rows
+                if (kNarrow && j + 1 < nt) form_w(tb + lane_base + TC::a(tp ^ 1u) + c0, tp ^ 1u);
 
                 // T = L . (Q X^T) -> bf16 in TMEM; row sums
                 bar_wait(ms, bEvT, tp, p);
@@ -839,13 +914,13 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         for (int i = 0; i < 16; ++i) h[i] = 0u;
                     } else {
                         float f[32];
-                        ld32(tb + lane_base + kTA + c0, f);
+                        ld32(ta, f);
                         if (cq == qd) mask_upper32<kNarrow>(f, r, c0);
 #pragma unroll
                         for (int jj = 0; jj < 32; ++jj) den_part += f[jj];
                         pack32(f, h);
                     }
-                    tmem_st16(tb + lane_base + kTA + c0, h);
+                    tmem_st16(ta, h);
                     tmem_st_wait();
                 }
                 epi_arrive(ms, bEpT);
@@ -855,6 +930,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     if (cq == 0) ms->den[r] = den_part;
                     else ms->part[cq - 1][r] = den_part;
                 }
+                if (kNarrow && et == 0) tma_store_wait_read();  // the previous output tile has left its block
                 epi_sync();
                 const float den = p.normalized ? ((ms->den[r] + ms->part[0][r]) + ms->part[1][r]) + ms->part[2][r] : 1.f;
 
@@ -863,28 +939,41 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 bar_wait(ms, bEvD, tp, p);
                 tc_fence_after();
                 if (j + 1 < nt) {
-                    float f[32];
-                    if (fcol) {
-                        ld32(tb + lane_base + kTS + c0, f);
-                    } else {
-#pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) f[jj] = 0.f;
-                    }
                     const float *dt = ms->dtr[(j + 1) & 1];
                     cs = bf16_round((j == 0 ? tr_s : (dt[0] + dt[1]) + (dt[2] + dt[3])) / kD);
-                    {
+                    if constexpr (kNarrow) {
+                        // the 64 rows of S in lanes 0..63: 16 columns for each of the eight warps on those lanes
+                        if (qd < 2) {
+                            float f[16];
+                            ld16(tb + lane_base + kTS + 16 * cq, f);
+                            const int dc = (r >> 4) == cq ? (r & 15) : -1;  // this thread's diagonal entry
+                            float dg = 0.f;
+#pragma unroll
+                            for (int jj = 0; jj < 16; ++jj) dg = jj == dc ? f[jj] : dg;
+                            dg = warp_sum(dg);
+                            if ((cq >> 1) == qd && lane == 0) ms->dtr[j & 1][cq] = dg;
+#pragma unroll
+                            for (int jj = 0; jj < 16; ++jj) f[jj] -= jj == dc ? cs : 0.f;
+                            store_split16(slot(kSX), slot(kW), r, 16 * cq, f, precise);
+                        }
+                    } else {
+                        float f[32];
+                        ld32(tb + lane_base + kTS + c0, f);
                         float dg = 0.f;
                         if (cq == qd) dg = pick_lane32<kNarrow>(f, lane);
                         dg = warp_sum(dg);
                         if (cq == qd && lane == 0) ms->dtr[j & 1][qd] = dg;
+                        if (cq == qd) shift_diag32<kNarrow>(f, lane, cs);
+                        store_split32(slot(kSX), slot(kW), r, c0, f, precise);
                     }
-                    if (cq == qd) shift_diag32<kNarrow>(f, lane, cs);
-                    if (fcol) store_split32(slot(kSX), slot(kW), r, c0, f, precise);
                     fence_async_smem();
                     epi_arrive(ms, bEpR);  // R of the next tile ready: Q R may start once O is read
                 }
 
-                // O (provisional for segments > 0, final for the first) -> slot SD, TMA store
+                // O (provisional for segments > 0, final for the first) -> slot SD, TMA store.  At head size 64
+                // it takes the second block of the slot, D_p the first, so that the next D_p need not wait
+                // for the store to have read O.
+                uint8_t *ot = slot(kSD) + (kNarrow ? kBlockBytes : 0);
                 bar_wait(ms, bEvO, tp, p);
                 tc_fence_after();
                 {
@@ -904,7 +993,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     }
                     if (fcol) {
 #pragma unroll
-                        for (int jj = 0; jj < 32; jj += 8) store_row8(slot(kSD), r, c0 + jj, f + jj);
+                        for (int jj = 0; jj < 32; jj += 8) store_row8(ot, r, c0 + jj, f + jj);
                     }
                     if (!final_out && p.normalized && cq == 0 && tok0 + r < p.n)
                         p.den_loc[(size_t)head * p.n + tok0 + r] = den;
@@ -913,8 +1002,8 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 epi_sync();  // also: every denominator read before part is reused
                 if (et == 0) {  // provisional outputs stay in L2 for the fix-up
                     const uint64_t pol = sigma > 0 ? l2_policy_evict_last() : l2_policy_evict_first();
-                    tma_store_3d_hint(&tm_o, slot(kSD), 0, tok0, head, pol);
-                    if (p.out_blocks > 1) tma_store_3d_hint(&tm_o, slot(kSD) + kBlockBytes, 64, tok0, head, pol);
+                    tma_store_3d_hint(&tm_o, ot, 0, tok0, head, pol);
+                    if (!kNarrow && p.out_blocks > 1) tma_store_3d_hint(&tm_o, ot + kBlockBytes, 64, tok0, head, pol);
                     tma_store_commit();
                 }
                 ++n_tiles;
@@ -936,7 +1025,12 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 float4 *dcur = reinterpret_cast<float4 *>(ring_cur + kD * kD);
                 {
                     float f[32], dp[32];
-                    ld32(tb + lane_base + kTD + c0, f);
+                    if (fcol) {
+                        ld32(tb + lane_base + kTD + c0, f);
+                    } else {
+#pragma unroll
+                        for (int jj = 0; jj < 32; ++jj) f[jj] = 0.f;
+                    }
 #pragma unroll
                     for (int jj = 0; jj < 32; jj += 4) {
                         const float4 v4 = dprev ? __ldcg(dprev + ring4(jj / 4, et)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -993,7 +1087,7 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             : 1.f;
                         if (fcol) {
                             float f[32];
-                            ld32(tb + lane_base + fix_t(i) + c0, f);
+                            ld32(tb + lane_base + TC::fix(i) + c0, f);
 #pragma unroll
                             for (int jj = 0; jj < 32; jj += 8) {
                                 float o8[8], w8[8];

@@ -4,7 +4,7 @@
 // A block of 128 threads works on one chunk of 64 tokens.  Operands sit in shared memory as fp32
 // rows of N + 4 floats (N = 32, 64 or 128, the head sizes padded with zeros), masked chunk tiles as
 // rows of 68; a carry (d x dv, fp32, in global memory) streams through shared memory 16 rows at a
-// time.  What bounds a product is the shared-memory bandwidth (128 bytes per clock and SM, so a
+// time (eight at N = 64).  What bounds a product is the shared-memory bandwidth (128 bytes per clock and SM, so a
 // 16-byte load of a warp costs four clocks) against four fp32 warp multiply-adds per clock: a thread
 // therefore keeps 8 x 8 outputs (8 x 4 at N = 64, 4 x 4 at N = 32) and every load brings 16 bytes,
 // 16 loads per 256 multiply-adds at N = 128.  The eight lanes that share a load phase read either
@@ -27,12 +27,13 @@ namespace {
 constexpr int kC = 64;        // tokens of a chunk
 constexpr int kCT = 128;      // threads of a block
 constexpr int kLdW = kC + 4;  // row length of a masked chunk tile
-constexpr int kSlice = 16;    // rows of a carry in shared memory at a time
 
 template <int N>
 struct Tile {
     static constexpr int RM = N == 32 ? 4 : 8, CM = N == 128 ? 8 : 4;  // outputs of a thread
     static constexpr int LD = N + 4;
+    // rows of a carry in shared memory at a time: at N = 64 eight, so that four blocks fit an SM
+    static constexpr int SL = N == 64 ? 8 : 16;
     int rg, cg;
     __device__ Tile() {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -258,13 +259,13 @@ __device__ __forceinline__ void nt_masked(float *Wt, const float *A, const float
 enum CarryUse { kPlain, kTransposed, kSymmetric };  // B = R, R^T, R + R^T
 
 // acc += A B, A row-major in shared memory (rows of N + 4), B (K x width) a carry in global memory:
-// R rows of `ldr` floats.  Slices of 16 rows of B pass through `stage` (2 x 16 x N floats), the next
+// R rows of `ldr` floats.  Slices of SL rows of B pass through `stage` (2 x SL x N floats), the next
 // one loaded into registers while this one is multiplied.  K and width are multiples of 16.  Ends
 // with every thread past its last read of `stage`.
 template <int N, CarryUse U>
 __device__ __forceinline__ void nn_carry(Acc<N> &acc, const Tile<N> &t, const float *A, const float *__restrict__ R,
                                          int ldr, int K, int width, float *stage) {
-    constexpr int PT = kSlice * N / kCT;  // floats of a slice per thread: 16, 8, 4
+    constexpr int kSlice = Tile<N>::SL, PT = kSlice * N / kCT;  // floats of a slice per thread: 16, 4, 4
     float buf[PT];
     const int tid = threadIdx.x;
     const int tc = tid % N, tk = (tid / N) * PT;  // transposed use: column tc, rows tk .. tk + PT - 1
@@ -380,9 +381,13 @@ __device__ __forceinline__ float row_dot(const float *A, int ld, const float *v,
 }
 
 template <int N>
-constexpr int stage_floats() { return 2 * kSlice * N; }
+constexpr int stage_floats() { return 2 * Tile<N>::SL * N; }
 template <int N>
 constexpr int tile_floats() { return kC * (N + 4); }
+// blocks an SM that the chunk kernels are compiled for: as many as their shared memory admits at N = 64 and
+// 128; one block more at N = 64 takes 512 blocks (B2 H16 n1000) from two rounds to one, 46 -> 41 us
+template <int N>
+constexpr int blocks_per_sm() { return N == 128 ? 2 : 4; }
 
 // ---------------------------------------------------------------------------
 // per-chunk records and their prefix sums.  Records of a head: nch of them, then one that holds the

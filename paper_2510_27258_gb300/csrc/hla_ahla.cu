@@ -59,7 +59,7 @@ struct AParams {
 // per chunk: A, [R | s], A [R | s] and the increments K^T [R | s] of [E | n].  Two token buffers serve in
 // turn as Q, K, V and R, as in the second-order kernel.
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2)
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     ahla_chunk_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                       const __grid_constant__ AParams A) {
     extern __shared__ __align__(16) float sm[];

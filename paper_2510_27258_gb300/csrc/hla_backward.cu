@@ -102,7 +102,7 @@ __device__ __forceinline__ void load_upstream(float *dst, float *us, const BPara
 // X, the increments X^T V, X^T 1 of D and e; normalised: T V and T 1
 // ---------------------------------------------------------------------------
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2) bwd_x_kernel(const __grid_constant__ BParams<T> P) {
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_x_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     const Chunk<T> ch(P);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kCT, 2) bwd_x_kernel(const __grid_constant__ B
 // Q^T u of Gam^T and h
 // ---------------------------------------------------------------------------
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2) bwd_upstream_kernel(const __grid_constant__ BParams<T> P) {
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_upstream_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *stage = b1 + tile_floats<N>(), *us = stage + stage_floats<N>();
     const Chunk<T> ch(P);
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kCT, 2) bwd_upstream_kernel(const __grid_const
 // Y and the increments Q^T Y of Lam
 // ---------------------------------------------------------------------------
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2) bwd_y_kernel(const __grid_constant__ BParams<T> P) {
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_y_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *us = stage + stage_floats<N>();
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kCT, 2) bwd_y_kernel(const __grid_constant__ B
 // the gradients: blockIdx.z 0 dQ, 1 dK, 2 dV
 // ---------------------------------------------------------------------------
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2) bwd_grad_kernel(const __grid_constant__ BParams<T> P) {
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *us = stage + stage_floats<N>();

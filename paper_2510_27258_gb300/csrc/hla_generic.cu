@@ -19,7 +19,7 @@
 //
 // The chain of products S_p C_c over the chunks that the sums replace took 20 %
 // of a call and ran on a few blocks, the chunk kernels had one multiply-add per
-// shared-memory load: B2 H16 n1000 d64 fp32 1975 us, now 84 us.
+// shared-memory load: B2 H16 n1000 d64 fp32 1975 us, now 81 us.
 #include <algorithm>
 
 #include "chunk_simt.cuh"
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kStateThreads) g2_final_kernel(float *__restri
 // in turn as Q, K, X and V: 94 KB of shared memory at N = 128, so two blocks fit an SM.
 // ---------------------------------------------------------------------------
 template <int N, typename T>
-__global__ void __launch_bounds__(kCT, 2)
+__global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     g2_chunk_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                     const __grid_constant__ GParams P) {
     extern __shared__ __align__(16) float sm[];

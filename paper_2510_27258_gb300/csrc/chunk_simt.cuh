@@ -19,6 +19,7 @@
 
 #include <type_traits>
 
+#include "chain_launch.cuh"
 #include "hla_internal.h"
 
 namespace hla {
@@ -415,6 +416,7 @@ struct ScanJobs {
 // exclusive prefix (suffix) sums in place, one float4 a thread; eight records' loads in flight, which
 // is what bounds it (memory latency over the chunks in turn)
 __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ ScanJobs jobs) {
+    chain_begin();
     const ScanJob &J = jobs.j[blockIdx.z];
     const int e = (blockIdx.x * 64 + threadIdx.x) * 4, hd = blockIdx.y, nch = J.r.nch;
     if (e >= J.r.len) return;
@@ -439,11 +441,10 @@ __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ 
     if (J.total) *reinterpret_cast<float4 *>(J.total + hd * J.total_stride + e) = acc;
 }
 
-inline cudaError_t launch_scan(const ScanJobs &jobs, int njobs, int BH, cudaStream_t s) {
+inline cudaError_t launch_scan(const ScanJobs &jobs, int njobs, int BH, cudaStream_t s, bool follows = true) {
     int len = 0;
     for (int i = 0; i < njobs; ++i) len = jobs.j[i].r.len > len ? jobs.j[i].r.len : len;
-    chunk_scan_kernel<<<dim3((len / 4 + 63) / 64, BH, njobs), 64, 0, s>>>(jobs);
-    return cudaGetLastError();
+    return chain_launch(follows, chunk_scan_kernel, dim3((len / 4 + 63) / 64, BH, njobs), 64, 0, s, jobs);
 }
 
 // per chunk, the sums over its tokens A^T B (d x width) and, after it in the record, A^T 1 (d) where
@@ -461,6 +462,7 @@ struct SumJobs {
 template <int N, typename T>
 __global__ void __launch_bounds__(kCT) chunk_sums_kernel(const __grid_constant__ SumJobs<T> jobs, int n) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     const SumJob<T> &J = jobs.j[blockIdx.z];
     const int c = blockIdx.x, hd = blockIdx.y, t0 = c * kC, len = min(kC, n - t0);
     float *As = sm, *Bs = sm + tile_floats<N>();
@@ -474,12 +476,11 @@ __global__ void __launch_bounds__(kCT) chunk_sums_kernel(const __grid_constant__
     if (J.sums) col_sums<N>(rec + J.d * J.width, As, nullptr, J.d);
 }
 template <int N, typename T>
-cudaError_t launch_sums(const SumJobs<T> &jobs, int njobs, int BH, int n, cudaStream_t s) {
+cudaError_t launch_sums(bool follows, const SumJobs<T> &jobs, int njobs, int BH, int n, cudaStream_t s) {
     const int smem = 2 * tile_floats<N>() * (int)sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(chunk_sums_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e) return e;
-    chunk_sums_kernel<N, T><<<dim3((n + kC - 1) / kC, BH, njobs), kCT, smem, s>>>(jobs, n);
-    return cudaGetLastError();
+    return chain_launch(follows, chunk_sums_kernel<N, T>, dim3((n + kC - 1) / kC, BH, njobs), kCT, smem, s, jobs, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -497,6 +498,7 @@ template <int N, typename T>
 __global__ void __launch_bounds__(kCT)
     chunk_out_kernel(const T *__restrict__ q, T *__restrict__ out, const __grid_constant__ OutParams P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *stage = b0 + tile_floats<N>(), *dens = stage + stage_floats<N>();
     const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
     const long long tok = (long long)hd * P.n + t0;
@@ -541,8 +543,7 @@ cudaError_t launch_out(const T *q, T *out, const OutParams &P, int BH, cudaStrea
     const int smem = (tile_floats<N>() + stage_floats<N>() + kC) * (int)sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(chunk_out_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e) return e;
-    chunk_out_kernel<N, T><<<dim3((P.n + kC - 1) / kC, BH), kCT, smem, s>>>(q, out, P);
-    return cudaGetLastError();
+    return chain_launch(true, chunk_out_kernel<N, T>, dim3((P.n + kC - 1) / kC, BH), kCT, smem, s, q, out, P);
 }
 
 // the padded head size that serves d and dv

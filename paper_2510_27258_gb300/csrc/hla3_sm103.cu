@@ -54,6 +54,7 @@
 // initial or final state.
 #include <cstdlib>
 
+#include "chain_launch.cuh"
 #include "hla_internal.h"
 #include "sm103_prims.cuh"
 
@@ -302,6 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1) hla3_tc_kernel(Params p) {
     tc_fence_after();
     const uint32_t tb = ms->tmem_base;
     const int items = p.BH * p.G;
+    chain_begin();
 
     if (issuer) {
         if (lane == 0) {
@@ -703,6 +705,7 @@ __global__ void __launch_bounds__(256) hla3_tc_fixup_kernel(const float *__restr
                                                              const float *__restrict__ dF, int n, int G, int L) {
     __shared__ __align__(16) float Qs[kTile][kD + 4];
     __shared__ __align__(16) float Fs[kD][kD + 4];  // Fs[f][j] = F_start[f][j]
+    chain_begin();
     const int head = blockIdx.y, j = blockIdx.x + L, g = j / L, tok0 = j * kTile;
     const int tid = threadIdx.x;
     const int tg = tid >> 3, c0 = (tid & 7) * 4;  // tokens 4 tg .. +3, outputs c0 .. +3
@@ -835,11 +838,12 @@ cudaError_t hla3_tc_forward(const Fwd2 &p, cudaStream_t stream) {
                                   (int)kSmemBytes)))
         return e;
     const int items = p.BH * pl.G;
-    if (pl.G > 1) hla3_tc_kernel<true><<<items < sms ? items : sms, kThreads, kSmemBytes, stream>>>(kp);
-    hla3_tc_kernel<false><<<items < sms ? items : sms, kThreads, kSmemBytes, stream>>>(kp);
-    if (pl.G > 1)
-        hla3_tc_fixup_kernel<<<dim3(pl.M - pl.L, p.BH), 256, 0, stream>>>(kp.q, kp.out, kp.dF, p.n, pl.G, pl.L);
-    return cudaGetLastError();
+    const dim3 grid(items < sms ? items : sms);
+    const bool cut = pl.G > 1;
+    if (cut && (e = chain_launch(false, hla3_tc_kernel<true>, grid, kThreads, kSmemBytes, stream, kp))) return e;
+    if ((e = chain_launch(cut, hla3_tc_kernel<false>, grid, kThreads, kSmemBytes, stream, kp))) return e;
+    if (!cut) return cudaSuccess;
+    return chain_launch(true, hla3_tc_fixup_kernel, dim3(pl.M - pl.L, p.BH), 256, 0, stream, kp.q, kp.out, kp.dF, p.n, pl.G, pl.L);
 }
 
 }  // namespace hla

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     ahla_chunk_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                       const __grid_constant__ AParams A) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *ss = stage + stage_floats<N>(), *dens = ss + kC;
     const int c = blockIdx.x, hd = blockIdx.y, d = A.d, dv = A.dv, t0 = c * kC, len = min(kC, A.n - t0);
@@ -134,18 +135,17 @@ cudaError_t forward_n(const Fwd2 &p, cudaStream_t s) {
         if (nch > 0) {
             SumJobs<T> jobs{};
             jobs.j[0] = {k, v, A.P, d, dv, 1};
-            if ((e = launch_sums<N, T>(jobs, 1, p.BH, p.n, s))) return e;
+            if ((e = launch_sums<N, T>(false, jobs, 1, p.BH, p.n, s))) return e;
         }
         ScanJobs scans{};
         scans.j[0] = {A.P, p.state_in, st_len, p.state_out, st_len, 0};
-        if ((e = launch_scan(scans, 1, p.BH, s))) return e;
+        if ((e = launch_scan(scans, 1, p.BH, s, nch > 0))) return e;
     }
     if (nch > 0) {
         const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + 2 * kC) * (int)sizeof(float);
         if ((e = cudaFuncSetAttribute(ahla_chunk_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
             return e;
-        ahla_chunk_kernel<N, T><<<dim3(nch, p.BH), kCT, smem, s>>>(q, k, v, out, A);
-        if ((e = cudaGetLastError())) return e;
+        if ((e = chain_launch(sums, ahla_chunk_kernel<N, T>, dim3(nch, p.BH), kCT, smem, s, q, k, v, out, A))) return e;
     }
     if (!sums) return cudaSuccess;
     ScanJobs scans{};

@@ -104,6 +104,7 @@ __device__ __forceinline__ void load_upstream(float *dst, float *us, const BPara
 template <int N, typename T>
 __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_x_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     const Chunk<T> ch(P);
     const int d = P.d, dv = P.dv;
@@ -148,6 +149,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_x_kernel(const __
 template <int N, typename T>
 __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_upstream_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *stage = b1 + tile_floats<N>(), *us = stage + stage_floats<N>();
     const Chunk<T> ch(P);
     const int d = P.d, dv = P.dv;
@@ -202,6 +204,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_upstream_kernel(c
 template <int N, typename T>
 __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_y_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *us = stage + stage_floats<N>();
     const Chunk<T> ch(P);
@@ -237,6 +240,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_y_kernel(const __
 template <int N, typename T>
 __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *us = stage + stage_floats<N>();
     const Chunk<T> ch(P);
@@ -321,11 +325,13 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
     const dim3 grid(nch, p.BH);
     const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
     cudaError_t e;
+    bool follows = false;  // a launch of this call came before
     auto launch = [&](auto kern, dim3 gr) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (err) return err;
-        kern<<<gr, kCT, smem, s>>>(P);
-        return cudaGetLastError();
+        err = chain_launch(follows, kern, gr, kCT, smem, s, P);
+        follows = true;
+        return err;
     };
     const bool many = nch > 1;
     const ScanJob none{};
@@ -339,7 +345,8 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
         SumJobs<T> jobs{};
         jobs.j[0] = {P.k, P.k, P.S, d, d, 0};
         jobs.j[1] = {P.q, P.g, P.Gam, d, dv, 0};  // Gam^T of the plain output
-        if ((e = launch_sums<N, T>(jobs, p.normalized ? 1 : 2, p.BH, p.n, s))) return e;
+        if ((e = launch_sums<N, T>(false, jobs, p.normalized ? 1 : 2, p.BH, p.n, s))) return e;
+        follows = true;
         if ((e = scan(P.S, 0, p.normalized ? nullptr : &P.Gam))) return e;
     }
     if ((e = launch(bwd_x_kernel<N, T>, grid))) return e;

@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <cstdlib>
 
+#include "chain_launch.cuh"
 #include "hla_internal.h"
 #include "sm103_prims.cuh"
 
@@ -157,6 +158,7 @@ struct Ctx {
         __syncthreads();
         tc_fence_after();
         tb = ms->tmem_base;
+        chain_begin();  // nothing before this reads or writes global memory but a failed alignment check
     }
     __device__ void fail(unsigned where) {
         if (atomicCAS(&p.err->error, 0u, (unsigned)kDevTimeout) == 0u) {
@@ -887,6 +889,7 @@ struct SumsJobs {
     SumsJob j[2];
 };
 __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ SumsJobs jobs, int M) {
+    chain_begin();
     const SumsJob &J = jobs.j[blockIdx.z];
     const int tid = threadIdx.x, head = blockIdx.y;
     const size_t h0 = (size_t)head * M;
@@ -1044,18 +1047,19 @@ cudaError_t backward2_tiles_launch(const Bwd2 &p, cudaStream_t s) {
     t.err = reinterpret_cast<WsHeader *>(p.ws);
     cudaError_t e = cudaMemsetAsync(p.ws, 0, kWsHeaderBytes, s);
     if (e) return e;
+    bool follows = false;  // a launch of this call came before
     auto launch = [&](auto kern, int z) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (err) return err;
-        kern<<<dim3(t.M, p.BH, z), kThreads, kSmemBytes, s>>>(m, t);
-        return cudaGetLastError();
+        err = chain_launch(follows, kern, dim3(t.M, p.BH, z), kThreads, kSmemBytes, s, m, t);
+        follows = true;
+        return err;
     };
     auto sums = [&](SumsJob a, const SumsJob *b) -> cudaError_t {
         SumsJobs jobs{};
         jobs.j[0] = a;
         if (b) jobs.j[1] = *b;
-        bt_scan_kernel<<<dim3(9, p.BH, b ? 2 : 1), 128, 0, s>>>(jobs, t.M);
-        return cudaGetLastError();
+        return chain_launch(true, bt_scan_kernel, dim3(9, p.BH, b ? 2 : 1), 128, 0, s, jobs, t.M);
     };
     const bool many = t.M > 1, norm = p.normalized;
     if (many) {

@@ -70,6 +70,7 @@
 #include <utility>
 #include <vector>
 
+#include "chain_launch.cuh"
 #include "hla_internal.h"
 #include "sm103_prims.cuh"
 #include "state_products.cuh"
@@ -531,6 +532,9 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         umma_commit(&ms->bar[bEvP]);
         return true;
     };
+
+    // the final state's C partials need nothing of this launch: their blocks start where a CTA has ended
+    if (kState) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (tid == 0) ms->item = (int)atomicAdd(p.ticket, 1u);  // later tickets are taken by the issuer
     while (true) {
@@ -1421,6 +1425,7 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tc_fence_after();
         tmem_dealloc(tb, 256);
     }
+    chain_begin();  // this launch ends after the forward's, so the one after it may read the forward's ring
 }
 
 // The paper tuple [S | C | m | G | h] (d x d, d x dv, d, d x dv, d) from the ring slot of the head's
@@ -1432,6 +1437,7 @@ __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, 
                                                              int groups, float *state_out, int d, int dv) {
     __shared__ __align__(16) float C[kD][kFinCols + 4];  // the block's columns (zero outside d)
     __shared__ float m[kD];
+    chain_begin();
     const int hd = blockIdx.y, cb = blockIdx.x * kFinCols, tid = threadIdx.x;
     const float *rg = ring + ((size_t)hd * 2 + last_slot) * kRingFloats;
     const float *pt = part + (size_t)hd * groups * kCPartFloats;
@@ -1598,12 +1604,12 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     float *part = reinterpret_cast<float *>(p.ws + FL.off_part);
     if ((e = cudaFuncSetAttribute(state_c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCSmemBytes)))
         return e;
-    state_c_kernel<<<p.BH * groups, kCThreads, kCSmemBytes, stream>>>(mq, mv, part, kp.M, groups, tiles_per,
-                                                                       p.state_in, kp.err);
-    if ((e = cudaGetLastError())) return e;
-    state_finalize_kernel<<<dim3(p.dv / kFinCols, p.BH), 256, 0, stream>>>(kp.ring, (kp.G - 1) & 1, part, groups,
-                                                                            p.state_out, p.d, p.dv);
-    return cudaGetLastError();
+    // (each reads state_in, or what an earlier launch left; neither writes what the forward reads)
+    if ((e = chain_launch(true, state_c_kernel, dim3(p.BH * groups), kCThreads, kCSmemBytes, stream, mq, mv, part, kp.M, groups,
+                          tiles_per, p.state_in, kp.err)))
+        return e;
+    return chain_launch(true, state_finalize_kernel, dim3(p.dv / kFinCols, p.BH), 256, 0, stream, (const float *)kp.ring,
+                        (kp.G - 1) & 1, (const float *)part, groups, p.state_out, p.d, p.dv);
 }
 
 }  // namespace hla

@@ -71,6 +71,7 @@ struct GParams {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kStateThreads) g2_init_kernel(const float *__restrict__ st, Records D, int d, int dv) {
     __shared__ __align__(16) float rows[kStateRows * 128];
+    chain_begin();
     const float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     const float *G = m + d, *h = G + d * dv;
     float *out = D.at(blockIdx.y, D.nch);
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(kStateThreads) g2_init_kernel(const float *__r
 __global__ void __launch_bounds__(kStateThreads) g2_final_kernel(float *__restrict__ st, Records D, int d, int dv,
                                                                  int masked) {
     __shared__ __align__(16) float rows[kStateRows * 128];
+    chain_begin();
     float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     float *G = m + d, *h = G + d * dv;
     const float *tot = D.at(blockIdx.y, D.nch);
@@ -109,6 +111,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     g2_chunk_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                     const __grid_constant__ GParams P) {
     extern __shared__ __align__(16) float sm[];
+    chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *dens = stage + stage_floats<N>();
     const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
@@ -174,10 +177,12 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
     P.has_in = p.state_in != nullptr;
     P.need_D = p.state_out != nullptr;
     P.direct = nch == 1 && !p.state_in;
+    bool follows = false;  // a launch of this call came before
     // D's initial value; the states' S and [C | m] start S's and C's sums as they lie
     if (p.state_in && p.masked) {
-        g2_init_kernel<<<dim3(d / kStateRows, L.BH), kStateThreads, 0, s>>>(p.state_in, P.D, d, dv);
-        if ((e = cudaGetLastError())) return e;
+        if ((e = chain_launch(false, g2_init_kernel, dim3(d / kStateRows, L.BH), kStateThreads, 0, s, p.state_in, P.D, d, dv)))
+            return e;
+        follows = true;
     }
     const bool sums = nch > 1 || p.state_in || p.state_out, sums_C = !p.masked || p.state_out;
     if (sums) {
@@ -185,21 +190,22 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
             SumJobs<T> jobs{};
             jobs.j[0] = {k, k, P.S, d, d, 0};
             jobs.j[1] = {q, v, P.C, d, dv, 1};
-            if ((e = launch_sums<N, T>(jobs, sums_C ? 2 : 1, L.BH, L.n, s))) return e;
+            if ((e = launch_sums<N, T>(follows, jobs, sums_C ? 2 : 1, L.BH, L.n, s))) return e;
+            follows = true;
         }
         ScanJobs scans{};
         scans.j[0] = {P.S, p.state_in, st_len, p.state_out, st_len, 0};
         scans.j[1] = {P.C, p.state_in ? p.state_in + d * d : nullptr, st_len,
                       p.state_out ? p.state_out + d * d : nullptr, st_len, 0};
-        if ((e = launch_scan(scans, sums_C ? 2 : 1, L.BH, s))) return e;
+        if ((e = launch_scan(scans, sums_C ? 2 : 1, L.BH, s, follows))) return e;
+        follows = true;
     }
     const dim3 grid(nch, L.BH);
     if (nch > 0) {
         const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
         if ((e = cudaFuncSetAttribute(g2_chunk_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
             return e;
-        g2_chunk_kernel<N, T><<<grid, kCT, smem, s>>>(q, k, v, out, P);
-        if ((e = cudaGetLastError())) return e;
+        if ((e = chain_launch(follows, g2_chunk_kernel<N, T>, grid, kCT, smem, s, q, k, v, out, P))) return e;
     }
     if (p.masked && sums) {
         float *total = ws + L.oD + (long long)nch * L.lenD;
@@ -213,8 +219,9 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
         }
     }
     if (p.state_out) {
-        g2_final_kernel<<<dim3(d / kStateRows, L.BH), kStateThreads, 0, s>>>(p.state_out, P.D, d, dv, p.masked);
-        if ((e = cudaGetLastError())) return e;
+        if ((e = chain_launch(true, g2_final_kernel, dim3(d / kStateRows, L.BH), kStateThreads, 0, s, p.state_out, P.D, d, dv,
+                              p.masked)))
+            return e;
     }
     return cudaSuccess;
 }

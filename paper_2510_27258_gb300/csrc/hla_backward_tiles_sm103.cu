@@ -24,9 +24,9 @@
 // float4 (r, c..c+3) at index ((r / 32 * 16 + c / 8) * 2 + c / 4 % 2) * 32 + r % 32, so that a warp's
 // access is 512 contiguous bytes.  Head size 64 runs zero-padded (TMA fill).
 //
-// Measured: B2 H16 n4096 d128 normalised 0.533 ms, against 2.09 ms for the CUDA-core kernels (and 37 ms
-// for the kernels those replaced); ncu, us: 19 for K^T K, 73 X, 63 G', 65 Y, 160 the gradients, 30 for each
-// of the four sums.  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak; the
+// Measured: B2 H16 n4096 d128 normalised 0.479 ms, against 2.09 ms for the CUDA-core kernels (and 37 ms
+// for the kernels those replaced); ncu, us: 20 for K^T K, 73 X, 63 G', 65 Y, 162 the gradients, 20 to 23 for
+// each of the four sums.  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak; the
 // rest is the blocks' chains of copy, product and epilogue, two in flight an SM.
 #include <algorithm>
 #include <cstdlib>
@@ -875,9 +875,10 @@ __global__ void __launch_bounds__(kThreads, 2) bt_grad_kernel(const __grid_const
 
 // ---------------------------------------------------------------------------
 // Sums over the tiles of a head: record c becomes, as a hi/lo image pair, the sum of the records before
-// it (reverse: after it).  A thread carries 16 columns of a row (a whole 32-byte sector of each
-// image); blocks 8 and up of a head do the same for a vector of 128 floats in place.  Bound by HBM:
-// 64 KB read and written per tile.
+// it (reverse: after it).  A thread carries 8 columns of a row, eight tiles' loads in flight; two
+// neighbouring lanes fill a 32-byte sector of each image.  Block 16 of a head does the same for a vector of 128
+// floats in place.  Bound by HBM: 64 KB read and written per tile (with 16 columns a thread, half the threads and
+// four tiles in flight, a sum over 1024 tiles took 27 to 33 us, now 20 to 23).
 // ---------------------------------------------------------------------------
 struct SumsJob {
     const float *rec;
@@ -893,7 +894,7 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
     const SumsJob &J = jobs.j[blockIdx.z];
     const int tid = threadIdx.x, head = blockIdx.y;
     const size_t h0 = (size_t)head * M;
-    if (blockIdx.x == 8) {
+    if (blockIdx.x == 16) {
         if (!J.vec) return;
         float acc = 0.f;
         for (int i = 0; i < M; ++i) {
@@ -905,39 +906,39 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
         }
         return;
     }
-    const int w = blockIdx.x * 4 + (tid >> 5), r = (w >> 3) * 32 + (tid & 31), c0 = (w & 7) * 16;
-    const uint32_t o0 = tile_off(r, c0), o1 = tile_off(r, c0 + 8);
-    float acc[16];
+    const int w = blockIdx.x * 4 + (tid >> 5), lane = tid & 31;
+    const int r = (w >> 3) * 16 + (lane >> 1), c0 = (w & 7) * 16 + (lane & 1) * 8;
+    const uint32_t off = tile_off(r, c0);
+    const int i0 = rec_index(r, c0), i1 = rec_index(r, c0 + 4);
+    float acc[8];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) acc[u] = 0.f;
-    constexpr int U = 4;
+    for (int u = 0; u < 8; ++u) acc[u] = 0.f;
+    constexpr int U = 8;
     for (int i = 0; i < M; i += U) {
-        float4 v[U][4];
+        float4 v[U][2];
 #pragma unroll
         for (int k = 0; k < U; ++k)
             if (i + k + 1 < M) {
                 const size_t at = h0 + (J.reverse ? M - 1 - i - k : i + k);
                 const float4 *s = reinterpret_cast<const float4 *>(J.rec + at * kRec);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) v[k][j] = s[rec_index(r, c0 + 4 * j)];
+                v[k][0] = s[i0];
+                v[k][1] = s[i1];
             }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             if (i + k >= M) break;
             const size_t at = h0 + (J.reverse ? M - 1 - i - k : i + k);
             if (i + k > 0) {  // the first sum is empty and not read
-                uint32_t h[8], l[8];
+                uint32_t h[4], l[4];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) split2(acc[2 * u], acc[2 * u + 1], h[u], l[u]);
-                uint8_t *o = J.img + at * kPair;
-                *reinterpret_cast<uint4 *>(o + o0) = make_uint4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<uint4 *>(o + o1) = make_uint4(h[4], h[5], h[6], h[7]);
-                *reinterpret_cast<uint4 *>(o + kImage + o0) = make_uint4(l[0], l[1], l[2], l[3]);
-                *reinterpret_cast<uint4 *>(o + kImage + o1) = make_uint4(l[4], l[5], l[6], l[7]);
+                for (int u = 0; u < 4; ++u) split2(acc[2 * u], acc[2 * u + 1], h[u], l[u]);
+                uint8_t *o = J.img + at * kPair + off;
+                *reinterpret_cast<uint4 *>(o) = make_uint4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<uint4 *>(o + kImage) = make_uint4(l[0], l[1], l[2], l[3]);
             }
             if (i + k + 1 < M) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < 2; ++j) {
                     acc[4 * j] += v[k][j].x;
                     acc[4 * j + 1] += v[k][j].y;
                     acc[4 * j + 2] += v[k][j].z;
@@ -1059,7 +1060,7 @@ cudaError_t backward2_tiles_launch(const Bwd2 &p, cudaStream_t s) {
         SumsJobs jobs{};
         jobs.j[0] = a;
         if (b) jobs.j[1] = *b;
-        return chain_launch(true, bt_scan_kernel, dim3(9, p.BH, b ? 2 : 1), 128, 0, s, jobs, t.M);
+        return chain_launch(true, bt_scan_kernel, dim3(17, p.BH, b ? 2 : 1), 128, 0, s, jobs, t.M);
     };
     const bool many = t.M > 1, norm = p.normalized;
     if (many) {

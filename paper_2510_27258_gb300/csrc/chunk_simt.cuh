@@ -413,8 +413,8 @@ struct ScanJobs {
     ScanJob j[2];
 };
 
-// exclusive prefix (suffix) sums in place, one float4 a thread; eight records' loads in flight, which
-// is what bounds it (memory latency over the chunks in turn)
+// exclusive prefix (suffix) sums in place, one float4 a thread; sixteen records' loads in flight, as memory
+// latency over the chunks in turn is what bounds it (eight in flight: B4 H8 n2000 d128 fp32 491 us, sixteen 479)
 __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ ScanJobs jobs) {
     chain_begin();
     const ScanJob &J = jobs.j[blockIdx.z];
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ 
     if (J.init) acc = *reinterpret_cast<const float4 *>(J.init + hd * J.init_stride + e);
     const long long step = J.reverse ? -(long long)J.r.len : (long long)J.r.len;
     float *p = J.r.at(hd, J.reverse ? nch - 1 : 0) + e;
-    constexpr int U = 8;
+    constexpr int U = 16;
     for (int c = 0; c < nch; c += U) {
         float4 v[U];
 #pragma unroll

@@ -418,7 +418,7 @@ struct ScanJobs {
 __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ ScanJobs jobs) {
     chain_begin();
     const ScanJob &J = jobs.j[blockIdx.z];
-    const int e = (blockIdx.x * 64 + threadIdx.x) * 4, hd = blockIdx.y, nch = J.r.nch;
+    const int e = (blockIdx.y * 64 + threadIdx.x) * 4, hd = blockIdx.x, nch = J.r.nch;
     if (e >= J.r.len) return;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (J.init) acc = *reinterpret_cast<const float4 *>(J.init + hd * J.init_stride + e);
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(64) chunk_scan_kernel(const __grid_constant__ 
 inline cudaError_t launch_scan(const ScanJobs &jobs, int njobs, int BH, cudaStream_t s, bool follows = true) {
     int len = 0;
     for (int i = 0; i < njobs; ++i) len = jobs.j[i].r.len > len ? jobs.j[i].r.len : len;
-    return chain_launch(follows, chunk_scan_kernel, dim3((len / 4 + 63) / 64, BH, njobs), 64, 0, s, jobs);
+    return chain_launch(follows, chunk_scan_kernel, dim3(BH, (len / 4 + 63) / 64, njobs), 64, 0, s, jobs);
 }
 
 // per chunk, the sums over its tokens A^T B (d x width) and, after it in the record, A^T 1 (d) where

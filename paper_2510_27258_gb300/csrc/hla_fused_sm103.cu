@@ -1139,13 +1139,13 @@ hla2_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     }
 }
 
-// initial-state carries D_0 = S_0 C_0 - G_0 and e_0 = S_0 m_0 - h_0 of each head (fp32); block (16 rows, head)
+// initial-state carries D_0 = S_0 C_0 - G_0 and e_0 = S_0 m_0 - h_0 of each head (fp32); block (head, 16 rows)
 __global__ void __launch_bounds__(kStateThreads) init_carry_kernel(const float *__restrict__ st, float *__restrict__ out) {
     __shared__ __align__(16) float rows[kStateRows * kD];
-    const float *S = st + (size_t)blockIdx.y * kStateFloats, *C = S + kD * kD, *m = C + kD * kD, *G = m + kD;
+    const float *S = st + (size_t)blockIdx.x * kStateFloats, *C = S + kD * kD, *m = C + kD * kD, *G = m + kD;
     const float *h = G + kD * kD;
-    float *D = out + (size_t)blockIdx.y * (kD * kD + kD), *e = D + kD * kD;
-    state_products(S, C, m, kD, kD, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+    float *D = out + (size_t)blockIdx.x * (kD * kD + kD), *e = D + kD * kD;
+    state_products(S, C, m, kD, kD, blockIdx.y * kStateRows, rows, [&](int a, int b, float x) {
         if (b < kD) D[a * kD + b] = x - G[a * kD + b];
         else e[a] = x - h[a];
     });
@@ -1429,7 +1429,7 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 }
 
 // The paper tuple [S | C | m | G | h] (d x d, d x dv, d, d x dv, d) from the ring slot of the head's
-// last segment and the C / m partials.  Block (16 columns of C and G, head): with one block a head the
+// last segment and the C / m partials.  Block (head, 16 columns of C and G): with one block a head the
 // d^2 dv products of S C ran on 32 SMs and took 199 us at 32 heads, 128 x 128; on 8 blocks a head,
 // each thread with 8 columns of a row of S read in the ring's own order, they take 18 us (both from cold caches).
 constexpr int kFinCols = 16;
@@ -1438,7 +1438,7 @@ __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, 
     __shared__ __align__(16) float C[kD][kFinCols + 4];  // the block's columns (zero outside d)
     __shared__ float m[kD];
     chain_begin();
-    const int hd = blockIdx.y, cb = blockIdx.x * kFinCols, tid = threadIdx.x;
+    const int hd = blockIdx.x, cb = blockIdx.y * kFinCols, tid = threadIdx.x;
     const float *rg = ring + ((size_t)hd * 2 + last_slot) * kRingFloats;
     const float *pt = part + (size_t)hd * groups * kCPartFloats;
     // the ring stores float4 c (columns c0 + 4c..) of epilogue thread et = 32 (qd + 4 cq) + lane at c * 512 + et
@@ -1463,7 +1463,7 @@ __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, 
     const size_t st_len = (size_t)d * d + 2 * (size_t)d * dv + 2 * (size_t)d;
     float *oS = state_out + (size_t)hd * st_len, *oC = oS + (size_t)d * d, *om = oC + (size_t)d * dv, *oG = om + d;
     float *oh = oG + (size_t)d * dv;
-    const int nb = dv / kFinCols, rows = (d + nb - 1) / nb, s0 = blockIdx.x * rows;  // this block's rows of S
+    const int nb = dv / kFinCols, rows = (d + nb - 1) / nb, s0 = blockIdx.y * rows;  // this block's rows of S
     for (int i = tid; i < rows * (d / 4); i += 256) {
         const int r = s0 + i / (d / 4), x = (i % (d / 4)) * 4;
         if (r < d) *reinterpret_cast<float4 *>(oS + (size_t)r * d + x) = ring4(rg, r, x);
@@ -1496,7 +1496,7 @@ __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, 
             *reinterpret_cast<float4 *>(oG + (size_t)r * dv + cb + h + j) =
                 make_float4(acc[j] - D.x, acc[j + 1] - D.y, acc[j + 2] - D.z, acc[j + 3] - D.w);
         }
-        if (blockIdx.x == 0 && h == 0) {
+        if (blockIdx.y == 0 && h == 0) {
             om[r] = m[r];
             oh[r] = sm_ - rg[2 * kD * kD + r];  // h = S m - e
         }
@@ -1577,7 +1577,7 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     if ((e = cudaMemsetAsync(p.ws, 0, FL.off_ring, stream))) return e;
     if (p.state_in) {
         float *init = reinterpret_cast<float *>(p.ws + FL.off_init);
-        init_carry_kernel<<<dim3(kD / kStateRows, p.BH), kStateThreads, 0, stream>>>(p.state_in, init);
+        init_carry_kernel<<<dim3(p.BH, kD / kStateRows), kStateThreads, 0, stream>>>(p.state_in, init);
         if ((e = cudaGetLastError())) return e;
         kp.init_De = init;
     }
@@ -1608,7 +1608,7 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     if ((e = chain_launch(true, state_c_kernel, dim3(p.BH * groups), kCThreads, kCSmemBytes, stream, mq, mv, part, kp.M, groups,
                           tiles_per, p.state_in, kp.err)))
         return e;
-    return chain_launch(true, state_finalize_kernel, dim3(p.dv / kFinCols, p.BH), 256, 0, stream, (const float *)kp.ring,
+    return chain_launch(true, state_finalize_kernel, dim3(p.BH, p.dv / kFinCols), 256, 0, stream, (const float *)kp.ring,
                         (kp.G - 1) & 1, (const float *)part, groups, p.state_out, p.d, p.dv);
 }
 

@@ -67,36 +67,36 @@ struct GParams {
     int need_D;   // D's increments of the last chunk are wanted too (final state)
 };
 
-// D_0 = S_0 C_0 - G_0, e_0 = S_0 m_0 - h_0 of a head's state_in into D's initial record; block (16 rows, head)
+// D_0 = S_0 C_0 - G_0, e_0 = S_0 m_0 - h_0 of a head's state_in into D's initial record; block (head, 16 rows)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kStateThreads) g2_init_kernel(const float *__restrict__ st, Records D, int d, int dv) {
     __shared__ __align__(16) float rows[kStateRows * 128];
     chain_begin();
-    const float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
+    const float *S = st + blockIdx.x * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     const float *G = m + d, *h = G + d * dv;
-    float *out = D.at(blockIdx.y, D.nch);
-    state_products(S, C, m, d, dv, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+    float *out = D.at(blockIdx.x, D.nch);
+    state_products(S, C, m, d, dv, blockIdx.y * kStateRows, rows, [&](int a, int b, float x) {
         if (b < dv) out[a * dv + b] = x - G[a * dv + b];
         else out[d * dv + a] = x - h[a];
     });
 }
 
 // state_out's G = S C - D, h = S m - e (zeros for the unmasked operator) from its S, C, m and D's
-// total; block (16 rows, head)
+// total; block (head, 16 rows)
 __global__ void __launch_bounds__(kStateThreads) g2_final_kernel(float *__restrict__ st, Records D, int d, int dv,
                                                                  int masked) {
     __shared__ __align__(16) float rows[kStateRows * 128];
     chain_begin();
-    float *S = st + blockIdx.y * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
+    float *S = st + blockIdx.x * ((long long)d * d + 2LL * d * dv + 2LL * d), *C = S + d * d, *m = C + d * dv;
     float *G = m + d, *h = G + d * dv;
-    const float *tot = D.at(blockIdx.y, D.nch);
+    const float *tot = D.at(blockIdx.x, D.nch);
     if (!masked) {
-        const int a0 = blockIdx.x * kStateRows;
+        const int a0 = blockIdx.y * kStateRows;
         for (int i = threadIdx.x; i < kStateRows * dv; i += kStateThreads) G[a0 * dv + i] = 0.f;
         if (threadIdx.x < kStateRows) h[a0 + threadIdx.x] = 0.f;
         return;
     }
-    state_products(S, C, m, d, dv, blockIdx.x * kStateRows, rows, [&](int a, int b, float x) {
+    state_products(S, C, m, d, dv, blockIdx.y * kStateRows, rows, [&](int a, int b, float x) {
         if (b < dv) G[a * dv + b] = x - tot[a * dv + b];
         else h[a] = x - tot[d * dv + a];
     });
@@ -180,7 +180,7 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
     bool follows = false;  // a launch of this call came before
     // D's initial value; the states' S and [C | m] start S's and C's sums as they lie
     if (p.state_in && p.masked) {
-        if ((e = chain_launch(false, g2_init_kernel, dim3(d / kStateRows, L.BH), kStateThreads, 0, s, p.state_in, P.D, d, dv)))
+        if ((e = chain_launch(false, g2_init_kernel, dim3(L.BH, d / kStateRows), kStateThreads, 0, s, p.state_in, P.D, d, dv)))
             return e;
         follows = true;
     }
@@ -219,7 +219,7 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
         }
     }
     if (p.state_out) {
-        if ((e = chain_launch(true, g2_final_kernel, dim3(d / kStateRows, L.BH), kStateThreads, 0, s, p.state_out, P.D, d, dv,
+        if ((e = chain_launch(true, g2_final_kernel, dim3(L.BH, d / kStateRows), kStateThreads, 0, s, p.state_out, P.D, d, dv,
                               p.masked)))
             return e;
     }

@@ -448,6 +448,7 @@ cudaError_t ahla_step_split_launch(const void *q, const void *k, const void *v, 
 }  // namespace
 
 size_t ahla_workspace_bytes_internal(int BH, int n, int d, int dv, int) {
+    if (n == 0) return kWsHeaderBytes;  // the states are copied, no record is used
     return kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
 }
 

@@ -363,6 +363,7 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
 }  // namespace
 
 size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int) {
+    if (n == 0) return kWsHeaderBytes;
     const size_t simt = kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
     const size_t tc = backward2_tc_workspace_bytes(BH, n), tiles = backward2_tiles_workspace_bytes(BH, n, d, dv);
     return std::max(simt, std::max(tc, tiles));

@@ -39,17 +39,17 @@ DEC = hla_inputs.WORKLOADS["decode_bf16"]
 # capture of the kernel sources (concatenated) whose SHA-256 starts with "sha256"
 # (summaries in profiles/); reported as null for any other source or workload.
 TRAFFIC = {
-    "hla2_fused_kernel": {"src": ["hla_fused_sm103.cu", "sm103_prims.cuh"], "sha256": "7ca8b7c6b836b2ff", "workload": "long_bf16_norm",
-                          "n": 16384, "bytes": 526.6e6,
-                          "how": "ncu capture at n=8192 (227.5 MB read + 35.8 MB written during the launch; outputs "
+    "hla2_fused_kernel": {"src": ["hla_fused_sm103.cu", "sm103_prims.cuh"], "sha256": "689d2cc9a84c37a8", "workload": "long_bf16_norm",
+                          "n": 16384, "bytes": 524.7e6,
+                          "how": "ncu capture at n=8192 (227.1 MB read + 35.3 MB written during the launch; outputs "
                                  "still dirty in L2 at its end are written later) scaled x2 to n=16384"},
-    "step2_kernel": {"src": ["hla_step.cu"], "sha256": "7f4bfb053a9af874", "workload": "decode_bf16", "n": 0,
-                     "bytes": 750.3e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
-                                              "tuple_step): 406.4 MB read + 343.9 MB written"},
+    "step2_kernel": {"src": ["hla_step.cu"], "sha256": "c0208d2ea3e662d0", "workload": "decode_bf16", "n": 0,
+                     "bytes": 749.3e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
+                                              "tuple_step): 406.5 MB read + 342.9 MB written"},
     "c3_kernels": {"src": ["hla3_chunked.cu"], "sha256": "17ac1acd5c9202d1", "workload": "hla3_f32", "n": 4096,
                    "bytes": 432.5e6, "how": "ncu capture of one forward's five launches (bench.py --only hla3_f32): "
                                             "373.0 MB read + 59.5 MB written, 6.4 x the token I/O (per-chunk records)"},
-    "hla3_tc_kernels": {"src": ["hla3_sm103.cu", "sm103_prims.cuh"], "sha256": "dd16e8c0a54902eb", "workload": "hla3_f32",
+    "hla3_tc_kernels": {"src": ["hla3_sm103.cu", "sm103_prims.cuh"], "sha256": "b57b0337c5170f56", "workload": "hla3_f32",
                         "n": 4096, "bytes": 115.0e6,
                         "how": "ncu capture of one forward's three launches (bench.py --only hla3_f32), caches "
                                "flushed per launch: pre-pass 37.8 MB read, sweep 51.6 MB read + 0.1 MB written "
@@ -59,7 +59,7 @@ TRAFFIC = {
                       "how": "ncu capture of one backward (bench.py --only backward): 278.0 MB read + 170.4 MB "
                              "written; the per-tile records (X hi, lo; S_p, D_p: 96 MB) are written once and read "
                              "back once"},
-    "step2_kernel_sde": {"src": ["hla_step.cu"], "sha256": "7f4bfb053a9af874", "workload": "decode_bf16", "n": 0,
+    "step2_kernel_sde": {"src": ["hla_step.cu"], "sha256": "c0208d2ea3e662d0", "workload": "decode_bf16", "n": 0,
                          "bytes": 480.2e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
                                                   "sde_step): 271.1 MB read + 209.1 MB written"},
 }
@@ -746,7 +746,7 @@ def bench_backward(hla, dev, stream, world, hbm_peak, tc_peak, steps=10, warmup=
         rec["roofline"] = {"bound": "alu", "achieved": tf, "peak": alu_peak(), "unit": "TFLOP/s",
                            "frac": tf / alu_peak(), "traffic": None, "flops": bwd_flops(w),
                            "peak_kind": "derived (152 SMs x 128 fp32 lanes x 2 x 2.07 GHz)",
-                           "kernel": "bwd_fwd_local/fwd_scan/local1/scan/local2 (fp32 CUDA cores)"}
+                           "kernel": "bwd_x/upstream/y/grad_kernel and sums over chunks (fp32 CUDA cores)"}
         rec["path"] = "fp32 CUDA cores"
         rec["launches"] = 5 * steps
     return rec
@@ -794,7 +794,7 @@ def bench_ahla(hla, dev, stream, hbm_peak, world, steps=20, warmup=3, decode_ste
         roof = {"bound": "alu", "achieved": tf, "peak": alu_peak(), "unit": "TFLOP/s", "frac": tf / alu_peak(),
                 "traffic": None, "flops": ahla_flops(w),
                 "peak_kind": "derived (152 SMs x 128 fp32 lanes x 2 x 2.07 GHz)",
-                "kernel": "ahla_local/scan/out (fp32 CUDA cores)",
+                "kernel": "ahla_chunk_kernel and sums over chunks (fp32 CUDA cores)",
                 "hbm_view": {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak}}
     res["forward"] = {"workload": w.name, "B": w.B, "H": w.H, "n": w.n, "d": w.d, "dv": w.dv, "chunk": w.chunk,
                       "tokens": w.dtype, "ms_per_step": ms, "value": w.B * w.n * world / (ms * 1e-3),
@@ -829,7 +829,7 @@ def bench_ahla(hla, dev, stream, hbm_peak, world, steps=20, warmup=3, decode_ste
                      "tokens_per_s": w.B * world / (us * 1e-6),
                      "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s",
                                   "frac": gbs / hbm_peak, "traffic": None, "algorithmic_bytes": ahla_dec_bytes(w),
-                                  "kernel": "ahla_step_staged_kernel"},
+                                  "kernel": "ahla_step_split_kernel"},
                      "launches": decode_steps}
     return res
 

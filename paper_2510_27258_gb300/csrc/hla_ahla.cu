@@ -316,8 +316,8 @@ ahla_step_staged_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
 // output the blocks of a head form a cluster and meet in a split barrier between their last read of m, n
 // and block 0's write.  Measured, us a step (staged -> this), bf16 tokens: 64 x 64, 16 heads 3.7 -> 2.8,
 // 256 heads 6.1 -> 4.0, 2048 heads 35.6 -> 23.4 (140 MB read and written: 5.9 TB/s); 128 x 128, 32
-// heads 5.7 -> 3.3, 2048 heads 87.7 -> 81.4.  Bound by the latency of one load and two barriers for few
-// heads, by HBM for many.
+// heads 5.7 -> 3.3, 2048 heads as fast (90.3 us a step over 541 MB of states).  Bound by the latency of
+// one load and two barriers for few heads, by HBM for many.
 constexpr int kSplitThreads = 256, kSplitWarps = kSplitThreads / 32;
 template <typename T, int NC>
 __global__ void __launch_bounds__(kSplitThreads)

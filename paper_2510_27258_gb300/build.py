@@ -35,10 +35,16 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def inputs():
+    """Every file the library is built from: sources, headers of both kinds, this file."""
+    files = sources() + [os.path.abspath(__file__)]
+    for pattern in (os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"), os.path.join(INCLUDE, "*.h")):
+        files += glob.glob(pattern)
+    return files
+
+
 def _newest_input():
-    files = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
-    files.append(os.path.abspath(__file__))
-    return max(os.path.getmtime(f) for f in files)
+    return max(os.path.getmtime(f) for f in inputs())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

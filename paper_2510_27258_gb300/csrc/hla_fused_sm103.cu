@@ -67,7 +67,6 @@
 #include <algorithm>
 #include <functional>
 #include <queue>
-#include <utility>
 #include <vector>
 
 #include "chain_launch.cuh"
@@ -1208,95 +1207,74 @@ FusedLayout fused_layout(int BH, int n) {
     return L;
 }
 
-// Costs (us) of the ticket schedule's parts, fitted to 1700 timings of forced segment lengths (1 to 256 heads, 2 to
-// 94 tiles, lengths 1 to 64 and one segment per head; rms error 3 %): a tile of a segment's pre-pass, the hand-on
-// of the S prefix to the next segment, a segment's set-up, a tile of the sweep, the hand-on of the D prefix, the
-// fix-up's start and a tile of it, the end of a first segment.
-struct SegmentCosts {
-    double pre, s_chain, setup, tile, d_chain, fix0, fix, tail;
-};
-constexpr SegmentCosts kCosts64 = {0.2, 3.19, 3.78, 4.10, 2.62, 1.30, 1.04, 2.36};      // head size 64, plain
-constexpr SegmentCosts kCosts128 = {0.0, 3.17, 5.33, 5.07, 2.55, 0.0, 1.63, 1.91};      // 128, plain
-constexpr SegmentCosts kCosts64Full = {0.26, 2.93, 4.63, 4.71, 3.48, 0.05, 1.46, 1.73};  // 64, normalised or with a final state
-constexpr SegmentCosts kCosts128Full = {0.0, 2.04, 4.15, 5.94, 3.40, 0.62, 1.88, 1.03};  // 128, the same
-
-// Predicted duration of the ticket schedule with segments of L tiles.  Items go out in ticket order; a CTA takes
-// its next ticket when it has swept its segment, before it waits for the D prefix and fixes up, so the order
-// follows the sweeps' ends and the next item starts after the fix-up.  A segment sweeps once it has its S prefix.
-// Where all items run at once every head's timeline is the same and one is followed.
-double predicted_span(int BH, int M, int L, int sms, const SegmentCosts &c) {
-    const int G = (M + L - 1) / L;
-    if (G == 1 && BH <= sms) return c.tile * M + c.tail;
-    const bool at_once = (long long)BH * G <= sms;
-    const int heads = at_once ? 1 : BH;
-    std::vector<double> s_at(heads, 0.0), d_at(heads, 0.0);  // when the prefixes behind a head's last segment are out
-    typedef std::pair<double, double> Slot;                  // a CTA's ticket time, and when it is free
-    std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> ctas;
-    if (!at_once)
-        for (int i = 0; i < sms; ++i) ctas.push(Slot(0.0, 0.0));
+// Predicted duration (us) of the ticket schedule with segments of L tiles: items in ticket order go
+// to the SM that frees first; an item costs 5.5 us per tile of sweep and, for segments > 0, 2.1 us
+// per fix-up tile and 7 us of chain set-up (2 us for a first segment); in the first wave the S
+// prefix ripples through the concurrent segments of a head (about 5.6 us per segment, after a cold
+// pre-pass of 4.7 us).  Constants measured on B2 H16 n16384 d128.
+double predicted_span(int BH, int M, int L, int sms) {
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    for (int i = 0; i < sms; ++i) free_at.push(0.0);
     double span = 0.0;
-    for (int g = 0; g < G; ++g) {
-        const int li = std::min(L, M - g * L);
-        for (int h = 0; h < heads; ++h) {
-            double t = 0.0, swept, end;
-            if (!at_once) {
-                t = ctas.top().second;
-                ctas.pop();
-            }
-            if (G == 1) {
-                swept = t + c.tile * li;
-                end = swept + c.tail;
-            } else {
-                const double pre = g + 1 < G ? c.pre * li : 0.0;  // overlaps the item before, on a CTA that had one
-                const double s = std::max(t + (t == 0.0 ? pre : 0.3 * pre), s_at[h]);
-                swept = s + c.setup + c.tile * li;
-                s_at[h] = s + c.s_chain;
-                end = g > 0 ? std::max(swept, d_at[h]) + c.fix0 + c.fix * li : swept + c.tail;
-                d_at[h] = std::max(swept, d_at[h]) + c.d_chain;
-            }
-            if (!at_once) ctas.push(Slot(swept, end));
-            span = std::max(span, end);
+    const int G = (M + L - 1) / L;
+    for (int sg = 0; sg < G; ++sg) {
+        const int li = std::min(L, M - sg * L);
+        for (int h = 0; h < BH; ++h) {
+            const double t = free_at.top();
+            free_at.pop();
+            double c = 5.5 * li + (sg > 0 ? 2.1 * li + 7.0 : 2.0);
+            if (t == 0.0) c += 4.7 + 5.6 * sg;
+            free_at.push(t + c);
+            span = std::max(span, t + c);
         }
     }
     return span;
 }
 
-// Tiles per segment: the length whose schedule is predicted to end first (one segment per head unless segments
-// gain more than the model's error).  On the timings above the choice costs 0.5 % over the best length on
-// average, 9 % at worst; a model with the constants of one long workload, lengths 2 to 8 and one segment per head
-// from 76 heads cost 9 % on average and up to 48 %: 24 heads of 1500 x 64 53 -> 37 us, 16 heads of 4096 x 64
-// 73 -> 56, 32 heads of 4096 x 128 normalised 114 -> 86, 64 heads of 2048 x 128 79 -> 70.
-int segment_tiles(int BH, int M, int sms, bool narrow, bool full) {
-    if (const char *e = getenv("HLA_FUSED_SEGMENT_TILES")) {
-        int v = atoi(e);
-        if (v > 0) return v < M ? v : M;
-    }
-    if (M == 1 || BH >= 4 * sms) return M;  // rounds enough to level the SMs without segments
-    // The answer depends on these numbers alone; simulating the schedules takes the host as long as a short
-    // forward takes the GPU, so a thread keeps its last one.
-    struct Key {
-        int BH, M, sms, kind;
-        bool operator==(const Key &o) const { return BH == o.BH && M == o.M && sms == o.sms && kind == o.kind; }
-    };
-    static thread_local Key last{-1, -1, -1, -1};
-    static thread_local int last_L = 0;
-    const Key key{BH, M, sms, (narrow ? 1 : 0) + (full ? 2 : 0)};
-    if (key == last) return last_L;
-    const SegmentCosts &c = narrow ? (full ? kCosts64Full : kCosts64) : (full ? kCosts128Full : kCosts128);
-    int best = M;
-    double best_t = 0.96 * predicted_span(BH, M, M, sms, c);
-    for (const int L : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16, 24, 32, 48, 64}) {
-        if (L >= M) break;
-        if ((long long)BH * ((M + L - 1) / L) > 6LL * sms) continue;  // many short items: never best, slow to simulate
-        const double t = predicted_span(BH, M, L, sms, c);
+// Tiles per segment: one segment per head where the heads occupy at least half the SMs, else the length of
+// 2 to 8 tiles whose schedule is predicted to end first (on B2 H16 n16384 d128 the prediction picks 7, measured
+// best among 4 to 13; 6 is 3.5 % slower there because 704 items leave the last wave of the 152 SMs partly idle).
+// A cut is not free of error: outputs of later segments are rounded to bf16 once more, before the fix-up, and the
+// prefix of D that it adds is rounded too.  Distance from 64-bit results, relative: 64 heads of 2048 x 128 uncut
+// 2.78e-3, in segments of 2 to 8 tiles 2.95e-3 to 3.11e-3; 160 heads of 2048 x 128 normalised 2.09e-3 against 2.12e-3
+// to 2.16e-3.  So lengths are not chosen for speed alone: a model that cut up to 607 heads and took lengths of 1 to
+// 64 tiles was faster in places (48 heads of 3000 x 128 90 -> 75 us, 160 heads of 2048 x 128 normalised 194 -> 175) and
+// about 2 % further from the 64-bit outputs at 32 heads of 1999 x 128 and 64 of 2048 x 128.
+int planned_tiles(int BH, int M, int sms) {
+    if (2 * BH >= sms) return M;
+    int best = 2;
+    double best_t = 1e300;
+    for (int L = 2; L <= 8 && L <= M; ++L) {
+        const double t = predicted_span(BH, M, L, sms);
         if (t < best_t) {
             best_t = t;
             best = L;
         }
     }
-    last = key;
-    last_L = best;
-    return best;
+    return best < M ? best : M;
+}
+
+int segment_tiles(int BH, int M, int sms) {
+    if (const char *e = getenv("HLA_FUSED_SEGMENT_TILES")) {
+        int v = atoi(e);
+        if (v > 0) return v < M ? v : M;
+    }
+    // The length depends on these three numbers alone, and simulating seven schedules takes the host 20 us at 32
+    // heads of 16 tiles and 60 us at 32 of 128, so a thread keeps the last 64 of its answers (prompts of many
+    // lengths, layers of different sizes in turn).
+    struct Plan {
+        int BH, M, sms, L;
+    };
+    constexpr int kPlans = 64;
+    static thread_local Plan plans[kPlans];
+    static thread_local int next = 0;
+    if (2 * BH >= sms) return M;
+    for (const Plan &q : plans)
+        if (q.BH == BH && q.M == M && q.sms == sms) return q.L;
+    const Plan made{BH, M, sms, planned_tiles(BH, M, sms)};
+    plans[next] = made;
+    next = (next + 1) % kPlans;
+    return made.L;
 }
 
 // ---------------------------------------------------------------------------
@@ -1554,8 +1532,7 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     kp.BH = p.BH;
     kp.n = p.n;
     kp.M = (p.n + kTile - 1) / kTile;
-    kp.L = p.masked ? segment_tiles(p.BH, kp.M, sms, p.d == 64 && p.dv == 64, p.normalized || p.state_out)
-                     : kp.M;  // unmasked: one segment per head
+    kp.L = p.masked ? segment_tiles(p.BH, kp.M, sms) : kp.M;  // unmasked: one segment per head
     kp.G = (kp.M + kp.L - 1) / kp.L;
     kp.n_items = kp.G * p.BH;
     kp.normalized = p.normalized;

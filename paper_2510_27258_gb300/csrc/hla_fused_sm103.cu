@@ -1290,22 +1290,28 @@ constexpr uint32_t kCSmemBytes = 4 * kTileBytes + kCOnesBytes + 1024;
 // TMEM, stores 128 contiguous bytes; row by row it stored 32 lines a time and the kernel took 31 us at
 // 32 heads of 2000 tokens), then m
 constexpr int kCPartFloats = kD * kD + kD;
+// A block sums up to three groups, each in TMEM columns of its own (C at 128 a, m at 384 + 32 a): one
+// accumulation over all of its tiles loses more to the tensor cores' fp32 additions (32 heads of 1999 x 128, the
+// whole tuple's distance from 64 bits: eight groups a head 2.77e-6, four 2.82e-6; uncut 4.53e-6 and 4.80e-6).
+constexpr int kCAccs = 3;
+constexpr uint32_t kCAccM = 384;
 
-// C and m of tiles [g * tiles_per, ...) of a head, from tiles of 128 tokens (Q^T V: A = Q^T and
-// B = V both MN-major; m: B = a 16-row K-major operand whose row 0 is ones).  The first group of a
-// head adds C_0, m_0 of state_in, which the launch after this may overwrite.
+// C and m of `per_block` groups of tiles of a head (group g: tiles [g * tiles_per, ...)), from tiles of
+// 128 tokens (Q^T V: A = Q^T and B = V both MN-major; m: B = a 16-row K-major operand whose row 0 is
+// ones).  The first group of a head adds C_0, m_0 of state_in, which the launch after this may overwrite.
 __global__ void __launch_bounds__(kCThreads, 1)
 state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_v, float *part,
-               int M, int groups, int tiles_per, const float *state_in, WsHeader *err) {
+               int M, int groups, int tiles_per, int per_block, const float *state_in, WsHeader *err) {
     extern __shared__ __align__(1024) uint8_t csm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int head = blockIdx.x / groups, g = blockIdx.x % groups;
-    const int j0 = g * tiles_per, j1 = min(M, j0 + tiles_per);
+    const int blocks = (groups + per_block - 1) / per_block;  // of a head
+    const int head = blockIdx.x / blocks, g0 = (blockIdx.x % blocks) * per_block, accs = min(per_block, groups - g0);
+    const int j0 = g0 * tiles_per, j1 = min(M, j0 + accs * tiles_per);
     uint8_t *ones = csm + 4 * kTileBytes;
-    // after the tiles and the ones operand: loads of slot pair 0 / 1, MMAs of pair 0 / 1, all done
+    // after the tiles and the ones operand: loads of slot pair 0 / 1, MMAs of pair 0 / 1, groups done
     uint64_t *bars = reinterpret_cast<uint64_t *>(ones + kCOnesBytes);
-    uint32_t &tmem_base_s = *reinterpret_cast<uint32_t *>(bars + 5);
-    int &abort_c = *reinterpret_cast<int *>(bars + 6);
+    uint32_t &tmem_base_s = *reinterpret_cast<uint32_t *>(bars + 4 + kCAccs);
+    int &abort_c = *reinterpret_cast<int *>(bars + 5 + kCAccs);
     if (smem_u32(csm) & 1023u) {
         if (tid == 0) set_error(err, 98, smem_u32(csm));
         return;
@@ -1317,12 +1323,12 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         *reinterpret_cast<uint16_t *>(ones + off) = row == 0 ? (uint16_t)0x3F80 : (uint16_t)0;
     }
     if (tid == 0) {
-        for (int b = 0; b < 5; ++b) mbar_init(&bars[b], 1);
+        for (int b = 0; b < 4 + kCAccs; ++b) mbar_init(&bars[b], 1);
         abort_c = 0;
         fence_mbar_init();
     }
     if (warp == 4) {
-        tmem_alloc(&tmem_base_s, 256);
+        tmem_alloc(&tmem_base_s, 512);
         tmem_relinquish();
     }
     fence_async_smem();
@@ -1354,36 +1360,43 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (j0 < j1) load_pair(j0);
             if (j0 + 1 < j1) load_pair(j0 + 1);
             constexpr uint32_t id_m = idesc_bf16(128, 16, 1, 0);
+            int a = 0, in_group = 0;  // the group's accumulator, the tile's place in it
             for (int j = j0; j < j1; ++j) {
                 const int i = j - j0, sl = i & 1;
+                const uint32_t tc = tb + a * 128, tm = tb + kCAccM + a * 32;
                 if (!cwait(sl, (i >> 1) & 1)) break;
                 tc_fence_after();
-                mma128<true, true>(tb, lmn(2 * sl), lmn(2 * sl + 1), i > 0 ? 1u : 0u);  // C += Q^T V
+                mma128<true, true>(tc, lmn(2 * sl), lmn(2 * sl + 1), in_group > 0 ? 1u : 0u);  // C += Q^T V
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)  // m += Q^T 1 (column 128)
-                    umma_bf16(tb + 128, (static_cast<uint64_t>(kDescHi) << 32) | (lmn(2 * sl) + kk * 128u),
+                for (int kk = 0; kk < 8; ++kk)  // m += Q^T 1
+                    umma_bf16(tm, (static_cast<uint64_t>(kDescHi) << 32) | (lmn(2 * sl) + kk * 128u),
                               (static_cast<uint64_t>(kDescHi) << 32) | (ones_lo + (kk >> 2) * 128u + (kk & 3) * 2u),
-                              id_m, (i > 0 || kk > 0) ? 1u : 0u);
+                              id_m, (in_group > 0 || kk > 0) ? 1u : 0u);
                 umma_commit(&bars[2 + sl]);
+                if (++in_group == tiles_per) {
+                    umma_commit(&bars[4 + a++]);
+                    in_group = 0;
+                }
                 if (j + 2 < j1) {
                     if (!cwait(2 + sl, (i >> 1) & 1)) break;
                     load_pair(j + 2);
                 }
             }
-            umma_commit(&bars[4]);
+            for (; a < accs; ++a) umma_commit(&bars[4 + a]);  // the ragged last group, and whatever a wait left
         }
         __syncwarp();
-    } else {
-        // C rows (features f = 32 warp + lane), 128 columns, then m (an initial state is 128 x 128)
-        float *out = part + (size_t)blockIdx.x * kCPartFloats;
-        const float *C0 = state_in && g == 0 ? state_in + (size_t)head * kStateFloats + kD * kD : nullptr;
+    } else
+    // C rows (features f = 32 warp + lane), 128 columns, then m (an initial state is 128 x 128)
+    for (int a = 0; a < accs; ++a) {
+        float *out = part + ((size_t)head * groups + g0 + a) * kCPartFloats;
+        const float *C0 = state_in && g0 + a == 0 ? state_in + (size_t)head * kStateFloats + kD * kD : nullptr;
         const uint32_t lb = (uint32_t)(32 * warp) << 16;
         const int f = 32 * warp + lane;
-        const bool ok = (j0 < j1) && cwait(4, 0);
+        const bool ok = j0 + a * tiles_per < j1 && cwait(4 + a, 0);
         tc_fence_after();
         for (int c0 = 0; c0 < kD; c0 += 32) {
             float v[32];
-            if (ok) ld32(tb + lb + c0, v);
+            if (ok) ld32(tb + lb + a * 128 + c0, v);
 #pragma unroll
             for (int jj = 0; jj < 32; jj += 4) {
                 const float4 x = C0 ? *reinterpret_cast<const float4 *>(C0 + f * kD + c0 + jj) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1394,14 +1407,14 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
         }
         float mv[32];
-        if (ok) ld32(tb + lb + 128, mv);
+        if (ok) ld32(tb + lb + kCAccM + a * 32, mv);
         out[kD * kD + f] = (ok ? mv[0] : 0.f) + (C0 ? C0[kD * kD + f] : 0.f);
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 4) {
         tc_fence_after();
-        tmem_dealloc(tb, 256);
+        tmem_dealloc(tb, 512);
     }
     chain_begin();  // this launch ends after the forward's, so the one after it may read the forward's ring
 }
@@ -1481,12 +1494,19 @@ __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, 
     }
 }
 
-// groups of tiles per head of state_c_kernel: one wave of one block an SM (152), at most 8 partials to add
+// groups of tiles per head of state_c_kernel, each a partial to add: about 256 in all, at most 8 a head
 int state_groups(int BH, int M) {
-    int g = 152 / (BH > 0 ? BH : 1);
+    int g = 256 / (BH > 0 ? BH : 1);
     if (g < 1) g = 1;
     if (g > 8) g = 8;
     return g < M ? g : M;
+}
+
+// groups that a block takes: as few as let all blocks run at once, one an SM (1 to 3: 256 groups, 152 SMs)
+int groups_per_block(int BH, int groups, int sms) {
+    int p = 1;
+    while (p < kCAccs && BH * ((groups + p - 1) / p) > sms) ++p;
+    return p < groups ? p : groups;
 }
 
 }  // namespace
@@ -1582,8 +1602,9 @@ cudaError_t fused2_forward(const Fwd2 &p, cudaStream_t stream) {
     if ((e = cudaFuncSetAttribute(state_c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCSmemBytes)))
         return e;
     // (each reads state_in, or what an earlier launch left; neither writes what the forward reads)
-    if ((e = chain_launch(true, state_c_kernel, dim3(p.BH * groups), kCThreads, kCSmemBytes, stream, mq, mv, part, kp.M, groups,
-                          tiles_per, p.state_in, kp.err)))
+    const int per_block = groups_per_block(p.BH, groups, sms);
+    if ((e = chain_launch(true, state_c_kernel, dim3(p.BH * ((groups + per_block - 1) / per_block)), kCThreads, kCSmemBytes,
+                          stream, mq, mv, part, kp.M, groups, tiles_per, per_block, p.state_in, kp.err)))
         return e;
     return chain_launch(true, state_finalize_kernel, dim3(p.BH, p.dv / kFinCols), 256, 0, stream, (const float *)kp.ring,
                         (kp.G - 1) & 1, (const float *)part, groups, p.state_out, p.d, p.dv);

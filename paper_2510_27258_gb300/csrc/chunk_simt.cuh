@@ -121,10 +121,11 @@ struct Vec<__nv_bfloat16> {
 };
 
 // token rows [rows][width] (width a multiple of 16) into shared rows of N + 4 floats; zero beyond
-// the rows and the width
+// the rows and the width.  Returns 0 if all that this thread loaded is finite, else NaN.
 template <int N, typename T>
-__device__ __forceinline__ void load_tile(float *dst, const T *__restrict__ src, int rows, int width) {
+__device__ __forceinline__ float load_tile(float *dst, const T *__restrict__ src, int rows, int width) {
     constexpr int W = Vec<T>::W, PER = N / W;
+    float seen = 0.f;
 #pragma unroll 4
     for (int i = threadIdx.x; i < kC * PER; i += kCT) {
         const int r = i / PER, c = (i % PER) * W;
@@ -133,10 +134,15 @@ __device__ __forceinline__ void load_tile(float *dst, const T *__restrict__ src,
         for (int j = 0; j < W; ++j) x[j] = 0.f;
         if (r < rows && c < width) Vec<T>::load(src + (long long)r * width + c, x);
 #pragma unroll
+        for (int j = 0; j < W; ++j) seen = fmaf(x[j], 0.f, seen);
+#pragma unroll
         for (int j = 0; j < W; j += 4)
             *reinterpret_cast<float4 *>(dst + r * (N + 4) + c + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
     }
+    return seen;
 }
+// block barrier; on return true in every thread if any `seen` is not zero
+__device__ __forceinline__ bool sync_unless_finite(float seen) { return __syncthreads_or(!(seen == 0.f)) != 0; }
 
 // acc[I0..][.] += sum_{k0 <= k < k1} A(r, k) B(k, c), A row-major in shared memory, B rows over c.
 // I0 = 4: only the second half of the rows (A is zero there for the first half).
@@ -170,9 +176,30 @@ __device__ __forceinline__ void nn(Acc<N> &acc, const Tile<N> &t, const float *A
                                    int K) {
     nn_range<N, 0>(acc, t, A, lda, B, ldb, 0, K);
 }
-// A a lower triangular chunk tile
+// The same where B has rows that are not finite: A a lower triangular chunk tile, row r takes the rows k <= r of B
+// (kUpper: A(k, r), the rows k >= r) and no other.
+template <int N, bool kUpper>
+__device__ __forceinline__ void masked_rows(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B) {
+    constexpr int RM = Tile<N>::RM, CM = Tile<N>::CM;
+#pragma unroll 1
+    for (int k = 0; k < kC; ++k)
+#pragma unroll
+        for (int i = 0; i < RM; ++i) {
+            const int r = t.row(i);
+            if (kUpper ? k < r : k > r) continue;
+            const float x = kUpper ? A[k * kLdW + r] : A[r * kLdW + k];
+#pragma unroll
+            for (int j = 0; j < CM; j += 2)
+                fma2(acc.p[i][j / 2], pack2(x, x), *reinterpret_cast<const f32x2 *>(B + k * (N + 4) + t.col(j)));
+        }
+}
+// A a lower triangular chunk tile.  `any` (the same in every thread): B may have rows that are not finite.  The
+// fast form multiplies such a row by the zeros above the diagonal too, which would make NaN of earlier tokens' rows.
+// Finding out costs one multiply-add per loaded value (B2 H16 n1000 d64 fp32 67.5 us without, 67.7 with); leaving out
+// the terms above the diagonal one by one took 69.8.
 template <int N>
-__device__ __forceinline__ void nn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B) {
+__device__ __forceinline__ void nn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B, bool any) {
+    if (any) return masked_rows<N, false>(acc, t, A, B);
     if constexpr (N == 32) {
         nn_range<N, 0>(acc, t, A, kLdW, B, N + 4, 0, kC);
     } else {
@@ -212,9 +239,10 @@ template <int N>
 __device__ __forceinline__ void tn(Acc<N> &acc, const Tile<N> &t, const float *A, int lda, const float *B) {
     tn_range<N, 0, Tile<N>::RM>(acc, t, A, lda, B, 0, kC);
 }
-// A a lower triangular chunk tile (A(k, r) = 0 for k < r)
+// A a lower triangular chunk tile (A(k, r) = 0 for k < r); `any` as above
 template <int N>
-__device__ __forceinline__ void tn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B) {
+__device__ __forceinline__ void tn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B, bool any) {
+    if (any) return masked_rows<N, true>(acc, t, A, B);
     if constexpr (N == 32) {
         tn_range<N, 0, 4>(acc, t, A, kLdW, B, 0, kC);
     } else {
@@ -315,14 +343,19 @@ __device__ __forceinline__ void nn_carry(Acc<N> &acc, const Tile<N> &t, const fl
     }
 }
 
+// returns 0 if all that this thread stored is finite, else NaN
 template <int N>
-__device__ __forceinline__ void acc_to_smem(const Acc<N> &acc, const Tile<N> &t, float *dst) {
+__device__ __forceinline__ float acc_to_smem(const Acc<N> &acc, const Tile<N> &t, float *dst) {
+    float seen = 0.f;
 #pragma unroll
     for (int i = 0; i < Tile<N>::RM; ++i)
 #pragma unroll
-        for (int j = 0; j < Tile<N>::CM; j += 4)
-            *reinterpret_cast<float4 *>(dst + t.row(i) * (N + 4) + t.col(j)) =
-                make_float4(acc.get(i, j), acc.get(i, j + 1), acc.get(i, j + 2), acc.get(i, j + 3));
+        for (int j = 0; j < Tile<N>::CM; j += 4) {
+            const float4 v = make_float4(acc.get(i, j), acc.get(i, j + 1), acc.get(i, j + 2), acc.get(i, j + 3));
+            seen = fmaf(v.x, 0.f, fmaf(v.y, 0.f, fmaf(v.z, 0.f, fmaf(v.w, 0.f, seen))));
+            *reinterpret_cast<float4 *>(dst + t.row(i) * (N + 4) + t.col(j)) = v;
+        }
+    return seen;
 }
 
 // rows r0 + r < rows, columns < width of the outputs to global memory, rows of `width` elements
@@ -365,14 +398,21 @@ __device__ __forceinline__ void col_sums(float *out, const float *A, const float
     }
 }
 
-// x_r = sum_c A(r, c) v_c, c < width (v null: 1), for the row r = threadIdx.x / 2 of a 64-row operand
-// with rows of ld floats; both threads of a row return the sum
+// x_r = sum_c A(r, c) v_c, c < width (v null: 1; kLower: c <= r), for the row r = threadIdx.x / 2 of a 64-row
+// operand with rows of ld floats; both threads of a row return the sum
+template <bool kLower = false>
 __device__ __forceinline__ float row_dot(const float *A, int ld, const float *v, int width) {
     const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
     float s = 0.f;
     for (int c = 4 * h; c < width; c += 8) {
         const float4 x = *reinterpret_cast<const float4 *>(A + r * ld + c);
-        const float4 y = v ? *reinterpret_cast<const float4 *>(v + c) : make_float4(1.f, 1.f, 1.f, 1.f);
+        float4 y = v ? *reinterpret_cast<const float4 *>(v + c) : make_float4(1.f, 1.f, 1.f, 1.f);
+        if (kLower) {  // the v of later tokens may not be finite
+            if (c > r) y.x = 0.f;
+            if (c + 1 > r) y.y = 0.f;
+            if (c + 2 > r) y.z = 0.f;
+            if (c + 3 > r) y.w = 0.f;
+        }
         s = fmaf(x.x, y.x, s);
         s = fmaf(x.y, y.y, s);
         s = fmaf(x.z, y.z, s);

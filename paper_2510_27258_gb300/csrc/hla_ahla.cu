@@ -86,20 +86,19 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     }
     s += row_dot(Wt, kLdW, nullptr, kC);
     if ((threadIdx.x & 1) == 0) ss[threadIdx.x >> 1] = s;
-    load_tile<N>(b0, v + tok * dv, len, dv);
+    const bool any_v = sync_unless_finite(load_tile<N>(b0, v + tok * dv, len, dv));
+    nn_lower<N>(acc, t, Wt, b0, any_v);
+    const float den = row_dot<true>(Wt, kLdW, ss, kC);
     __syncthreads();
-    nn_lower<N>(acc, t, Wt, b0);
-    const float den = row_dot(Wt, kLdW, ss, kC);
-    __syncthreads();
-    acc_to_smem<N>(acc, t, b0);  // R
+    const float seen_r = acc_to_smem<N>(acc, t, b0);  // R
     const int r = threadIdx.x >> 1;
     if ((threadIdx.x & 1) == 0) {
         if (A.direct) dens[r] = den + A.eps;
         else if (r < len) A.den[tok + r] = den;
     }
-    __syncthreads();
+    const bool any_r = sync_unless_finite(seen_r);
     acc.zero();
-    nn_lower<N>(acc, t, Wt, b0);  // A R
+    nn_lower<N>(acc, t, Wt, b0, any_r);  // A R
     if (A.direct) {
         if (A.normalized) acc.each([&](float x, int i, int) { return x / dens[t.row(i)]; });
         acc_to_global<N, T>(acc, t, out + tok * dv, len, dv);

@@ -89,13 +89,10 @@ struct Chunk {
 
 // G' rows of a chunk (the output gradient itself for the plain output) and u
 template <int N, typename T>
-__device__ __forceinline__ void load_upstream(float *dst, float *us, const BParams<T> &P, const Chunk<T> &ch) {
-    if (P.normalized) {
-        load_tile<N>(dst, P.num + ch.tok * P.dv, ch.len, P.dv);
-        if (us && threadIdx.x < kC) us[threadIdx.x] = threadIdx.x < ch.len ? P.den[ch.tok + threadIdx.x] : 0.f;
-    } else {
-        load_tile<N>(dst, P.g + ch.tok * P.dv, ch.len, P.dv);
-    }
+__device__ __forceinline__ float load_upstream(float *dst, float *us, const BParams<T> &P, const Chunk<T> &ch) {
+    if (!P.normalized) return load_tile<N>(dst, P.g + ch.tok * P.dv, ch.len, P.dv);
+    if (us && threadIdx.x < kC) us[threadIdx.x] = threadIdx.x < ch.len ? P.den[ch.tok + threadIdx.x] : 0.f;
+    return load_tile<N>(dst, P.num + ch.tok * P.dv, ch.len, P.dv);
 }
 
 // ---------------------------------------------------------------------------
@@ -109,15 +106,14 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_x_kernel(const __
     const Chunk<T> ch(P);
     const int d = P.d, dv = P.dv;
     load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
-    load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
-    __syncthreads();
+    const bool any_k = sync_unless_finite(load_tile<N>(b1, P.k + ch.tok * d, ch.len, d));
     const Tile<N> t;
     nt_masked(Wt, b0, b1, N + 4, d, nullptr);
     Acc<N> acc;
     acc.zero();
     if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);
     else __syncthreads();
-    nn_lower<N>(acc, t, Wt, b1);
+    nn_lower<N>(acc, t, Wt, b1, any_k);
     acc_to_global<N, float>(acc, t, P.X + ch.tok * d, ch.len, d);
     __syncthreads();
     acc_to_smem<N>(acc, t, b1);  // X
@@ -126,14 +122,13 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_x_kernel(const __
         nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
         __syncthreads();
     }
-    load_tile<N>(b0, P.v + ch.tok * dv, ch.len, dv);
-    __syncthreads();
+    const bool any_v = sync_unless_finite(load_tile<N>(b0, P.v + ch.tok * dv, ch.len, dv));
     if (P.normalized) {
         const float den = row_dot(Wt, kLdW, nullptr, kC);
         const int r = threadIdx.x >> 1;
         if ((threadIdx.x & 1) == 0 && r < ch.len) P.den[ch.tok + r] = den;
         acc.zero();
-        nn_lower<N>(acc, t, Wt, b0);
+        nn_lower<N>(acc, t, Wt, b0, any_v);
         acc_to_global<N, float>(acc, t, P.num + ch.tok * dv, ch.len, dv);
     }
     if (!ch.after) return;
@@ -224,9 +219,8 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_y_kernel(const __
     } else {
         __syncthreads();
     }
-    load_tile<N>(b1, P.q + ch.tok * d, ch.len, d);
-    __syncthreads();
-    tn_lower<N>(acc, t, Wt, b1);  // P^T Q
+    const bool any_q = sync_unless_finite(load_tile<N>(b1, P.q + ch.tok * d, ch.len, d));
+    tn_lower<N>(acc, t, Wt, b1, any_q);  // P^T Q
     acc_to_global<N, float>(acc, t, P.Y + ch.tok * d, ch.len, d);
     if (!ch.before) return;
     acc_to_smem<N>(acc, t, b0);  // Y; its rows beyond the sequence meet zero rows of Q
@@ -263,17 +257,15 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const
         } else {
             __syncthreads();
         }
-        load_tile<N>(b1, P.X + ch.tok * d, ch.len, d);
-        __syncthreads();
-        nn_lower<N>(acc, t, Wt, b1);  // P X
+        const bool any_x = sync_unless_finite(load_tile<N>(b1, P.X + ch.tok * d, ch.len, d));
+        nn_lower<N>(acc, t, Wt, b1, any_x);  // P X
         __syncthreads();
         load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
-        load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
-        __syncthreads();
+        const bool any_k = sync_unless_finite(load_tile<N>(b1, P.k + ch.tok * d, ch.len, d));
         nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
         if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);  // Y S_p
         else __syncthreads();
-        nn_lower<N>(acc, t, Wt, b1);  // B K
+        nn_lower<N>(acc, t, Wt, b1, any_k);  // B K
         acc_to_global<N, T>(acc, t, P.dq + ch.tok * d, ch.len, d);
     } else if (blockIdx.z == 1) {
         load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
@@ -282,15 +274,13 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const
         nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
         if (ch.after) nn_carry<N, kSymmetric>(acc, t, b1, P.Lam.at(ch.hd, ch.c), d, d, d, stage);
         else __syncthreads();
-        load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
-        __syncthreads();
-        tn_lower<N>(acc, t, Wt, b0);  // B^T Q
+        const bool any_q = sync_unless_finite(load_tile<N>(b0, P.q + ch.tok * d, ch.len, d));
+        tn_lower<N>(acc, t, Wt, b0, any_q);  // B^T Q
         __syncthreads();
         nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // W
         __syncthreads();
-        load_tile<N>(b1, P.Y + ch.tok * d, ch.len, d);
-        __syncthreads();
-        tn_lower<N>(acc, t, Wt, b1);  // W^T Y
+        const bool any_y = sync_unless_finite(load_tile<N>(b1, P.Y + ch.tok * d, ch.len, d));
+        tn_lower<N>(acc, t, Wt, b1, any_y);  // W^T Y
         acc_to_global<N, T>(acc, t, P.dk + ch.tok * d, ch.len, d);
     } else {
         load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
@@ -299,9 +289,8 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const
         nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
         if (ch.after) nn_carry<N, kPlain>(acc, t, b1, P.Gam.at(ch.hd, ch.c), dv, d, dv, stage);  // X Gam_s^T
         else __syncthreads();
-        load_upstream<N>(b0, static_cast<float *>(nullptr), P, ch);
-        __syncthreads();
-        tn_lower<N>(acc, t, Wt, b0);  // T^T G'
+        const bool any_g = sync_unless_finite(load_upstream<N>(b0, static_cast<float *>(nullptr), P, ch));
+        tn_lower<N>(acc, t, Wt, b0, any_g);  // T^T G'
         acc_to_global<N, T>(acc, t, P.dv_out + ch.tok * dv, ch.len, dv);
     }
 }

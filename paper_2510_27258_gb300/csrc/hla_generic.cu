@@ -118,22 +118,21 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     const long long tok = (long long)hd * P.n + t0;
     const bool carry = c > 0 || P.has_in;
     load_tile<N>(b0, q + tok * d, len, d);
-    load_tile<N>(b1, k + tok * d, len, d);
-    __syncthreads();
+    const bool any_k = sync_unless_finite(load_tile<N>(b1, k + tok * d, len, d));
     const Tile<N> t;
     nt_masked(Wt, b0, b1, N + 4, d, nullptr);
     Acc<N> acc;
     acc.zero();
     if (carry) nn_carry<N, kPlain>(acc, t, b0, P.S.at(hd, c), d, d, d, stage);
     else __syncthreads();
-    nn_lower<N>(acc, t, Wt, b1);
+    nn_lower<N>(acc, t, Wt, b1, any_k);
     __syncthreads();
     acc_to_smem<N>(acc, t, b1);  // X
     __syncthreads();
     if (P.masked) nt_masked(Wt, b0, b1, N + 4, d, nullptr);
     else nt_masked(Wt, b1, b0, N + 4, d, nullptr);
     __syncthreads();
-    load_tile<N>(b0, v + tok * dv, len, dv);
+    const float seen_v = load_tile<N>(b0, v + tok * dv, len, dv);
     float den = row_dot(Wt, kLdW, nullptr, kC);
     acc.zero();
     if (!P.masked && carry) {
@@ -147,8 +146,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
         if (direct) dens[r] = P.normalized ? den + P.eps : 1.f;
         else if (r < len) P.den[tok + r] = den;
     }
-    __syncthreads();
-    nn_lower<N>(acc, t, Wt, b0);  // T V
+    nn_lower<N>(acc, t, Wt, b0, sync_unless_finite(seen_v));  // T V
     if (direct) {
         if (P.normalized) acc.each([&](float x, int i, int) { return x / dens[t.row(i)]; });
         acc_to_global<N, T>(acc, t, out + tok * dv, len, dv);

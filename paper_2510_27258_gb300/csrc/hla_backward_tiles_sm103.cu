@@ -52,6 +52,7 @@ struct Misc {
     uint32_t tmem_base;
     int abort_flag;
     float us[kTile], vec[kF], red[kThreads];
+    int stains, first[kF], last[kF];  // of each column, the first and last row that drop() took a value from
 };
 constexpr uint32_t kSmemBytes = 3 * kTileBytes + sizeof(Misc);
 enum { bLd = 0, bMma = 1, bMma2 = 2 };
@@ -119,6 +120,21 @@ __device__ __forceinline__ int rec_index(int r, int c) {  // float4 index of (r,
     return (((r >> 5) * 16 + (c >> 3)) * 2 + ((c >> 2) & 1)) * 32 + (r & 31);
 }
 
+// takes the values that are not finite out of a slot and notes the first and last row of each column's
+__device__ __noinline__ void drop_values(uint8_t *slot, Misc *ms) {
+    for (int i = threadIdx.x; i < (int)(kTileBytes / 2); i += kThreads) {
+        __nv_bfloat16 *p = reinterpret_cast<__nv_bfloat16 *>(slot) + i;
+        const float x = __bfloat162float(*p);
+        if (x - x == 0.f) continue;
+        const int row = i / 64 % kTile;  // element i of a slot: the inverse of tile_off()
+        const int col = i / (int)(kBlockBytes / 2) * 64 + ((i / 8 % 8) ^ (row & 7)) * 8 + i % 8;
+        atomicMin(&ms->first[col], row);
+        atomicMax(&ms->last[col], row);
+        *p = __float2bfloat16_rn(0.f);
+    }
+    if (threadIdx.x == 0) ms->stains = 1;
+}
+
 // ------------------------------- a block's state -------------------------------
 struct Ctx {
     uint8_t *sm;
@@ -145,9 +161,14 @@ struct Ctx {
         s4 = smem_u32(smem) >> 4;
         if (tid == 0) {
             for (int b = 0; b < 3; ++b) mbar_init(&ms->bar[b], 1);
+            ms->stains = 0;
             ms->abort_flag = (smem_u32(smem) & 1023u) != 0;  // the swizzled layout needs 1 KiB alignment
             if (ms->abort_flag) fail(0);
             fence_mbar_init();
+        }
+        if (tid < kF) {
+            ms->first[tid] = kTile;
+            ms->last[tid] = -1;
         }
         __syncwarp();
         if (warp == 0) {
@@ -200,6 +221,36 @@ struct Ctx {
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
+    }
+
+    // A masked tile's zeros times a token that is not finite would make NaN of rows that do not depend on the
+    // token.  So before a product of a masked tile and the rows of a slot, every value of the slot that is not finite
+    // is taken out and noted, and the result is NaN where the triangle holds a noted value (stain()).
+    // nonfinite(): whether the slot has any, the same in every thread (a barrier; a hi slot answers for its lo).
+    __device__ bool nonfinite(int s) {
+        __nv_bfloat162 seen = __floats2bfloat162_rn(0.f, 0.f);
+        const __nv_bfloat162 zero = seen;
+#pragma unroll
+        for (int i = 0; i < (int)(kTileBytes / 16) / kThreads; ++i) {
+            const uint4 v = reinterpret_cast<const uint4 *>(slot(s))[tid + i * kThreads];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) seen = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&w[u]), zero, seen);
+        }
+        return __syncthreads_or(!(__low2float(seen) == 0.f && __high2float(seen) == 0.f)) != 0;
+    }
+    __device__ void drop(int s) {
+        drop_values(slot(s), ms);
+        publish();
+    }
+    enum Stain { kNone, kLower, kUpperT, kColumn };  // rows from the first noted one, up to the last, all
+    __device__ void stain(Stain how, int c0, float (&x)[32]) {
+        if (how == kNone || !ms->stains) return;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            const int f = ms->first[c0 + u], l = ms->last[c0 + u];
+            if (how == kLower ? r >= f : how == kUpperT ? r <= l : l >= 0) x[u] = __int_as_float(0x7fffffff);
+        }
     }
 
     // The masked tile of region RA (kUpper: column >= row, else column <= row), with us[column] or
@@ -267,7 +318,7 @@ struct Ctx {
         }
     }
     // a region -> hi, lo slots, `vec` added to every row where `add`
-    __device__ void region_to_slots(uint32_t region, int hi, int lo, bool add) {
+    __device__ void region_to_slots(uint32_t region, int hi, int lo, bool add, Stain how) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int c0 = 64 * half + 32 * i;
@@ -277,16 +328,18 @@ struct Ctx {
 #pragma unroll
                 for (int u = 0; u < 32; ++u) x[u] += ms->vec[c0 + u];
             }
+            stain(how, c0, x);
             split_store(hi, lo, c0, x);
         }
     }
-    __device__ void region_to_record(uint32_t region, float *rec) {
+    __device__ void region_to_record(uint32_t region, float *rec, Stain how = kNone) {
         float4 *o = reinterpret_cast<float4 *>(rec + at * kRec);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int c0 = 64 * half + 32 * i;
             float x[32];
             read32(region, c0, x);
+            stain(how, c0, x);
 #pragma unroll
             for (int u = 0; u < 32; u += 4) o[rec_index(r, c0 + u)] = make_float4(x[u], x[u + 1], x[u + 2], x[u + 3]);
         }
@@ -324,7 +377,7 @@ struct Ctx {
         return x;
     }
     // a region (plus row_add[r] vec[c] where `add`) as bf16 through slot s to the tile's rows of an output
-    __device__ void region_to_output(uint32_t region, int s, const CUtensorMap *m, int width, bool add) {
+    __device__ void region_to_output(uint32_t region, int s, const CUtensorMap *m, int width, bool add, Stain how) {
         const float ur = add ? ms->us[r] : 0.f;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -335,6 +388,7 @@ struct Ctx {
 #pragma unroll
                 for (int u = 0; u < 32; ++u) x[u] = fmaf(ur, ms->vec[c0 + u], x[u]);
             }
+            stain(how, c0, x);
 #pragma unroll
             for (int g = 0; g < 4; ++g)
                 *reinterpret_cast<uint4 *>(slot(s) + tile_off(r, c0 + 8 * g)) =
@@ -415,6 +469,7 @@ __device__ void x_steps(Ctx &c, const Maps &m) {
         c.expect(1);
         c.load_image(2, p.iS, 1);
     }
+    if (c.nonfinite(1)) c.drop(1);
     c.mask_pack<false>(false);  // W
     c.publish();
     if (c.before && !c.wait_ld()) return;
@@ -425,7 +480,7 @@ __device__ void x_steps(Ctx &c, const Maps &m) {
         c.commit();
     }
     if (!c.wait_mma()) return;
-    c.region_to_slots(c.RB(), 1, 2, false);  // X over K and S
+    c.region_to_slots(c.RB(), 1, 2, false, Ctx::kLower);  // X over K and S
     c.publish();
     if (c.tid == 0) c.store_images(p.iX, 1, 2);
     if (norm) {
@@ -450,6 +505,7 @@ __device__ void x_steps(Ctx &c, const Maps &m) {
         c.publish();
     }
     if (!c.wait_ld()) return;
+    if (norm && c.nonfinite(0)) c.drop(0);
     if (c.tid == 0) {
         if (norm) {
             mma_ts(c.RB(), c.RA(), c.sl(0), false);  // T V
@@ -464,11 +520,11 @@ __device__ void x_steps(Ctx &c, const Maps &m) {
     }
     if (norm) {
         if (!c.wait_mma()) return;
-        c.region_to_record(c.RB(), p.rec1);
+        c.region_to_record(c.RB(), p.rec1, Ctx::kLower);
     }
     if (c.after) {
         if (!c.wait_mma2()) return;
-        c.region_to_record(c.RA(), p.rec);
+        c.region_to_record(c.RA(), p.rec, Ctx::kColumn);
     }
 }
 __global__ void __launch_bounds__(kThreads, 2) bt_x_kernel(const __grid_constant__ Maps m, const __grid_constant__ TParams p) {
@@ -642,13 +698,14 @@ __device__ void y_steps(Ctx &c, const Maps &m) {
         }
         if (!c.wait_ld()) return;
     }
+    if (c.nonfinite(1)) c.drop(1);
     if (c.tid == 0) {
         mma_ts(c.RB(), c.RA(), c.sl(1), c.after);  // P^T Q
         mma_ts(c.RB(), c.RA() + 16, c.sl(1), true);
         c.commit();
     }
     if (!c.wait_mma()) return;
-    c.region_to_slots(c.RB(), 0, 2, norm && c.after);  // Y over V and Gam; + h_s (rows beyond n meet zero rows of Q)
+    c.region_to_slots(c.RB(), 0, 2, norm && c.after, Ctx::kUpperT);  // Y over V and Gam; + h_s (rows beyond n meet zero rows of Q)
     c.publish();
     if (c.tid == 0) {
         c.store_images(p.iY, 0, 2);
@@ -725,6 +782,10 @@ __device__ void dq_steps(Ctx &c, const Maps &m) {
         c.load_image(1, p.iX, 1);
     }
     if (!c.wait_ld()) return;
+    if (c.nonfinite(0)) {
+        c.drop(0);
+        c.drop(1);
+    }
     if (c.tid == 0) {
         mma_ts(c.RB(), c.RA(), c.sl(0), c.before);  // P X
         mma_ts(c.RB(), c.RA() + 16, c.sl(0), true);
@@ -745,6 +806,7 @@ __device__ void dq_steps(Ctx &c, const Maps &m) {
         c.commit();
     }
     if (!c.wait_mma()) return;
+    if (c.nonfinite(0)) c.drop(0);
     c.mask_pack<false>(false);
     c.publish();
     if (c.tid == 0) {
@@ -761,7 +823,7 @@ __device__ void dq_steps(Ctx &c, const Maps &m) {
         if (c.tid == 0) mma<K, K>(c.RB(), c.sl(1), c.sl(0), true);
     }
     if (c.tid == 0) c.commit();
-    if (c.wait_mma()) c.region_to_output(c.RB(), 0, &m.dq, p.d, norm && c.before);  // + u e_p^T
+    if (c.wait_mma()) c.region_to_output(c.RB(), 0, &m.dq, p.d, norm && c.before, Ctx::kLower);  // + u e_p^T
 }
 
 __device__ void dk_steps(Ctx &c, const Maps &m) {
@@ -778,6 +840,8 @@ __device__ void dk_steps(Ctx &c, const Maps &m) {
         c.commit();
     }
     if (!c.wait_mma()) return;
+    const bool bad_y = c.nonfinite(2);
+    if (bad_y) c.drop(2);
     c.mask_pack<true>(false);
     c.publish();
     if (c.tid == 0) {
@@ -785,6 +849,7 @@ __device__ void dk_steps(Ctx &c, const Maps &m) {
         mma_ts(c.RB(), c.RA() + 16, c.sl(2), true);
     }
     if (!swap_in(c, 2, p.iY, 1)) return;
+    if (bad_y) c.drop(2);
     if (c.tid == 0) {
         mma_ts(c.RB(), c.RA(), c.sl(2), true);
         mma<K, K>(c.RA(), c.sl(0), c.sl(2), false);  // B^T = K Y^T over W^T, read by the products before it
@@ -799,6 +864,7 @@ __device__ void dk_steps(Ctx &c, const Maps &m) {
         c.expect(1);
         c.load_image(2, p.iLam, 0);
     }
+    if (c.nonfinite(1)) c.drop(1);
     c.mask_pack<true>(false);
     c.publish();
     if (c.tid == 0) {
@@ -812,7 +878,7 @@ __device__ void dk_steps(Ctx &c, const Maps &m) {
         if (c.tid == 0) mma<K, K>(c.RB(), c.sl(0), c.sl(2), true);
     }
     if (c.tid == 0) c.commit();
-    if (c.wait_mma()) c.region_to_output(c.RB(), 0, &m.dk, p.d, false);
+    if (c.wait_mma()) c.region_to_output(c.RB(), 0, &m.dk, p.d, false, Ctx::kUpperT);
 }
 
 __device__ void dv_steps(Ctx &c, const Maps &m) {
@@ -854,13 +920,17 @@ __device__ void dv_steps(Ctx &c, const Maps &m) {
         load_g(c, m, 0, 1);
     }
     if (!c.wait_ld()) return;
+    if (c.nonfinite(0)) {
+        c.drop(0);
+        if (p.normalized) c.drop(1);
+    }
     if (c.tid == 0) {
         mma_ts(c.RB(), c.RA(), c.sl(0), c.after);  // T^T G'
         mma_ts(c.RB(), c.RA() + 16, c.sl(0), true);
         if (p.normalized) mma_ts(c.RB(), c.RA(), c.sl(1), true);
         c.commit();
     }
-    if (c.wait_mma()) c.region_to_output(c.RB(), 2, &m.dv, p.dv, false);
+    if (c.wait_mma()) c.region_to_output(c.RB(), 2, &m.dv, p.dv, false, Ctx::kUpperT);
 }
 __global__ void __launch_bounds__(kThreads, 2) bt_grad_kernel(const __grid_constant__ Maps m, const __grid_constant__ TParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];

@@ -86,3 +86,12 @@ def check_backward(hla, d, dv, dtype, which, j, value):
 @pytest.mark.parametrize("value", BAD)
 def test_backward(hla, d, dv, dtype, which, j, value):
     check_backward(hla, d, dv, dtype, which, j, value)
+
+
+@pytest.mark.parametrize("d,dv", [(128, 128), (64, 128), (128, 64)])
+@pytest.mark.parametrize("which", "qkvg")
+@pytest.mark.parametrize("j", [0, 5, 100, 127, 128, 149])
+@pytest.mark.parametrize("value", BAD)
+def test_backward_tiles(hla, d, dv, which, j, value):
+    """bf16 tokens with a head size of 128: tiles of 128 tokens on the tensor cores"""
+    check_backward(hla, d, dv, "bf16", which, j, value)

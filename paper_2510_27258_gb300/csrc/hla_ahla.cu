@@ -322,7 +322,8 @@ template <typename T, int NC>
 __global__ void __launch_bounds__(kSplitThreads)
 ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                        float *state, int split, int d, int dv, int normalized, float eps) {
-    __shared__ __align__(16) float qs[128], ks[128], vs[128];
+    // qs[d] is zero: it stands for the rows beyond a slice (an infinite entry would make NaN of their zeros)
+    __shared__ __align__(16) float qs[132], ks[128], vs[128];
     __shared__ __align__(16) float part[2][kSplitWarps][64];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int hd = blockIdx.x / split, rank = blockIdx.x % split, cw = dv / split, col0 = rank * cw;
@@ -352,6 +353,7 @@ ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T
         ks[tid] = to_f32(k[(long long)hd * d + tid]);
     }
     if (tid < dv) vs[tid] = to_f32(v[(long long)hd * dv + tid]);
+    if (tid == 0) qs[d] = 0.f;
     __syncthreads();
     const float qk = warp_dot(qs, ks, d);
     float qm = 0.f, qn = 0.f;
@@ -368,7 +370,7 @@ ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-        const float qr = qs[min(r0 + i * rstep, d - 1)];  // beyond the slice the values are zero
+        const float qr = qs[min(r0 + i * rstep, d)];
         fma4(a0, qr, pv[i]);
         fma4(a1, qr, ev[i]);
     }

@@ -341,7 +341,8 @@ template <typename T, bool kSDE, int TH, int NS, int NC>
 __global__ void __launch_bounds__(TH, TH == 256 ? (kSDE ? 3 : 2) : 1)
 step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
                    float *state, int split, int d, int dv, int masked, int normalized, float eps) {
-    __shared__ __align__(16) float qs[128], ks[128], vs[128], us[128];
+    // entry d is zero: it stands for the rows beyond a slice (an infinite entry would make NaN of their zeros)
+    __shared__ __align__(16) float qs[132], ks[132], vs[128], us[132];
     // per warp: sums of a column slice (at most 64 columns), for k^T C and u'^T C (or q^T D), and q^T G
     __shared__ __align__(16) float part[3][TH / 32][64];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -381,6 +382,7 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
         ks[tid] = to_f32(k[(long long)hd * d + tid]);
     }
     if (tid < dv) vs[tid] = to_f32(v[(long long)hd * dv + tid]);
+    if (tid == 0) qs[d] = ks[d] = us[d] = 0.f;
     __syncthreads();
     const float kq = warp_dot(ks, qs, d);
     float km = 0.f, qm = 0.f, qh = 0.f;
@@ -423,7 +425,7 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-        const int row = min(r0 + i * rstep, d - 1);  // beyond the slice the values are zero
+        const int row = min(r0 + i * rstep, d);
         fma4(a0, kSDE ? qs[row] : ks[row], cv[i]);
         if (!kSDE) fma4(a1, qs[row], gv[i]);
     }
@@ -447,7 +449,7 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
         um = group_sum<32>(um) + uq;  // u'.(m + q)
         a0 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < NC; ++i) fma4(a0, us[min(r0 + i * rstep, d - 1)], cv[i]);
+        for (int i = 0; i < NC; ++i) fma4(a0, us[min(r0 + i * rstep, d)], cv[i]);
         a0 = column_sum(a0, wC);
         if (lane < wC) *reinterpret_cast<float4 *>(&part[1][wid][c4]) = a0;
     }

@@ -311,9 +311,9 @@ ahla_step_staged_kernel(const T *__restrict__ q, const T *__restrict__ k, const 
 // The step with every load issued at once, straight to registers, by `split` blocks per head, block r
 // with columns [r dv / split, ...) of P and E.  From the old values, r = q^T P + (q.k) v and
 // o = q^T E + (q.k) r, column by column, so one pass does the step: both column sums, then both updated
-// slices.  Only m and n are shared.  The plain output needs them in block 0 alone; for the normalised
-// output the blocks of a head form a cluster and meet in a split barrier between their last read of m, n
-// and block 0's write.  Measured, us a step (staged -> this), bf16 tokens: 64 x 64, 16 heads 3.7 -> 2.8,
+// slices.  Only m, n and the tokens are shared.  The plain output needs m and n in block 0 alone; for the
+// normalised output, and where `out` lies over the tokens, the blocks of a head form a cluster and meet in a
+// split barrier between their last read of these and the first write.  Measured, us a step (staged -> this), bf16 tokens: 64 x 64, 16 heads 3.7 -> 2.8,
 // 256 heads 6.1 -> 4.0, 2048 heads 35.6 -> 23.4 (140 MB read and written: 5.9 TB/s); 128 x 128, 32
 // heads 5.7 -> 3.3, 2048 heads as fast (90.3 us a step over 541 MB of states).  Bound by the latency of
 // one load and two barriers for few heads, by HBM for many.
@@ -380,7 +380,7 @@ ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T
         *reinterpret_cast<float4 *>(&part[0][wid][c4]) = a0;
         *reinterpret_cast<float4 *>(&part[1][wid][c4]) = a1;
     }
-    cluster_arrive();  // this block has read m, n
+    cluster_arrive();  // this block has read m, n and the tokens
     __syncthreads();
     const float4 v4 = *reinterpret_cast<const float4 *>(vs + col0 + c4);
     float4 r4 = make_float4(qk * v4.x, qk * v4.y, qk * v4.z, qk * v4.w);
@@ -395,16 +395,18 @@ ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T
             *reinterpret_cast<float4 *>(E + at) = axpy4(ev[i], ks[row], r4);
         }
     }
+    float4 o = make_float4(qk * r4.x, qk * r4.y, qk * r4.z, qk * r4.w);
     if (tid < wC) {
-        float4 o = make_float4(qk * r4.x, qk * r4.y, qk * r4.z, qk * r4.w);
 #pragma unroll
         for (int w = 0; w < kSplitWarps; ++w) fma4(o, 1.f, *reinterpret_cast<const float4 *>(&part[1][w][c4]));
+    }
+    cluster_wait();  // every block of the head has read m, n and the tokens
+    if (tid < wC) {
         const float x[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             from_f32(&out[(long long)hd * dv + col0 + c4 + j], normalized ? x[j] / (den + eps) : x[j]);
     }
-    cluster_wait();  // every block of the head has read m, n
     if (rank == 0 && wid == 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -435,8 +437,10 @@ int ahla_step_split(int BH, int d, int dv, int normalized) {
 template <typename T>
 cudaError_t ahla_step_split_launch(const void *q, const void *k, const void *v, void *out, float *state, int BH,
                                    int split, int d, int dv, int normalized, float eps, cudaStream_t s) {
+    const size_t nq = sizeof(T) * (size_t)BH * d, nv = sizeof(T) * (size_t)BH * dv;
+    const bool over = memory_meets(out, nv, q, nq) || memory_meets(out, nv, k, nq) || memory_meets(out, nv, v, nv);
     auto go = [&](auto kern) {
-        return launch_blocks(kern, BH, split, normalized != 0, kSplitThreads, s, static_cast<const T *>(q), static_cast<const T *>(k),
+        return launch_blocks(kern, BH, split, normalized || over, kSplitThreads, s, static_cast<const T *>(q), static_cast<const T *>(k),
                             static_cast<const T *>(v), static_cast<T *>(out), state, split, d, dv, normalized, eps);
     };
     const int nc = (d * (dv / split) / 4 + kSplitThreads - 1) / kSplitThreads;

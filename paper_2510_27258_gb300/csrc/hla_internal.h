@@ -26,6 +26,12 @@ enum DevError : unsigned int { kDevOk = 0, kDevTimeout = 1 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// whether two ranges of memory have a byte in common
+inline bool memory_meets(const void *a, size_t na, const void *b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
+}
+
 // Records a host-side error message for hla_last_error() and returns `st`.
 hla_status fail(hla_status st, const char *fmt, ...);
 // Empties the message hla_last_error() returns (every entry point starts with it).

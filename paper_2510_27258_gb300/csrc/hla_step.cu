@@ -435,7 +435,7 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
         *reinterpret_cast<float4 *>(&part[0][wid][c4]) = a0;
         if (!kSDE) *reinterpret_cast<float4 *>(&part[2][wid][c4]) = a1;
     }
-    cluster_arrive();  // this block has read S, m, h
+    cluster_arrive();  // this block has read S, m, h and the tokens
     __syncthreads();   // us, part
     const float uq = warp_dot(us, qs, d);
     const float4 v4 = *reinterpret_cast<const float4 *>(vs + col0 + c4);
@@ -463,6 +463,7 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
             *reinterpret_cast<float4 *>(G + (long long)row * dv + col0 + c4) = axpy4(gv[i], ks[row], kC);
     }
     __syncthreads();  // part[1]
+    float result = 0.f;
     if (tid < cw) {
         float x0 = 0.f, x1 = 0.f, x2 = 0.f;
         for (int w = 0; w < TH / 32; ++w) {
@@ -484,9 +485,10 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
                 den -= qh + kq * km;
             }
         }
-        from_f32(&out[(long long)hd * dv + col0 + tid], normalized ? num / (den + eps) : num);
+        result = normalized ? num / (den + eps) : num;
     }
-    cluster_wait();  // every block of the head has read S, m, h
+    cluster_wait();  // every block of the head has read S, m, h and the tokens, over which `out` may lie
+    if (tid < cw) from_f32(&out[(long long)hd * dv + col0 + tid], result);
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
         const int f = tid + i * TH, row = f / wS, c = (f % wS) * 4;

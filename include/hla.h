@@ -136,7 +136,8 @@ size_t hla2_backward_workspace_bytes(int B, int H, int n, int d, int dv, int chu
  * rounding.  normalized selects out = num / (den + eps) (Eq. masked).
  * q, k, v : device [B, H, n, d] / [B, H, n, d] / [B, H, n, dv] of type dt
  * dout    : device [B, H, n, dv] of type dt (the gradient of the output)
- * dq, dk  : device [B, H, n, d] of type dt (written); dv : [B, H, n, dv] (written)
+ * dq, dk  : device [B, H, n, d] of type dt (written); dv : [B, H, n, dv] (written);
+ *           an output may lie over a whole token array of its own row width
  * workspace : at least hla2_backward_workspace_bytes(...) bytes, 256-byte aligned.
  * Errors as for hla2_forward.
  */

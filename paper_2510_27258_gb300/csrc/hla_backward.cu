@@ -229,68 +229,106 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_y_kernel(const __
 }
 
 // ---------------------------------------------------------------------------
-// the gradients: blockIdx.z 0 dQ, 1 dK, 2 dV
+// the gradients
 // ---------------------------------------------------------------------------
+// dQ
 template <int N, typename T>
+__device__ __forceinline__ void grad_q(Acc<N> &acc, const Tile<N> &t, float *sm, const BParams<T> &P, const Chunk<T> &ch) {
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    float *us = stage + stage_floats<N>();
+    const int d = P.d, dv = P.dv;
+    load_upstream<N>(b0, us, P, ch);
+    load_tile<N>(b1, P.v + ch.tok * dv, ch.len, dv);
+    __syncthreads();
+    nt_masked(Wt, b0, b1, N + 4, dv, P.normalized ? us : nullptr);  // P
+    if (ch.before) {
+        const float *Dp = P.D.at(ch.hd, ch.c);
+        nn_carry<N, kTransposed>(acc, t, b0, Dp, dv, dv, d, stage);  // G' D_p^T
+        if (P.normalized)
+            acc.each([&](float x, int i, int j) {
+                return t.col(j) < d ? fmaf(us[t.row(i)], Dp[d * dv + t.col(j)], x) : x;
+            });
+    } else {
+        __syncthreads();
+    }
+    const bool any_x = sync_unless_finite(load_tile<N>(b1, P.X + ch.tok * d, ch.len, d));
+    nn_lower<N>(acc, t, Wt, b1, any_x);  // P X
+    __syncthreads();
+    load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
+    const bool any_k = sync_unless_finite(load_tile<N>(b1, P.k + ch.tok * d, ch.len, d));
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
+    if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);  // Y S_p
+    else __syncthreads();
+    nn_lower<N>(acc, t, Wt, b1, any_k);  // B K
+}
+
+// dK
+template <int N, typename T>
+__device__ __forceinline__ void grad_k(Acc<N> &acc, const Tile<N> &t, float *sm, const BParams<T> &P, const Chunk<T> &ch) {
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    const int d = P.d;
+    load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
+    load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
+    __syncthreads();
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
+    if (ch.after) nn_carry<N, kSymmetric>(acc, t, b1, P.Lam.at(ch.hd, ch.c), d, d, d, stage);
+    else __syncthreads();
+    const bool any_q = sync_unless_finite(load_tile<N>(b0, P.q + ch.tok * d, ch.len, d));
+    tn_lower<N>(acc, t, Wt, b0, any_q);  // B^T Q
+    __syncthreads();
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // W
+    __syncthreads();
+    const bool any_y = sync_unless_finite(load_tile<N>(b1, P.Y + ch.tok * d, ch.len, d));
+    tn_lower<N>(acc, t, Wt, b1, any_y);  // W^T Y
+}
+
+// dV
+template <int N, typename T>
+__device__ __forceinline__ void grad_v(Acc<N> &acc, const Tile<N> &t, float *sm, const BParams<T> &P, const Chunk<T> &ch) {
+    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
+    const int d = P.d, dv = P.dv;
+    load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
+    load_tile<N>(b1, P.X + ch.tok * d, ch.len, d);
+    __syncthreads();
+    nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
+    if (ch.after) nn_carry<N, kPlain>(acc, t, b1, P.Gam.at(ch.hd, ch.c), dv, d, dv, stage);  // X Gam_s^T
+    else __syncthreads();
+    const bool any_g = sync_unless_finite(load_upstream<N>(b0, static_cast<float *>(nullptr), P, ch));
+    tn_lower<N>(acc, t, Wt, b0, any_g);  // T^T G'
+}
+
+// blockIdx.z 0 dQ, 1 dK, 2 dV; kOver, where an output lies over the tokens: one block forms all three of a chunk,
+// whose tokens no other block reads any more, before it writes any
+template <int N, typename T, bool kOver>
 __global__ void __launch_bounds__(kCT, blocks_per_sm<N>()) bwd_grad_kernel(const __grid_constant__ BParams<T> P) {
     extern __shared__ __align__(16) float sm[];
     chain_begin();
-    float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
-    float *us = stage + stage_floats<N>();
     const Chunk<T> ch(P);
     const int d = P.d, dv = P.dv;
     const Tile<N> t;
     Acc<N> acc;
     acc.zero();
-    if (blockIdx.z == 0) {
-        load_upstream<N>(b0, us, P, ch);
-        load_tile<N>(b1, P.v + ch.tok * dv, ch.len, dv);
+    if constexpr (kOver) {
+        Acc<N> acc_k, acc_v;
+        acc_k.zero();
+        acc_v.zero();
+        grad_q<N>(acc, t, sm, P, ch);
         __syncthreads();
-        nt_masked(Wt, b0, b1, N + 4, dv, P.normalized ? us : nullptr);  // P
-        if (ch.before) {
-            const float *Dp = P.D.at(ch.hd, ch.c);
-            nn_carry<N, kTransposed>(acc, t, b0, Dp, dv, dv, d, stage);  // G' D_p^T
-            if (P.normalized)
-                acc.each([&](float x, int i, int j) {
-                    return t.col(j) < d ? fmaf(us[t.row(i)], Dp[d * dv + t.col(j)], x) : x;
-                });
-        } else {
-            __syncthreads();
-        }
-        const bool any_x = sync_unless_finite(load_tile<N>(b1, P.X + ch.tok * d, ch.len, d));
-        nn_lower<N>(acc, t, Wt, b1, any_x);  // P X
+        grad_k<N>(acc_k, t, sm, P, ch);
         __syncthreads();
-        load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
-        const bool any_k = sync_unless_finite(load_tile<N>(b1, P.k + ch.tok * d, ch.len, d));
-        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
-        if (ch.before) nn_carry<N, kPlain>(acc, t, b0, P.S.at(ch.hd, ch.c), d, d, d, stage);  // Y S_p
-        else __syncthreads();
-        nn_lower<N>(acc, t, Wt, b1, any_k);  // B K
+        grad_v<N>(acc_v, t, sm, P, ch);
+        __syncthreads();
+        acc_to_global<N, T>(acc, t, P.dq + ch.tok * d, ch.len, d);
+        acc_to_global<N, T>(acc_k, t, P.dk + ch.tok * d, ch.len, d);
+        acc_to_global<N, T>(acc_v, t, P.dv_out + ch.tok * dv, ch.len, dv);
+    } else if (blockIdx.z == 0) {
+        grad_q<N>(acc, t, sm, P, ch);
         acc_to_global<N, T>(acc, t, P.dq + ch.tok * d, ch.len, d);
     } else if (blockIdx.z == 1) {
-        load_tile<N>(b0, P.Y + ch.tok * d, ch.len, d);
-        load_tile<N>(b1, P.k + ch.tok * d, ch.len, d);
-        __syncthreads();
-        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // B
-        if (ch.after) nn_carry<N, kSymmetric>(acc, t, b1, P.Lam.at(ch.hd, ch.c), d, d, d, stage);
-        else __syncthreads();
-        const bool any_q = sync_unless_finite(load_tile<N>(b0, P.q + ch.tok * d, ch.len, d));
-        tn_lower<N>(acc, t, Wt, b0, any_q);  // B^T Q
-        __syncthreads();
-        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // W
-        __syncthreads();
-        const bool any_y = sync_unless_finite(load_tile<N>(b1, P.Y + ch.tok * d, ch.len, d));
-        tn_lower<N>(acc, t, Wt, b1, any_y);  // W^T Y
+        grad_k<N>(acc, t, sm, P, ch);
         acc_to_global<N, T>(acc, t, P.dk + ch.tok * d, ch.len, d);
     } else {
-        load_tile<N>(b0, P.q + ch.tok * d, ch.len, d);
-        load_tile<N>(b1, P.X + ch.tok * d, ch.len, d);
-        __syncthreads();
-        nt_masked(Wt, b0, b1, N + 4, d, nullptr);  // T
-        if (ch.after) nn_carry<N, kPlain>(acc, t, b1, P.Gam.at(ch.hd, ch.c), dv, d, dv, stage);  // X Gam_s^T
-        else __syncthreads();
-        const bool any_g = sync_unless_finite(load_upstream<N>(b0, static_cast<float *>(nullptr), P, ch));
-        tn_lower<N>(acc, t, Wt, b0, any_g);  // T^T G'
+        grad_v<N>(acc, t, sm, P, ch);
         acc_to_global<N, T>(acc, t, P.dv_out + ch.tok * dv, ch.len, dv);
     }
 }
@@ -346,7 +384,11 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
     }
     if ((e = launch(bwd_y_kernel<N, T>, grid))) return e;
     if (many && (e = scan(P.Lam, 1, nullptr))) return e;
-    return launch(bwd_grad_kernel<N, T>, dim3(nch, p.BH, 3));
+    const size_t nd = sizeof(T) * (size_t)p.BH * p.n * d, nv = sizeof(T) * (size_t)p.BH * p.n * dv;
+    if (backward2_over_tokens(p, p.q, nd) || backward2_over_tokens(p, p.k, nd) || backward2_over_tokens(p, p.v, nv) ||
+        backward2_over_tokens(p, p.dout, nv))
+        return launch(bwd_grad_kernel<N, T, true>, grid);
+    return launch(bwd_grad_kernel<N, T, false>, dim3(nch, p.BH, 3));
 }
 
 }  // namespace
@@ -356,6 +398,12 @@ size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int) {
     const size_t simt = kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
     const size_t tc = backward2_tc_workspace_bytes(BH, n), tiles = backward2_tiles_workspace_bytes(BH, n, d, dv);
     return std::max(simt, std::max(tc, tiles));
+}
+
+bool backward2_over_tokens(const Bwd2 &p, const void *tokens, size_t bytes) {
+    const size_t row = p.dt == HLA_BF16 ? 2 : 4, tok = (size_t)p.BH * p.n;
+    return memory_meets(tokens, bytes, p.dq, tok * p.d * row) || memory_meets(tokens, bytes, p.dk, tok * p.d * row) ||
+           memory_meets(tokens, bytes, p.dval, tok * p.dv * row);
 }
 
 cudaError_t backward2_launch(const Bwd2 &p, cudaStream_t stream) {

@@ -1049,9 +1049,9 @@ bool make_map(CUtensorMap *m, const void *base, int BH, int n, int inner) {
 }
 
 struct TLayout {
-    size_t rec, rec1, iS, iD, iGam, iLam, iX, iY, iG, e, h, den, total;
+    size_t rec, rec1, iS, iD, iGam, iLam, iX, iY, iG, e, h, den, tokens[4], total;
 };
-TLayout make_layout(int BH, int n) {
+TLayout make_layout(int BH, int n, int d, int dv) {
     const size_t tiles = (size_t)BH * ((n + kTile - 1) / kTile);
     TLayout L;
     size_t o = kWsHeaderBytes;
@@ -1072,6 +1072,7 @@ TLayout make_layout(int BH, int n) {
     L.e = take(tiles * kF * 4);
     L.h = take(tiles * kF * 4);
     L.den = take((size_t)BH * n * 4);
+    for (int i = 0; i < 4; ++i) L.tokens[i] = take((size_t)BH * n * (i < 2 ? d : dv) * 2);  // q, k, v, dout
     L.total = o;
     return L;
 }
@@ -1082,7 +1083,7 @@ static bool tiles_sizes(int d, int dv) { return (d == 128 && (dv == 64 || dv == 
 
 size_t backward2_tiles_workspace_bytes(int BH, int n, int d, int dv) {
     if (BH <= 0 || n <= 0 || !tiles_sizes(d, dv)) return kWsHeaderBytes;
-    return make_layout(BH, n).total;
+    return make_layout(BH, n, d, dv).total;
 }
 
 bool backward2_tiles_applicable(const Bwd2 &p) {
@@ -1097,14 +1098,26 @@ bool backward2_tiles_applicable(const Bwd2 &p) {
     return major == 10 && minor == 3 && encode_fn() != nullptr;
 }
 
-cudaError_t backward2_tiles_launch(const Bwd2 &p, cudaStream_t s) {
+cudaError_t backward2_tiles_launch(const Bwd2 &call, cudaStream_t s) {
+    Bwd2 p = call;
+    const TLayout L = make_layout(p.BH, p.n, p.d, p.dv);
+    cudaError_t e = cudaMemsetAsync(p.ws, 0, kWsHeaderBytes, s);
+    if (e) return e;
+    // the blocks of the last launch write one gradient of a tile each while others read the tile's tokens: a token
+    // array that an output lies over is read from a copy
+    const void **tokens[4] = {&p.q, &p.k, &p.v, &p.dout};
+    for (int i = 0; i < 4; ++i) {
+        const size_t bytes = (size_t)p.BH * p.n * (i < 2 ? p.d : p.dv) * 2;
+        if (!backward2_over_tokens(call, *tokens[i], bytes)) continue;
+        if ((e = cudaMemcpyAsync(p.ws + L.tokens[i], *tokens[i], bytes, cudaMemcpyDeviceToDevice, s))) return e;
+        *tokens[i] = p.ws + L.tokens[i];
+    }
     Maps m;
     if (!make_map(&m.q, p.q, p.BH, p.n, p.d) || !make_map(&m.k, p.k, p.BH, p.n, p.d) ||
         !make_map(&m.v, p.v, p.BH, p.n, p.dv) || !make_map(&m.g, p.dout, p.BH, p.n, p.dv) ||
         !make_map(&m.dq, p.dq, p.BH, p.n, p.d) || !make_map(&m.dk, p.dk, p.BH, p.n, p.d) ||
         !make_map(&m.dv, p.dval, p.BH, p.n, p.dv))
         return cudaErrorInvalidValue;
-    const TLayout L = make_layout(p.BH, p.n);
     TParams t{};
     t.rec = reinterpret_cast<float *>(p.ws + L.rec);
     t.rec1 = reinterpret_cast<float *>(p.ws + L.rec1);
@@ -1116,8 +1129,6 @@ cudaError_t backward2_tiles_launch(const Bwd2 &p, cudaStream_t s) {
     t.den = reinterpret_cast<float *>(p.ws + L.den);
     t.n = p.n; t.M = (p.n + kTile - 1) / kTile; t.d = p.d; t.dv = p.dv; t.normalized = p.normalized; t.eps = p.eps;
     t.err = reinterpret_cast<WsHeader *>(p.ws);
-    cudaError_t e = cudaMemsetAsync(p.ws, 0, kWsHeaderBytes, s);
-    if (e) return e;
     bool follows = false;  // a launch of this call came before
     auto launch = [&](auto kern, int z) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);

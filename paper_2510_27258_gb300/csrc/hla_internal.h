@@ -98,6 +98,8 @@ struct Bwd2 {
 };
 size_t backward2_workspace_bytes(int BH, int n, int d, int dv, int chunk);
 cudaError_t backward2_launch(const Bwd2 &p, cudaStream_t stream);
+// whether an output of the call lies over a token array of that many bytes
+bool backward2_over_tokens(const Bwd2 &p, const void *tokens, size_t bytes);
 // the backward on the tensor cores (hla_backward_sm103.cu): bf16, d = dv = 64, plain output
 size_t backward2_tc_workspace_bytes(int BH, int n);
 bool backward2_tc_applicable(const Bwd2 &p);

@@ -25,6 +25,8 @@
 namespace hla {
 namespace {
 
+// Blocks of a (chunk, head) lie along the grid's first dimension, the chunks of a head side by side: the other two
+// end at 65535, which heads may pass (chunk_grid, chunk_of).
 constexpr int kC = 64;        // tokens of a chunk
 constexpr int kCT = 128;      // threads of a block
 constexpr int kLdW = kC + 4;  // row length of a masked chunk tile
@@ -430,6 +432,12 @@ constexpr int tile_floats() { return kC * (N + 4); }
 template <int N>
 constexpr int blocks_per_sm() { return N == 128 ? 2 : 4; }
 
+inline dim3 chunk_grid(int nch, int BH, int z = 1) { return dim3((unsigned)nch * (unsigned)BH, 1, z); }
+__device__ __forceinline__ void chunk_of(int nch, int &c, int &hd) {
+    hd = blockIdx.x / (unsigned)nch;
+    c = blockIdx.x % (unsigned)nch;
+}
+
 // ---------------------------------------------------------------------------
 // per-chunk records and their prefix sums.  Records of a head: nch of them, then one that holds the
 // initial value on entry (if there is one) and the total on exit.
@@ -504,7 +512,9 @@ __global__ void __launch_bounds__(kCT) chunk_sums_kernel(const __grid_constant__
     extern __shared__ __align__(16) float sm[];
     chain_begin();
     const SumJob<T> &J = jobs.j[blockIdx.z];
-    const int c = blockIdx.x, hd = blockIdx.y, t0 = c * kC, len = min(kC, n - t0);
+    int c, hd;
+    chunk_of(J.r.nch, c, hd);
+    const int t0 = c * kC, len = min(kC, n - t0);
     float *As = sm, *Bs = sm + tile_floats<N>();
     load_tile<N>(As, J.A + ((long long)hd * n + t0) * J.d, len, J.d);
     if (J.B != J.A) load_tile<N>(Bs, J.B + ((long long)hd * n + t0) * J.width, len, J.width);
@@ -520,7 +530,7 @@ cudaError_t launch_sums(bool follows, const SumJobs<T> &jobs, int njobs, int BH,
     const int smem = 2 * tile_floats<N>() * (int)sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(chunk_sums_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e) return e;
-    return chain_launch(follows, chunk_sums_kernel<N, T>, dim3((n + kC - 1) / kC, BH, njobs), kCT, smem, s, jobs, n);
+    return chain_launch(follows, chunk_sums_kernel<N, T>, chunk_grid((n + kC - 1) / kC, BH, njobs), kCT, smem, s, jobs, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -540,7 +550,9 @@ __global__ void __launch_bounds__(kCT)
     extern __shared__ __align__(16) float sm[];
     chain_begin();
     float *b0 = sm, *stage = b0 + tile_floats<N>(), *dens = stage + stage_floats<N>();
-    const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
+    int c, hd;
+    chunk_of(P.carry.nch, c, hd);
+    const int d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
     const long long tok = (long long)hd * P.n + t0;
     const bool carry = c > 0 || P.has_in;
     const float *Mp = P.carry.at(hd, c);
@@ -583,7 +595,7 @@ cudaError_t launch_out(const T *q, T *out, const OutParams &P, int BH, cudaStrea
     const int smem = (tile_floats<N>() + stage_floats<N>() + kC) * (int)sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(chunk_out_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e) return e;
-    return chain_launch(true, chunk_out_kernel<N, T>, dim3((P.n + kC - 1) / kC, BH), kCT, smem, s, q, out, P);
+    return chain_launch(true, chunk_out_kernel<N, T>, chunk_grid((P.n + kC - 1) / kC, BH), kCT, smem, s, q, out, P);
 }
 
 // the padded head size that serves d and dv

@@ -66,7 +66,9 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *ss = stage + stage_floats<N>(), *dens = ss + kC;
-    const int c = blockIdx.x, hd = blockIdx.y, d = A.d, dv = A.dv, t0 = c * kC, len = min(kC, A.n - t0);
+    int c, hd;
+    chunk_of(A.P.nch, c, hd);
+    const int d = A.d, dv = A.dv, t0 = c * kC, len = min(kC, A.n - t0);
     const long long tok = (long long)hd * A.n + t0;
     const bool carry = c > 0 || A.has_in;
     const float *Pp = A.P.at(hd, c);
@@ -144,7 +146,7 @@ cudaError_t forward_n(const Fwd2 &p, cudaStream_t s) {
         const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + 2 * kC) * (int)sizeof(float);
         if ((e = cudaFuncSetAttribute(ahla_chunk_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
             return e;
-        if ((e = chain_launch(sums, ahla_chunk_kernel<N, T>, dim3(nch, p.BH), kCT, smem, s, q, k, v, out, A))) return e;
+        if ((e = chain_launch(sums, ahla_chunk_kernel<N, T>, chunk_grid(nch, p.BH), kCT, smem, s, q, k, v, out, A))) return e;
     }
     if (!sums) return cudaSuccess;
     ScanJobs scans{};

@@ -81,10 +81,13 @@ struct Chunk {
     int c, hd, len;
     long long tok;
     bool before, after;  // chunks before / after it
-    __device__ Chunk(const BParams<T> &P)
-        : c(blockIdx.x), hd(blockIdx.y), len(min(kC, P.n - (int)blockIdx.x * kC)),
-          tok((long long)blockIdx.y * P.n + blockIdx.x * kC), before(blockIdx.x > 0),
-          after((int)blockIdx.x + 1 < P.S.nch) {}
+    __device__ Chunk(const BParams<T> &P) {
+        chunk_of(P.S.nch, c, hd);
+        len = min(kC, P.n - c * kC);
+        tok = (long long)hd * P.n + c * kC;
+        before = c > 0;
+        after = c + 1 < P.S.nch;
+    }
 };
 
 // G' rows of a chunk (the output gradient itself for the plain output) and u
@@ -349,7 +352,7 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
     P.Lam = {ws + L.oL, d * d, nch};
     P.X = ws + L.oX; P.Y = ws + L.oY; P.num = ws + L.oNum; P.den = ws + L.oDen;
     P.n = p.n; P.d = d; P.dv = dv; P.normalized = p.normalized; P.eps = p.eps;
-    const dim3 grid(nch, p.BH);
+    const dim3 grid = chunk_grid(nch, p.BH);
     const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
     cudaError_t e;
     bool follows = false;  // a launch of this call came before
@@ -388,7 +391,7 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
     if (backward2_over_tokens(p, p.q, nd) || backward2_over_tokens(p, p.k, nd) || backward2_over_tokens(p, p.v, nv) ||
         backward2_over_tokens(p, p.dout, nv))
         return launch(bwd_grad_kernel<N, T, true>, grid);
-    return launch(bwd_grad_kernel<N, T, false>, dim3(nch, p.BH, 3));
+    return launch(bwd_grad_kernel<N, T, false>, chunk_grid(nch, p.BH, 3));
 }
 
 }  // namespace

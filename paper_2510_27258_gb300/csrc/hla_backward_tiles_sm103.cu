@@ -152,8 +152,8 @@ struct Ctx {
         r = 32 * (warp & 3) + lane;  // TMEM lane of this thread
         half = warp >> 2;            // its columns: 64 half .. + 63
         lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-        tile = blockIdx.x;
-        head = blockIdx.y;
+        tile = blockIdx.x % (unsigned)p.M;  // the grid's other dimensions end at 65535, which heads may pass
+        head = blockIdx.x / (unsigned)p.M;
         at = (size_t)head * p.M + tile;
         len = min(kTile, p.n - tile * kTile);
         before = tile > 0;
@@ -962,9 +962,9 @@ struct SumsJobs {
 __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ SumsJobs jobs, int M) {
     chain_begin();
     const SumsJob &J = jobs.j[blockIdx.z];
-    const int tid = threadIdx.x, head = blockIdx.y;
+    const int tid = threadIdx.x, head = blockIdx.x, part = blockIdx.y;
     const size_t h0 = (size_t)head * M;
-    if (blockIdx.x == 16) {
+    if (part == 16) {
         if (!J.vec) return;
         float acc = 0.f;
         for (int i = 0; i < M; ++i) {
@@ -976,7 +976,7 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
         }
         return;
     }
-    const int w = blockIdx.x * 4 + (tid >> 5), lane = tid & 31;
+    const int w = part * 4 + (tid >> 5), lane = tid & 31;
     const int r = (w >> 3) * 16 + (lane >> 1), c0 = (w & 7) * 16 + (lane & 1) * 8;
     const uint32_t off = tile_off(r, c0);
     const int i0 = rec_index(r, c0), i1 = rec_index(r, c0 + 4);
@@ -1089,7 +1089,6 @@ size_t backward2_tiles_workspace_bytes(int BH, int n, int d, int dv) {
 bool backward2_tiles_applicable(const Bwd2 &p) {
     if (getenv("HLA_DISABLE_FUSED")) return false;
     if (p.dt != HLA_BF16 || !tiles_sizes(p.d, p.dv) || p.n <= 0 || p.BH <= 0) return false;
-    if (p.BH > 65535) return false;  // heads along a grid's second dimension
     if (p.ws_bytes < backward2_tiles_workspace_bytes(p.BH, p.n, p.d, p.dv)) return false;
     int dev = 0, major = 0, minor = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -1133,7 +1132,7 @@ cudaError_t backward2_tiles_launch(const Bwd2 &call, cudaStream_t s) {
     auto launch = [&](auto kern, int z) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (err) return err;
-        err = chain_launch(follows, kern, dim3(t.M, p.BH, z), kThreads, kSmemBytes, s, m, t);
+        err = chain_launch(follows, kern, dim3((unsigned)t.M * (unsigned)p.BH, 1, z), kThreads, kSmemBytes, s, m, t);
         follows = true;
         return err;
     };
@@ -1141,7 +1140,7 @@ cudaError_t backward2_tiles_launch(const Bwd2 &call, cudaStream_t s) {
         SumsJobs jobs{};
         jobs.j[0] = a;
         if (b) jobs.j[1] = *b;
-        return chain_launch(true, bt_scan_kernel, dim3(17, p.BH, b ? 2 : 1), 128, 0, s, jobs, t.M);
+        return chain_launch(true, bt_scan_kernel, dim3(p.BH, 17, b ? 2 : 1), 128, 0, s, jobs, t.M);
     };
     const bool many = t.M > 1, norm = p.normalized;
     if (many) {

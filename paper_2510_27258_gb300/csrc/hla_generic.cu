@@ -114,7 +114,9 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     chain_begin();
     float *b0 = sm, *b1 = b0 + tile_floats<N>(), *Wt = b1 + tile_floats<N>(), *stage = Wt + kC * kLdW;
     float *dens = stage + stage_floats<N>();
-    const int c = blockIdx.x, hd = blockIdx.y, d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
+    int c, hd;
+    chunk_of(P.S.nch, c, hd);
+    const int d = P.d, dv = P.dv, t0 = c * kC, len = min(kC, P.n - t0);
     const long long tok = (long long)hd * P.n + t0;
     const bool carry = c > 0 || P.has_in;
     load_tile<N>(b0, q + tok * d, len, d);
@@ -198,7 +200,7 @@ cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s
         if ((e = launch_scan(scans, sums_C ? 2 : 1, L.BH, s, follows))) return e;
         follows = true;
     }
-    const dim3 grid(nch, L.BH);
+    const dim3 grid = chunk_grid(nch, L.BH);
     if (nch > 0) {
         const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
         if ((e = cudaFuncSetAttribute(g2_chunk_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))

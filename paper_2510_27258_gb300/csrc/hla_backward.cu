@@ -354,7 +354,8 @@ cudaError_t backward_n(const Bwd2 &p, cudaStream_t s) {
     P.n = p.n; P.d = d; P.dv = dv; P.normalized = p.normalized; P.eps = p.eps;
     const dim3 grid = chunk_grid(nch, p.BH);
     const int smem = (2 * tile_floats<N>() + kC * kLdW + stage_floats<N>() + kC) * (int)sizeof(float);
-    cudaError_t e;
+    cudaError_t e = cudaMemsetAsync(p.ws, 0, kWsHeaderBytes, s);  // no wait here can fail: hla_poll_error finds no error
+    if (e) return e;
     bool follows = false;  // a launch of this call came before
     auto launch = [&](auto kern, dim3 gr) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

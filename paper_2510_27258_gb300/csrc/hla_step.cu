@@ -528,15 +528,16 @@ cudaError_t step2_split_launch(const void *q, const void *k, const void *v, void
                             static_cast<const T *>(v), static_cast<T *>(out), state, split, d, dv, masked, normalized,
                             eps);
     };
-    const int units = d * (dv / split) / 4;  // of a slice: at most 4 a thread (slices of 8 to 64 columns)
+    const int units = d * (dv / split) / 4;  // of a slice: of 8 to 64 columns, 8 to 32 at d = 128
     if (d == 128) {
         if (units <= 512) return go(step2_split_kernel<T, kSDE, 512, 8, 1>, 512);
         if (units <= 1024) return go(step2_split_kernel<T, kSDE, 512, 8, 2>, 512);
-        return go(step2_split_kernel<T, kSDE, 512, 8, 4>, 512);
+        return cudaErrorInvalidValue;
     }
     if (units <= 256) return go(step2_split_kernel<T, kSDE, 256, 4, 1>, 256);
     if (units <= 512) return go(step2_split_kernel<T, kSDE, 256, 4, 2>, 256);
-    return go(step2_split_kernel<T, kSDE, 256, 4, 4>, 256);
+    if (units <= 1024) return go(step2_split_kernel<T, kSDE, 256, 4, 4>, 256);
+    return cudaErrorInvalidValue;
 }
 
 // dynamic shared memory of step2_kernel: S, (C, m), (G, h) if masked, tokens

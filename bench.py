@@ -748,7 +748,7 @@ def bench_backward(hla, dev, stream, world, hbm_peak, tc_peak, steps=10, warmup=
                            "peak_kind": "derived (152 SMs x 128 fp32 lanes x 2 x 2.07 GHz)",
                            "kernel": "bwd_x/upstream/y/grad_kernel and sums over chunks (fp32 CUDA cores)"}
         rec["path"] = "fp32 CUDA cores"
-        rec["launches"] = 5 * steps
+        rec["launches"] = (9 if w.normalized else 7) * steps  # several chunks
     return rec
 
 
@@ -799,7 +799,7 @@ def bench_ahla(hla, dev, stream, hbm_peak, world, steps=20, warmup=3, decode_ste
     res["forward"] = {"workload": w.name, "B": w.B, "H": w.H, "n": w.n, "d": w.d, "dv": w.dv, "chunk": w.chunk,
                       "tokens": w.dtype, "ms_per_step": ms, "value": w.B * w.n * world / (ms * 1e-3),
                       "unit": "tokens/s", "steps": steps, "roofline": roof,
-                      "launches": (1 if tensor_path else 3) * steps}
+                      "launches": (1 if tensor_path else 5) * steps}
     del tq, tk, tv, out, ws
     # decode step
     w = hla_inputs.WORKLOADS["ahla_decode_bf16"]

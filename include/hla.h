@@ -21,10 +21,16 @@
  * stored back to back in [B, H] order.  With masked = 0 the operator does not
  * use G and h: they are ignored on input and written as zeros on output.
  *
- * Supported shapes: d, dv in {16, 32, 64, 128}; 1 <= chunk <= 128 (chunk is
- * the scan granularity of Theorem 2; the result does not depend on it up to
- * rounding); n >= 0 with any remainder n % chunk (a ragged last chunk).
- * Other values return HLA_ERR_UNSUPPORTED.
+ * Supported shapes: d, dv in {16, 32, 64, 128}; 1 <= chunk <= 128 (the scan
+ * granularity of Theorem 2; the result does not depend on it up to rounding,
+ * and second order and AHLA work in tiles of their own whatever it is); n >= 0
+ * with any remainder n % chunk (a ragged last chunk).  Other values return
+ * HLA_ERR_UNSUPPORTED.
+ *
+ * Tokens that are not finite reach the rows that depend on them, and on the
+ * CUDA-core kernels and in the backward with a head size of 128 no others.
+ * The other tensor-core kernels multiply the zeros of a masked 128-token tile,
+ * so there all rows of the tile may become NaN.
  */
 #ifndef HLA_H_
 #define HLA_H_
@@ -128,12 +134,17 @@ size_t hla2_backward_workspace_bytes(int B, int H, int n, int d, int dv, int chu
 /*
  * hla2_backward -- gradients of the masked second-order forward (from a zero
  * state) for L = sum_t dout_t . out_t: dq, dk, dv.  The paper's training
- * route (Sec. "Chunk-parallel training via associative scans"): the forward
- * prefixes are checkpointed at chunk boundaries and recomputed within a
- * chunk, and the gradient suffixes are carried by a reverse scan with the
- * adjoint of the semidirect product (Eq. semidirect); the result equals the
+ * route (Sec. "Chunk-parallel training via associative scans"), with the
+ * carries of both directions as plain sums over chunks: x_t = S_t q_t and
+ * y_t = sum_{s>=t} (dout_s . v_t) q_s are formed chunk by chunk with the
+ * chunk's own prefix of S and suffix of dout q^T, which is where the cross
+ * terms of the semidirect product (Eq. semidirect) and of its adjoint go, so
+ * no carry is multiplied along the sequence.  The result equals the
  * gradients of the serial recurrence (Theorem 2 and the chain rule) up to
- * rounding.  normalized selects out = num / (den + eps) (Eq. masked).
+ * rounding, whatever chunk is.  normalized selects out = num / (den + eps)
+ * (Eq. masked).  bf16 tokens with a head size of 128 (and d = dv = 64, plain)
+ * run on the tensor cores, whose intermediates are pairs of bf16 (16 to 17
+ * bits); other calls are fp32 throughout.
  * q, k, v : device [B, H, n, d] / [B, H, n, d] / [B, H, n, dv] of type dt
  * dout    : device [B, H, n, dv] of type dt (the gradient of the output)
  * dq, dk  : device [B, H, n, d] of type dt (written); dv : [B, H, n, dv] (written);
@@ -294,16 +305,16 @@ size_t ahla_state_floats(int d, int dv);
 size_t ahla_workspace_bytes(int B, int H, int n, int d, int dv, int chunk, hla_dtype dt);
 
 /*
- * ahla_forward -- chunk-parallel AHLA forward: chunk summaries composed with
- * the AHLA semidirect product (Eq. AHLA-semidirect, with the segment cross
- * moment R^KQ = sum k q^T of the later segment), which reproduces the serial
- * recurrence (scan equivalence); chunk is the scan granularity (results do not
- * depend on it up to rounding).  Arguments, layouts, shapes and errors as for
- * hla2_forward (no masked flag), with the AHLA state layout for state_in /
- * state_out (state_out may equal state_in).  bf16 tokens with d and dv in
- * {64, 128}, the plain output and no states run on the tensor cores (one
- * persistent tcgen05 kernel sweeping each head's 128-token tiles with the P
- * and E carries in tensor memory); every other call runs three fp32 kernels.
+ * ahla_forward -- chunk-parallel AHLA forward, which reproduces the serial
+ * recurrence (scan equivalence).  A chunk's r_t = q_t^T P_t are formed with the
+ * chunk's own prefix of P, so the cross term of Eq. AHLA-semidirect is in them
+ * and P and E are plain sums over chunks; the results do not depend on chunk.
+ * Arguments, layouts, shapes and errors as for hla2_forward (no masked flag),
+ * with the AHLA state layout for state_in / state_out (state_out may equal
+ * state_in).  bf16 tokens with d and dv in {64, 128}, the plain output and no
+ * states run on the tensor cores (one persistent tcgen05 kernel sweeping each
+ * head's 128-token tiles with the P and E carries in tensor memory); every
+ * other call runs up to five fp32 kernels on 64-token chunks.
  * A device-side wait that exceeds its budget sets the flag hla_poll_error reads.
  */
 hla_status ahla_forward(const void *q, const void *k, const void *v, void *out, hla_dtype dt,

@@ -334,7 +334,9 @@ step2_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restri
 // 12.1 -> 5.9, 2048 heads 74.9 -> 43.7; (S, D, e) 64 x 64, 16 heads 4.6 -> 4.1, 2048 heads 44.9 -> 28.9;
 // tuple 128 x 128, 8 heads 7.7 -> 6.3, 32 heads 7.9 -> 6.7.  It is bound by the latency of a load,
 // three barriers and the shuffles between them; with many heads by its registers (two or three blocks
-// an SM; one more spilled and was slower).
+// an SM; one more spilled and was slower).  Sums over a slice take an entry that is exactly zero for the rows
+// beyond it, and the output is written after the cluster's barrier: 0 to 4 % less time for up to 256 heads, 2048
+// heads of 64 x 64 on the tuple 47.7 -> 49.7 (8 bytes spilled).
 // NS, NC: float4 units that a thread takes of S and of a column slice.
 // ---------------------------------------------------------------------------
 template <typename T, bool kSDE, int TH, int NS, int NC>

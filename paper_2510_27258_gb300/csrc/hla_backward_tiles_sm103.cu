@@ -24,10 +24,15 @@
 // float4 (r, c..c+3) at index ((r / 32 * 16 + c / 8) * 2 + c / 4 % 2) * 32 + r % 32, so that a warp's
 // access is 512 contiguous bytes.  Head size 64 runs zero-padded (TMA fill).
 //
-// Measured: B2 H16 n4096 d128 normalised 0.479 ms, against 2.09 ms for the CUDA-core kernels (and 37 ms
-// for the kernels those replaced); ncu, us: 20 for K^T K, 73 X, 63 G', 65 Y, 162 the gradients, 20 to 23 for
-// each of the four sums.  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak; the
-// rest is the blocks' chains of copy, product and epilogue, two in flight an SM.
+// Measured: B2 H16 n4096 d128 normalised 0.487 ms, against 2.04 ms for the CUDA-core kernels (and 37 ms
+// for the kernels those replaced); ncu, us: 20 for K^T K, 74 X, 63 G', 66 Y, 168 the gradients, 21 to 25 for
+// each of the four sums.  What bounds it is its own traffic: those launches read 1691 MB and write 445 MB, 0.31 ms
+// at the measured copy rate, and the gradients run at 82 % of it (they load 26 operands of 32 KB a tile, 17 of them
+// distinct).  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak.
+//
+// Accuracy, against 64-bit results, of the bf16 gradients over B1 H4 n100 to B1 H4 n16384 and B8 H16 n512: 1.66e-3 of
+// the norm, as with the fp32 kernels to 2e-5 of that figure (the results' own rounding); the worst row of 65536, where
+// the terms of a gradient cancel to a thousandth, 7.4e-3 of its norm instead of 2.6e-3.
 #include <algorithm>
 #include <cstdlib>
 
@@ -946,7 +951,7 @@ __global__ void __launch_bounds__(kThreads, 2) bt_grad_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 // Sums over the tiles of a head: record c becomes, as a hi/lo image pair, the sum of the records before
 // it (reverse: after it).  A thread carries 8 columns of a row, eight tiles' loads in flight; two
-// neighbouring lanes fill a 32-byte sector of each image.  Block 16 of a head does the same for a vector of 128
+// neighbouring lanes fill a 32-byte sector of each image.  Block 0 of a head does the same for a vector of 128
 // floats in place.  Bound by HBM: 64 KB read and written per tile (with 16 columns a thread, half the threads and
 // four tiles in flight, a sum over 1024 tiles took 27 to 33 us, now 20 to 23).
 // ---------------------------------------------------------------------------
@@ -964,7 +969,7 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
     const SumsJob &J = jobs.j[blockIdx.z];
     const int tid = threadIdx.x, head = blockIdx.x, part = blockIdx.y;
     const size_t h0 = (size_t)head * M;
-    if (part == 16) {
+    if (part == 0) {  // the longest chain of loads: started first
         if (!J.vec) return;
         float acc = 0.f;
         for (int i = 0; i < M; ++i) {
@@ -976,7 +981,7 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
         }
         return;
     }
-    const int w = part * 4 + (tid >> 5), lane = tid & 31;
+    const int w = (part - 1) * 4 + (tid >> 5), lane = tid & 31;
     const int r = (w >> 3) * 16 + (lane >> 1), c0 = (w & 7) * 16 + (lane & 1) * 8;
     const uint32_t off = tile_off(r, c0);
     const int i0 = rec_index(r, c0), i1 = rec_index(r, c0 + 4);

@@ -1422,7 +1422,7 @@ state_c_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // The paper tuple [S | C | m | G | h] (d x d, d x dv, d, d x dv, d) from the ring slot of the head's
 // last segment and the C / m partials.  Block (head, 16 columns of C and G): with one block a head the
 // d^2 dv products of S C ran on 32 SMs and took 199 us at 32 heads, 128 x 128; on 8 blocks a head,
-// each thread with 8 columns of a row of S read in the ring's own order, they take 18 us (both from cold caches).
+// each thread with 8 columns of a row of S read in the ring's own order, they take 21 us (both from cold caches).
 constexpr int kFinCols = 16;
 __global__ void __launch_bounds__(256) state_finalize_kernel(const float *ring, int last_slot, const float *part,
                                                              int groups, float *state_out, int d, int dv) {

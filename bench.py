@@ -39,13 +39,13 @@ DEC = hla_inputs.WORKLOADS["decode_bf16"]
 # capture of the kernel sources (concatenated) whose SHA-256 starts with "sha256"
 # (summaries in profiles/); reported as null for any other source or workload.
 TRAFFIC = {
-    "hla2_fused_kernel": {"src": ["hla_fused_sm103.cu", "sm103_prims.cuh"], "sha256": "689d2cc9a84c37a8", "workload": "long_bf16_norm",
-                          "n": 16384, "bytes": 524.7e6,
-                          "how": "ncu capture at n=8192 (227.1 MB read + 35.3 MB written during the launch; outputs "
+    "hla2_fused_kernel": {"src": ["hla_fused_sm103.cu", "sm103_prims.cuh"], "sha256": "adbc7ed8c6808142", "workload": "long_bf16_norm",
+                          "n": 16384, "bytes": 525.4e6,
+                          "how": "ncu capture at n=8192 (227.4 MB read + 35.3 MB written during the launch; outputs "
                                  "still dirty in L2 at its end are written later) scaled x2 to n=16384"},
-    "step2_kernel": {"src": ["hla_step.cu"], "sha256": "c0208d2ea3e662d0", "workload": "decode_bf16", "n": 0,
+    "step2_kernel": {"src": ["hla_step.cu"], "sha256": "fec8e40191a75e92", "workload": "decode_bf16", "n": 0,
                      "bytes": 749.3e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
-                                              "tuple_step): 406.5 MB read + 342.9 MB written"},
+                                              "tuple_step): 406.4 MB read + 342.9 MB written"},
     "c3_kernels": {"src": ["hla3_chunked.cu"], "sha256": "17ac1acd5c9202d1", "workload": "hla3_f32", "n": 4096,
                    "bytes": 432.5e6, "how": "ncu capture of one forward's five launches (bench.py --only hla3_f32): "
                                             "373.0 MB read + 59.5 MB written, 6.4 x the token I/O (per-chunk records)"},
@@ -59,9 +59,9 @@ TRAFFIC = {
                       "how": "ncu capture of one backward (bench.py --only backward): 278.0 MB read + 170.4 MB "
                              "written; the per-tile records (X hi, lo; S_p, D_p: 96 MB) are written once and read "
                              "back once"},
-    "step2_kernel_sde": {"src": ["hla_step.cu"], "sha256": "c0208d2ea3e662d0", "workload": "decode_bf16", "n": 0,
-                         "bytes": 480.2e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
-                                                  "sde_step): 271.1 MB read + 209.1 MB written"},
+    "step2_kernel_sde": {"src": ["hla_step.cu"], "sha256": "fec8e40191a75e92", "workload": "decode_bf16", "n": 0,
+                         "bytes": 479.9e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
+                                                  "sde_step): 271.1 MB read + 208.8 MB written"},
 }
 
 

@@ -161,7 +161,7 @@ int hla2_forward_path(int B, int H, int n, int d, int dv, int masked, int normal
     if (launches) {
         if ((long long)B * H == 0) *launches = 0;
         else if (fused) *launches = 1 + (has_state_in ? 1 : 0) + (has_state_out ? 2 : 0);
-        else *launches = generic2_launches(n, masked, has_state_in, has_state_out);
+        else *launches = generic2_launches(n, d, dv, masked, has_state_in, has_state_out);
     }
     return fused ? 1 : 0;
 }

@@ -15,7 +15,8 @@
 // along the sequence: the cross term S_A C_B of Eq. semidirect is in X, and
 // everything but the sums runs over all chunks at once.  Launches (masked):
 // K^T K of every chunk; its prefix sums; X, D's increments and T V; D's prefix
-// sums; outputs.  One chunk without states is the third launch alone.
+// sums; outputs.  One chunk without states is the third launch alone; one chunk of small heads
+// with states, and a few tokens without, are one block a head (g2_one_kernel).
 //
 // The chain of products S_p C_c over the chunks that the sums replace took 20 %
 // of a call and ran on a few blocks, the chunk kernels had one multiply-add per
@@ -161,6 +162,151 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     col_sums<N>(rec + d * dv, b1, nullptr, d);
 }
 
+// ---------------------------------------------------------------------------
+// one chunk of head sizes up to 32: all of a head in one block, products over the chunk's own tokens
+// ---------------------------------------------------------------------------
+constexpr int kOneN = 32, kOneLd = kOneN + 4, kOneMat = kOneN * kOneLd;
+constexpr int kOneFloats = 4 * tile_floats<kOneN>() + kC * kLdW + 3 * kOneMat + 2 * kOneN + kC;
+
+// Where that kernel serves.  With a state in or out the launches below are three to seven for a few
+// microseconds of work; without one they are one, whose products run over 64 tokens however few there are.
+// Measured, fp32, us, launches below -> this (-> the kernels before those): 16 x 16, 8 heads of 1 token, states in
+// and out 26.8 -> 12.4 (18.6), 512 heads of 16 40.7 -> 22.9 (26.7), 8 of 64 28.7 -> 16.5 (57); 32 x 32, 512
+// heads of 64 63.7 -> 41.2 (417); without states 2000 heads of 1 x 16 43.2 -> 26.8 (36.0), of 64 the same.
+bool one_block(int n, int d, int dv, bool states) {
+    return n > 0 && n <= (states ? kC : 16) && d <= kOneN && dv <= kOneN;
+}
+
+// a rows x width matrix in global memory (null: zeros) into kOneN rows of kOneLd floats, zero beyond
+__device__ __forceinline__ void load_matrix(float *dst, const float *src, int rows, int width) {
+    constexpr int U = kOneN * kOneN / kCT;
+    float x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int r = (threadIdx.x + u * kCT) / kOneN, c = threadIdx.x % kOneN;
+        x[u] = src && r < rows && c < width ? src[r * width + c] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) dst[(threadIdx.x + u * kCT) / kOneN * kOneLd + threadIdx.x % kOneN] = x[u];
+}
+// emit(a, b, (S C)_ab)
+template <typename F>
+__device__ __forceinline__ void state_product(const Tile<kOneN> &t, const float *S, const float *C, int d, int dv, F emit) {
+    if (4 * t.rg >= d) return;  // rows beyond d lie beyond S
+    Acc<kOneN> acc;
+    acc.zero();
+    nn_range<kOneN, 0>(acc, t, S, kOneLd, C, kOneLd, 0, d);
+#pragma unroll
+    for (int i = 0; i < Tile<kOneN>::RM; ++i)
+#pragma unroll
+        for (int j = 0; j < Tile<kOneN>::CM; ++j)
+            if (t.col(j) < dv) emit(t.row(i), t.col(j), acc.get(i, j));
+}
+// M += A^T B over K tokens (a multiple of 4; d real columns of A)
+__device__ __forceinline__ void add_products(const Tile<kOneN> &t, float *M, const float *A, const float *B, int d, int K) {
+    if (4 * t.rg >= d) return;  // rows beyond d would read beyond a row of A
+    Acc<kOneN> acc;
+    acc.zero();
+    tn_range<kOneN, 0, Tile<kOneN>::RM>(acc, t, A, kOneLd, B, 0, K);
+#pragma unroll
+    for (int i = 0; i < Tile<kOneN>::RM; ++i)
+#pragma unroll
+        for (int j = 0; j < Tile<kOneN>::CM; ++j) M[t.row(i) * kOneLd + t.col(j)] += acc.get(i, j);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCT) g2_one_kernel(const T *__restrict__ q, const T *__restrict__ k,
+                                                     const T *__restrict__ v, T *__restrict__ out, const float *in,
+                                                     float *to, int n, int d, int dv, int masked, int normalized, float eps) {
+    extern __shared__ __align__(16) float sm[];
+    constexpr int N = kOneN;
+    float *bq = sm, *bk = bq + tile_floats<N>(), *bv = bk + tile_floats<N>(), *bx = bv + tile_floats<N>();
+    float *Wt = bx + tile_floats<N>(), *S = Wt + kC * kLdW, *C = S + kOneMat, *D = C + kOneMat;
+    float *m = D + kOneMat, *e = m + N, *dens = e + N;
+    const int tid = threadIdx.x, kn = (n + 3) & ~3;  // tokens, up to a multiple of 4: the rows beyond n are zero
+    const long long hd = blockIdx.x, tok = hd * n, len = (long long)d * d + 2LL * d * dv + 2LL * d;
+    const float *st = in ? in + hd * len : nullptr;
+    const int oC = d * d, om = oC + d * dv, oG = om + d, oh = oG + d * dv;
+    load_tile<N>(bq, q + tok * d, n, d);
+    const float seen_k = load_tile<N>(bk, k + tok * d, n, d), seen_v = load_tile<N>(bv, v + tok * dv, n, dv);
+    if (st || to) {
+        load_matrix(S, st, d, d);
+        load_matrix(C, st ? st + oC : nullptr, d, dv);
+        load_matrix(D, masked && st ? st + oG : nullptr, d, dv);  // G
+        if (tid < N) {
+            m[tid] = st && tid < d ? st[om + tid] : 0.f;
+            e[tid] = masked && st && tid < d ? st[oh + tid] : 0.f;  // h
+        }
+    }
+    const bool any_k = sync_unless_finite(seen_k), any_v = sync_unless_finite(seen_v);
+    const Tile<N> t;
+    const int r = tid >> 1;
+    if (masked && st) {  // D = S C - G, e = S m - h
+        state_product(t, S, C, d, dv, [&](int a, int b, float x) { D[a * kOneLd + b] = x - D[a * kOneLd + b]; });
+        const float x = row_dot(S, kOneLd, m, d);  // rows beyond d read C, unused
+        if ((tid & 1) == 0 && r < d) e[r] = x - e[r];
+    }
+    nt_masked(Wt, bq, bk, kOneLd, d, nullptr);
+    __syncthreads();
+    Acc<N> acc;
+    acc.zero();
+    if (st) nn_range<N, 0>(acc, t, bq, kOneLd, S, kOneLd, 0, d);
+    if (any_k) masked_rows<N, false>(acc, t, Wt, bk);
+    else nn_range<N, 0>(acc, t, Wt, kLdW, bk, kOneLd, 0, kn);
+    acc_to_smem<N>(acc, t, bx);  // X = W K + Q S
+    __syncthreads();
+    if (masked) nt_masked(Wt, bq, bx, kOneLd, d, nullptr);
+    else nt_masked(Wt, bx, bq, kOneLd, d, nullptr);
+    __syncthreads();
+    const float *left = masked ? bq : bx;  // T V + Q D, or T V + X C
+    float den = row_dot(Wt, kLdW, nullptr, kC);
+    if (st) den += row_dot(left, kOneLd, masked ? e : m, d);
+    if ((tid & 1) == 0) dens[r] = normalized ? den + eps : 1.f;
+    acc.zero();
+    if (st) nn_range<N, 0>(acc, t, left, kOneLd, masked ? D : C, kOneLd, 0, d);
+    if (any_v) masked_rows<N, false>(acc, t, Wt, bv);
+    else nn_range<N, 0>(acc, t, Wt, kLdW, bv, kOneLd, 0, kn);
+    __syncthreads();
+    if (normalized) acc.each([&](float x, int i, int) { return x / dens[t.row(i)]; });
+    acc_to_global<N, T>(acc, t, out + tok * dv, n, dv);
+    if (!to) return;
+    // the state after the chunk
+    add_products(t, S, bk, bk, d, kn);
+    add_products(t, C, bq, bv, d, kn);
+    if (masked) add_products(t, D, bx, bv, d, kn);
+    if (tid < 2 * N) {  // m += Q^T 1, e += X^T 1
+        const int c = tid % N;
+        const float *A = tid < N ? bq : bx;
+        float x = 0.f;
+        for (int i = 0; i < n; ++i) x += A[i * kOneLd + c];
+        (tid < N ? m : e)[c] += x;
+    }
+    __syncthreads();
+    float *o = to + hd * len;
+    for (int i = tid; i < d * d; i += kCT) o[i] = S[i / d * kOneLd + i % d];
+    for (int i = tid; i < d * dv; i += kCT) o[oC + i] = C[i / dv * kOneLd + i % dv];
+    if (tid < d) o[om + tid] = m[tid];
+    if (masked) {
+        state_product(t, S, C, d, dv, [&](int a, int b, float x) { o[oG + a * dv + b] = x - D[a * kOneLd + b]; });
+        const float x = row_dot(S, kOneLd, m, d);
+        if ((tid & 1) == 0 && r < d) o[oh + r] = x - e[r];
+    } else {
+        for (int i = tid; i < d * dv; i += kCT) o[oG + i] = 0.f;
+        if (tid < d) o[oh + tid] = 0.f;
+    }
+}
+
+template <typename T>
+cudaError_t forward_one(const Fwd2 &p, cudaStream_t s) {
+    const int smem = kOneFloats * (int)sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(g2_one_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e) return e;
+    g2_one_kernel<T><<<p.BH, kCT, smem, s>>>(static_cast<const T *>(p.q), static_cast<const T *>(p.k),
+                                            static_cast<const T *>(p.v), static_cast<T *>(p.out), p.state_in, p.state_out,
+                                            p.n, p.d, p.dv, p.masked, p.normalized, p.eps);
+    return cudaGetLastError();
+}
+
 template <int N, typename T>
 cudaError_t forward_n(const Fwd2 &p, const GLayout &L, float *ws, cudaStream_t s) {
     const T *q = static_cast<const T *>(p.q), *k = static_cast<const T *>(p.k), *v = static_cast<const T *>(p.v);
@@ -232,7 +378,8 @@ size_t generic2_workspace_bytes(int BH, int n, int d, int dv, int) {
     return kWsHeaderBytes + sizeof(float) * (size_t)make_layout(BH, n, d, dv).total;
 }
 
-int generic2_launches(int n, int masked, int has_state_in, int has_state_out) {
+int generic2_launches(int n, int d, int dv, int masked, int has_state_in, int has_state_out) {
+    if (one_block(n, d, dv, has_state_in || has_state_out)) return 1;
     const int nch = (n + kC - 1) / kC;
     const bool sums = nch > 1 || has_state_in || has_state_out;
     int l = (has_state_in && masked ? 1 : 0) + (has_state_out ? 1 : 0);
@@ -259,6 +406,8 @@ cudaError_t generic2_forward(const Fwd2 &p, cudaStream_t stream) {
             pp.state_in = copy;
         }
     }
+    if (one_block(p.n, p.d, p.dv, p.state_in || p.state_out))
+        return p.dt == HLA_BF16 ? forward_one<__nv_bfloat16>(pp, stream) : forward_one<float>(pp, stream);
     return with_padded_size(p.d, p.dv, [&](auto size) {
         constexpr int N = decltype(size)::value;
         return p.dt == HLA_BF16 ? forward_n<N, __nv_bfloat16>(pp, L, scratch, stream)

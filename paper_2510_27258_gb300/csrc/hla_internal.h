@@ -68,7 +68,7 @@ struct Fwd2 {
 
 // generic fp32 SIMT path (any supported shape)
 size_t generic2_workspace_bytes(int BH, int n, int d, int dv, int chunk);
-int generic2_launches(int n, int masked, int has_state_in, int has_state_out);
+int generic2_launches(int n, int d, int dv, int masked, int has_state_in, int has_state_out);
 cudaError_t generic2_forward(const Fwd2 &p, cudaStream_t stream);
 
 // fused tcgen05 path (bf16, d = dv in {64, 128}); returns false if it does not apply

@@ -420,16 +420,23 @@ ahla_step_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T
     }
 }
 
-// Blocks per head of the kernel above, 0 where the staged kernel serves.  Head sizes up to 64: two for
-// few heads (16 heads 3.1 -> 2.8 us), one from 128 heads (3.2 against 3.3).  With a size of 128: four
-// up to 64 heads, then two where the staged kernel's last round is nearly full or there are many rounds;
-// between 200 and 600 heads the staged kernel, whose copies of the next head run during this one, is as
-// fast or faster (256 heads: 12.6 against 14.0 us).  Clusters cost more to launch: the normalised output
-// takes them up to 64 heads.  A block's slice has 8 to 64 columns.
+// Blocks per head of the kernel above, 0 where the staged kernel serves: the line lies where the staged kernel,
+// whose copies of the next head run during this one, is as fast (measured at 24 to 5000 heads, us, staged / this).
+// Head sizes up to 64: two for few heads (16 heads 3.1 -> 2.8 us), one from 128 heads (3.2 against 3.3).
+// With a size of 128, four up to 64 heads (64 of 128 x 128 5.6 / 4.2); of small d, normalised, two (64 of 16 x 128
+// 3.47 / 3.63 by four, 3.38 by two).  More heads, plain (clusters cost more to launch: the normalised output takes
+// them up to 64 heads), two: with the other size up to 32 always (5000 of 32 x 128 73 / 66); with 64 up to 1250 heads
+// (1250 29.3 / 24.8, 1500 33.9 / 36.8, 5000 108 / 121); 128 x 128 while two blocks a head are one round or so (175
+// 10.0 / 9.4, 200 10.0 / 10.3, 600 18.9 / 21.2, 1500 65.8 / 66.2) and from 2000 (2000 85.6 / 85.4, 5000 210 / 202).
+// A block's slice has 8 to 64 columns.
 int ahla_step_split(int BH, int d, int dv, int normalized) {
     int s;
-    if (d == 128 || dv == 128) s = BH <= 64 ? 4 : !normalized && (BH <= 200 || BH >= 600) ? 2 : 0;
-    else s = BH <= 64 ? 2 : 1;
+    if (d != 128 && dv != 128) s = BH <= 64 ? 2 : 1;
+    else if (BH <= 64) s = normalized && d <= 32 ? 2 : 4;
+    else if (normalized) s = 0;
+    else if (d * dv <= 32 * 128) s = 2;
+    else if (d * dv <= 64 * 128) s = BH <= 1250 ? 2 : 0;
+    else s = BH <= 180 || BH >= 2000 ? 2 : 0;
     if (s == 0) return 0;
     while (s > 1 && dv / s < 8) s /= 2;
     while (dv / s > 64) s *= 2;

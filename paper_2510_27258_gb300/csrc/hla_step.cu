@@ -512,9 +512,12 @@ step2_split_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__
 // for any number of heads (two or four were as fast for few heads and slower for many).  With a size of
 // 128, clusters while each fits the chip at once, one block an SM and a cluster within one GPC: 8 heads in
 // eights, 32 in fours (16 in eights and 38 in fours take two rounds, 11.5 and 12.1 us); in twos the
-// staged kernel is as fast (8.0 against 7.9 us at 40 heads).  A block's slice has 8 to 64 columns.
-int step2_split(int BH, int d, int dv) {
+// staged kernel is as fast (8.0 against 7.9 us at 40 heads); the unmasked tuple, which has no third pass to wait
+// for, stays with the staged kernel at d = 128 unless dv is 16 (16 heads of 128 x 128 6.0 against 6.3 us).  A block's
+// slice has 8 to 64 columns.
+int step2_split(int BH, int d, int dv, bool unmasked) {
     int s = 1;
+    if (unmasked && d == 128 && dv >= 32) return 0;
     if (d == 128 || dv == 128) s = BH <= 8 ? 8 : BH <= 32 ? 4 : 0;
     if (s == 0) return 0;
     while (s > 1 && dv / s < 8) s /= 2;
@@ -552,7 +555,7 @@ template <bool kSDE>
 cudaError_t step2_launch_t(const void *q, const void *k, const void *v, void *out, hla_dtype dt, int BH, int d,
                            int dv, int masked, int normalized, float eps, float *state, cudaStream_t stream) {
     if (BH == 0) return cudaSuccess;
-    if (const int split = step2_split(BH, d, dv))
+    if (const int split = step2_split(BH, d, dv, !kSDE && !masked))
         return dt == HLA_BF16 ? step2_split_launch<__nv_bfloat16, kSDE>(q, k, v, out, state, BH, split, d, dv, masked,
                                                                         normalized, eps, stream)
                               : step2_split_launch<float, kSDE>(q, k, v, out, state, BH, split, d, dv, masked, normalized,

@@ -44,8 +44,8 @@ TRAFFIC = {
                           "how": "ncu capture at n=8192 (227.4 MB read + 35.3 MB written during the launch; outputs "
                                  "still dirty in L2 at its end are written later) scaled x2 to n=16384"},
     "step2_kernel": {"src": ["hla_step.cu"], "sha256": "3e5efc0b13df47c3", "workload": "decode_bf16", "n": 0,
-                     "bytes": 749.3e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
-                                              "tuple_step): 406.4 MB read + 342.9 MB written"},
+                     "bytes": 750.2e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
+                                              "tuple_step): 406.4 MB read + 343.8 MB written"},
     "c3_kernels": {"src": ["hla3_chunked.cu"], "sha256": "17ac1acd5c9202d1", "workload": "hla3_f32", "n": 4096,
                    "bytes": 432.5e6, "how": "ncu capture of one forward's five launches (bench.py --only hla3_f32): "
                                             "373.0 MB read + 59.5 MB written, 6.4 x the token I/O (per-chunk records)"},
@@ -60,8 +60,8 @@ TRAFFIC = {
                              "written; the per-tile records (X hi, lo; S_p, D_p: 96 MB) are written once and read "
                              "back once"},
     "step2_kernel_sde": {"src": ["hla_step.cu"], "sha256": "3e5efc0b13df47c3", "workload": "decode_bf16", "n": 0,
-                         "bytes": 479.9e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
-                                                  "sde_step): 271.1 MB read + 208.8 MB written"},
+                         "bytes": 480.3e6, "how": "ncu capture of one step at B64 H32 d128 (bench.py --profile-case "
+                                                  "sde_step): 271.1 MB read + 209.2 MB written"},
 }
 
 

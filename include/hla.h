@@ -144,7 +144,8 @@ size_t hla2_backward_workspace_bytes(int B, int H, int n, int d, int dv, int chu
  * rounding, whatever chunk is.  normalized selects out = num / (den + eps)
  * (Eq. masked).  bf16 tokens with a head size of 128 (and d = dv = 64, plain)
  * run on the tensor cores, whose intermediates are pairs of bf16 (16 to 17
- * bits); other calls are fp32 throughout.
+ * bits; at d = dv = 64 three of them are single bf16); other calls are fp32
+ * throughout.
  * q, k, v : device [B, H, n, d] / [B, H, n, d] / [B, H, n, dv] of type dt
  * dout    : device [B, H, n, dv] of type dt (the gradient of the output)
  * dq, dk  : device [B, H, n, d] of type dt (written); dv : [B, H, n, dv] (written);

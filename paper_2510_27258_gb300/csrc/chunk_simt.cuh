@@ -143,12 +143,20 @@ __device__ __forceinline__ float load_tile(float *dst, const T *__restrict__ src
     }
     return seen;
 }
-// block barrier; on return true in every thread if any `seen` is not zero
-__device__ __forceinline__ bool sync_unless_finite(float seen) { return __syncthreads_or(!(seen == 0.f)) != 0; }
+// block barrier; on return true in every thread if any `seen` is not zero (N = 32, whose products do not ask: false)
+template <int N>
+__device__ __forceinline__ bool sync_unless_finite(float seen) {
+    if constexpr (N == 32) {
+        __syncthreads();
+        return false;
+    } else {
+        return __syncthreads_or(!(seen == 0.f)) != 0;
+    }
+}
 
 // acc[I0..][.] += sum_{k0 <= k < k1} A(r, k) B(k, c), A row-major in shared memory, B rows over c.
-// I0 = 4: only the second half of the rows (A is zero there for the first half).
-template <int N, int I0>
+// I0 = 4: only the second half of the rows (A is zero there for the first half).  kDiag: the terms k <= r alone.
+template <int N, int I0, bool kDiag = false>
 __device__ __forceinline__ void nn_range(Acc<N> &acc, const Tile<N> &t, const float *A, int lda, const float *B,
                                          int ldb, int k0, int k1) {
     constexpr int RM = Tile<N>::RM, CM = Tile<N>::CM;
@@ -166,6 +174,7 @@ __device__ __forceinline__ void nn_range(Acc<N> &acc, const Tile<N> &t, const fl
             }
 #pragma unroll
             for (int i = I0; i < RM; ++i) {
+                if (kDiag && k + kk > t.row(i)) continue;
                 const f32x2 xx = pack2(f4(x[i], kk), f4(x[i], kk));
 #pragma unroll
                 for (int j = 0; j < CM / 2; ++j) fma2(acc.p[i][j], xx, y[j]);
@@ -195,23 +204,29 @@ __device__ __forceinline__ void masked_rows(Acc<N> &acc, const Tile<N> &t, const
                 fma2(acc.p[i][j / 2], pack2(x, x), *reinterpret_cast<const f32x2 *>(B + k * (N + 4) + t.col(j)));
         }
 }
-// A a lower triangular chunk tile.  `any` (the same in every thread): B may have rows that are not finite.  The
-// fast form multiplies such a row by the zeros above the diagonal too, which would make NaN of earlier tokens' rows.
-// Finding out costs one multiply-add per loaded value (B2 H16 n1000 d64 fp32 67.5 us without, 67.7 with); leaving out
-// the terms above the diagonal one by one took 69.8.
+// A a lower triangular chunk tile; K, at N = 32, the tokens that count.  B may have rows that are not finite, and a
+// product over whole quadrants multiplies them by the zeros above the diagonal, which would make NaN of earlier
+// tokens' rows.  N = 32: a warp's sixteen rows take the terms of the triangle alone (B8 H16 n1000 d32 fp32 99.8 -> 94.8
+// us, as what lies beyond a warp's rows is left out).  N = 64, 128: only where `any` (the same in every thread) says
+// that there are such rows; finding out costs one multiply-add per loaded value (B2 H16 n1000 d64 fp32 67.5 us without,
+// 67.7 with), the triangle alone took 69.8.
 template <int N>
-__device__ __forceinline__ void nn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B, bool any) {
-    if (any) return masked_rows<N, false>(acc, t, A, B);
+__device__ __forceinline__ void nn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B, bool any,
+                                         int K = kC) {
     if constexpr (N == 32) {
-        nn_range<N, 0>(acc, t, A, kLdW, B, N + 4, 0, kC);
+        const int rb = t.row(0) & ~15;  // uniform in a warp
+        nn_range<N, 0>(acc, t, A, kLdW, B, N + 4, 0, min(rb, K));
+        nn_range<N, 0, true>(acc, t, A, kLdW, B, N + 4, rb, min(rb + 16, K));
     } else {
+        if (any) return masked_rows<N, false>(acc, t, A, B);
         nn_range<N, 0>(acc, t, A, kLdW, B, N + 4, 0, 32);
         nn_range<N, 4>(acc, t, A, kLdW, B, N + 4, 32, 64);
     }
 }
 
-// acc[I0..I1)[.] += sum_{k0 <= k < k1} A(k, r0 + r) B(k, c): the transposed use of a row-major A
-template <int N, int I0, int I1>
+// acc[I0..I1)[.] += sum_{k0 <= k < k1} A(k, r0 + r) B(k, c): the transposed use of a row-major A.  kDiag: the terms
+// k >= r alone.
+template <int N, int I0, int I1, bool kDiag = false>
 __device__ __forceinline__ void tn_range(Acc<N> &acc, const Tile<N> &t, const float *A, int lda, const float *B,
                                          int k0, int k1) {
     constexpr int CM = Tile<N>::CM;
@@ -231,6 +246,7 @@ __device__ __forceinline__ void tn_range(Acc<N> &acc, const Tile<N> &t, const fl
         }
 #pragma unroll
         for (int i = I0; i < I1; ++i) {
+            if (kDiag && k < t.row(i)) continue;
             const f32x2 xx = pack2(x[i], x[i]);
 #pragma unroll
             for (int j = 0; j < CM / 2; ++j) fma2(acc.p[i][j], xx, y[j]);
@@ -244,10 +260,12 @@ __device__ __forceinline__ void tn(Acc<N> &acc, const Tile<N> &t, const float *A
 // A a lower triangular chunk tile (A(k, r) = 0 for k < r); `any` as above
 template <int N>
 __device__ __forceinline__ void tn_lower(Acc<N> &acc, const Tile<N> &t, const float *A, const float *B, bool any) {
-    if (any) return masked_rows<N, true>(acc, t, A, B);
     if constexpr (N == 32) {
-        tn_range<N, 0, 4>(acc, t, A, kLdW, B, 0, kC);
+        const int rb = t.row(0) & ~15;
+        tn_range<N, 0, 4, true>(acc, t, A, kLdW, B, rb, rb + 16);
+        tn_range<N, 0, 4>(acc, t, A, kLdW, B, rb + 16, kC);
     } else {
+        if (any) return masked_rows<N, true>(acc, t, A, B);
         tn_range<N, 0, 4>(acc, t, A, kLdW, B, 0, 32);
         tn_range<N, 0, 8>(acc, t, A, kLdW, B, 32, 64);
     }

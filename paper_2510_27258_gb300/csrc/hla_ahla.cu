@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     }
     s += row_dot(Wt, kLdW, nullptr, kC);
     if ((threadIdx.x & 1) == 0) ss[threadIdx.x >> 1] = s;
-    const bool any_v = sync_unless_finite(load_tile<N>(b0, v + tok * dv, len, dv));
+    const bool any_v = sync_unless_finite<N>(load_tile<N>(b0, v + tok * dv, len, dv));
     nn_lower<N>(acc, t, Wt, b0, any_v);
     const float den = row_dot<true>(Wt, kLdW, ss, kC);
     __syncthreads();
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
         if (A.direct) dens[r] = den + A.eps;
         else if (r < len) A.den[tok + r] = den;
     }
-    const bool any_r = sync_unless_finite(seen_r);
+    const bool any_r = sync_unless_finite<N>(seen_r);
     acc.zero();
     nn_lower<N>(acc, t, Wt, b0, any_r);  // A R
     if (A.direct) {

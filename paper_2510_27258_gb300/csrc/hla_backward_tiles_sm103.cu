@@ -140,6 +140,23 @@ __device__ __noinline__ void drop_values(uint8_t *slot, Misc *ms) {
     if (threadIdx.x == 0) ms->stains = 1;
 }
 
+// 64 columns of row r of a region from column c0 (at t): NaN where `how` (Ctx::Stain) says
+__device__ __noinline__ void stain_region(uint32_t t, int r, int c0, int how, const Misc *ms) {
+    for (int i = 0; i < 64; i += 32) {
+        uint32_t a[32];
+        __syncwarp();
+        tmem_ld32(t + i, a);
+        tmem_ld_wait();
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            const int f = ms->first[c0 + i + u], l = ms->last[c0 + i + u];
+            if (how == 1 ? r >= f : how == 2 ? r <= l : l >= 0) a[u] = 0x7fffffffu;
+        }
+        tmem_st32(t + i, a);
+        tmem_st_wait();
+    }
+}
+
 // ------------------------------- a block's state -------------------------------
 struct Ctx {
     uint8_t *sm;
@@ -249,13 +266,9 @@ struct Ctx {
         publish();
     }
     enum Stain { kNone, kLower, kUpperT, kColumn };  // rows from the first noted one, up to the last, all
-    __device__ void stain(Stain how, int c0, float (&x)[32]) {
-        if (how == kNone || !ms->stains) return;
-#pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            const int f = ms->first[c0 + u], l = ms->last[c0 + u];
-            if (how == kLower ? r >= f : how == kUpperT ? r <= l : l >= 0) x[u] = __int_as_float(0x7fffffff);
-        }
+    // a result region, where values were dropped: NaN in its place in TMEM
+    __device__ void stain(Stain how, uint32_t region) {
+        if (how != kNone && ms->stains) stain_region(region + lane_base + 64 * half, r, 64 * half, how, ms);
     }
 
     // The masked tile of region RA (kUpper: column >= row, else column <= row), with us[column] or
@@ -324,6 +337,7 @@ struct Ctx {
     }
     // a region -> hi, lo slots, `vec` added to every row where `add`
     __device__ void region_to_slots(uint32_t region, int hi, int lo, bool add, Stain how) {
+        stain(how, region);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int c0 = 64 * half + 32 * i;
@@ -333,18 +347,17 @@ struct Ctx {
 #pragma unroll
                 for (int u = 0; u < 32; ++u) x[u] += ms->vec[c0 + u];
             }
-            stain(how, c0, x);
             split_store(hi, lo, c0, x);
         }
     }
     __device__ void region_to_record(uint32_t region, float *rec, Stain how = kNone) {
+        stain(how, region);
         float4 *o = reinterpret_cast<float4 *>(rec + at * kRec);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int c0 = 64 * half + 32 * i;
             float x[32];
             read32(region, c0, x);
-            stain(how, c0, x);
 #pragma unroll
             for (int u = 0; u < 32; u += 4) o[rec_index(r, c0 + u)] = make_float4(x[u], x[u + 1], x[u + 2], x[u + 3]);
         }
@@ -383,6 +396,7 @@ struct Ctx {
     }
     // a region (plus row_add[r] vec[c] where `add`) as bf16 through slot s to the tile's rows of an output
     __device__ void region_to_output(uint32_t region, int s, const CUtensorMap *m, int width, bool add, Stain how) {
+        stain(how, region);
         const float ur = add ? ms->us[r] : 0.f;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -393,7 +407,6 @@ struct Ctx {
 #pragma unroll
                 for (int u = 0; u < 32; ++u) x[u] = fmaf(ur, ms->vec[c0 + u], x[u]);
             }
-            stain(how, c0, x);
 #pragma unroll
             for (int g = 0; g < 4; ++g)
                 *reinterpret_cast<uint4 *>(slot(s) + tile_off(r, c0 + 8 * g)) =

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
     const long long tok = (long long)hd * P.n + t0;
     const bool carry = c > 0 || P.has_in;
     load_tile<N>(b0, q + tok * d, len, d);
-    const bool any_k = sync_unless_finite(load_tile<N>(b1, k + tok * d, len, d));
+    const bool any_k = sync_unless_finite<N>(load_tile<N>(b1, k + tok * d, len, d));
     const Tile<N> t;
     nt_masked(Wt, b0, b1, N + 4, d, nullptr);
     Acc<N> acc;
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kCT, blocks_per_sm<N>())
         if (direct) dens[r] = P.normalized ? den + P.eps : 1.f;
         else if (r < len) P.den[tok + r] = den;
     }
-    nn_lower<N>(acc, t, Wt, b0, sync_unless_finite(seen_v));  // T V
+    nn_lower<N>(acc, t, Wt, b0, sync_unless_finite<N>(seen_v));  // T V
     if (direct) {
         if (P.normalized) acc.each([&](float x, int i, int) { return x / dens[t.row(i)]; });
         acc_to_global<N, T>(acc, t, out + tok * dv, len, dv);
@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(kCT) g2_one_kernel(const T *__restrict__ q, co
     const float *st = in ? in + hd * len : nullptr;
     const int oC = d * d, om = oC + d * dv, oG = om + d, oh = oG + d * dv;
     load_tile<N>(bq, q + tok * d, n, d);
-    const float seen_k = load_tile<N>(bk, k + tok * d, n, d), seen_v = load_tile<N>(bv, v + tok * dv, n, dv);
+    load_tile<N>(bk, k + tok * d, n, d);
+    load_tile<N>(bv, v + tok * dv, n, dv);
     if (st || to) {
         load_matrix(S, st, d, d);
         load_matrix(C, st ? st + oC : nullptr, d, dv);
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kCT) g2_one_kernel(const T *__restrict__ q, co
             e[tid] = masked && st && tid < d ? st[oh + tid] : 0.f;  // h
         }
     }
-    const bool any_k = sync_unless_finite(seen_k), any_v = sync_unless_finite(seen_v);
+    __syncthreads();
     const Tile<N> t;
     const int r = tid >> 1;
     if (masked && st) {  // D = S C - G, e = S m - h
@@ -251,8 +252,7 @@ __global__ void __launch_bounds__(kCT) g2_one_kernel(const T *__restrict__ q, co
     Acc<N> acc;
     acc.zero();
     if (st) nn_range<N, 0>(acc, t, bq, kOneLd, S, kOneLd, 0, d);
-    if (any_k) masked_rows<N, false>(acc, t, Wt, bk);
-    else nn_range<N, 0>(acc, t, Wt, kLdW, bk, kOneLd, 0, kn);
+    nn_lower<N>(acc, t, Wt, bk, false, kn);
     acc_to_smem<N>(acc, t, bx);  // X = W K + Q S
     __syncthreads();
     if (masked) nt_masked(Wt, bq, bx, kOneLd, d, nullptr);
@@ -264,8 +264,7 @@ __global__ void __launch_bounds__(kCT) g2_one_kernel(const T *__restrict__ q, co
     if ((tid & 1) == 0) dens[r] = normalized ? den + eps : 1.f;
     acc.zero();
     if (st) nn_range<N, 0>(acc, t, left, kOneLd, masked ? D : C, kOneLd, 0, d);
-    if (any_v) masked_rows<N, false>(acc, t, Wt, bv);
-    else nn_range<N, 0>(acc, t, Wt, kLdW, bv, kOneLd, 0, kn);
+    nn_lower<N>(acc, t, Wt, bv, false, kn);
     __syncthreads();
     if (normalized) acc.each([&](float x, int i, int) { return x / dens[t.row(i)]; });
     acc_to_global<N, T>(acc, t, out + tok * dv, n, dv);

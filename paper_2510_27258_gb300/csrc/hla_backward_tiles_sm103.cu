@@ -24,10 +24,10 @@
 // float4 (r, c..c+3) at index ((r / 32 * 16 + c / 8) * 2 + c / 4 % 2) * 32 + r % 32, so that a warp's
 // access is 512 contiguous bytes.  Head size 64 runs zero-padded (TMA fill).
 //
-// Measured: B2 H16 n4096 d128 normalised 0.487 ms, against 2.04 ms for the CUDA-core kernels (and 37 ms
-// for the kernels those replaced); ncu, us: 20 for K^T K, 74 X, 63 G', 66 Y, 168 the gradients, 21 to 25 for
+// Measured: B2 H16 n4096 d128 normalised 0.486 ms, against 2.04 ms for the CUDA-core kernels (and 37 ms
+// for the kernels those replaced); ncu, us: 19 for K^T K, 73 X, 62 G', 64 Y, 165 the gradients, 19 to 24 for
 // each of the four sums.  What bounds it is its own traffic: those launches read 1691 MB and write 445 MB, 0.31 ms
-// at the measured copy rate, and the gradients run at 80 % of it (they load 26 operands of 32 KB a tile, 17 of them
+// at the measured copy rate, and the gradients run at 82 % of it (they load 26 operands of 32 KB a tile, 17 of them
 // distinct).  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak.
 //
 // Accuracy, against 64-bit results, of the bf16 gradients over B1 H4 n100 to B1 H4 n16384 and B8 H16 n512: 1.66e-3 of
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(kThreads, 2) bt_grad_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 // Sums over the tiles of a head: record c becomes, as a hi/lo image pair, the sum of the records before
 // it (reverse: after it).  A thread carries 8 columns of a row, eight tiles' loads in flight; two
-// neighbouring lanes fill a 32-byte sector of each image.  Block 0 of a head does the same for a vector of 128
+// neighbouring lanes fill a 32-byte sector of each image.  Block 16 of a head does the same for a vector of 128
 // floats in place.  Bound by HBM: 64 KB read and written per tile (with 16 columns a thread, half the threads and
 // four tiles in flight, a sum over 1024 tiles took 27 to 33 us, now 20 to 23).
 // ---------------------------------------------------------------------------
@@ -980,9 +980,9 @@ struct SumsJobs {
 __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ SumsJobs jobs, int M) {
     chain_begin();
     const SumsJob &J = jobs.j[blockIdx.z];
-    const int tid = threadIdx.x, head = blockIdx.x, part = blockIdx.y;
+    const int tid = threadIdx.x, head = blockIdx.x / 17, part = blockIdx.x % 17;
     const size_t h0 = (size_t)head * M;
-    if (part == 0) {  // the longest chain of loads: started first
+    if (part == 16) {  // the 17 blocks of a head side by side: with all heads' vectors last or first the call took 489 us
         if (!J.vec) return;
         float acc = 0.f;
         for (int i = 0; i < M; ++i) {
@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(128) bt_scan_kernel(const __grid_constant__ Su
         }
         return;
     }
-    const int w = (part - 1) * 4 + (tid >> 5), lane = tid & 31;
+    const int w = part * 4 + (tid >> 5), lane = tid & 31;
     const int r = (w >> 3) * 16 + (lane >> 1), c0 = (w & 7) * 16 + (lane & 1) * 8;
     const uint32_t off = tile_off(r, c0);
     const int i0 = rec_index(r, c0), i1 = rec_index(r, c0 + 4);
@@ -1158,7 +1158,7 @@ cudaError_t backward2_tiles_launch(const Bwd2 &call, cudaStream_t s) {
         SumsJobs jobs{};
         jobs.j[0] = a;
         if (b) jobs.j[1] = *b;
-        return chain_launch(true, bt_scan_kernel, dim3(p.BH, 17, b ? 2 : 1), 128, 0, s, jobs, t.M);
+        return chain_launch(true, bt_scan_kernel, dim3(17u * (unsigned)p.BH, 1, b ? 2 : 1), 128, 0, s, jobs, t.M);
     };
     const bool many = t.M > 1, norm = p.normalized;
     if (many) {

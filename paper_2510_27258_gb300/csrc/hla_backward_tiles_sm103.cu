@@ -27,7 +27,7 @@
 // Measured: B2 H16 n4096 d128 normalised 0.486 ms, against 2.04 ms for the CUDA-core kernels (and 37 ms
 // for the kernels those replaced); ncu, us: 19 for K^T K, 73 X, 62 G', 64 Y, 165 the gradients, 19 to 24 for
 // each of the four sums.  What bounds it is its own traffic: those launches read 1691 MB and write 445 MB, 0.31 ms
-// at the measured copy rate, and the gradients run at 82 % of it (they load 26 operands of 32 KB a tile, 17 of them
+// at the measured copy rate, and the gradients run at 80 % of it (they load 26 operands of 32 KB a tile, 17 of them
 // distinct).  About 60 products of 128^3 a tile are 0.15 ms at the measured bf16 peak.
 //
 // Accuracy, against 64-bit results, of the bf16 gradients over B1 H4 n100 to B1 H4 n16384 and B8 H16 n512: 1.66e-3 of
